@@ -74,7 +74,7 @@ bool needs_mask(const rlbm_config &c) { return c.solid || c.walls_y || (is_strip
 
 struct Layout {
   size_t pop[2], nbmask, err, ctr, EY, G[2], coef[2], mode_kx, row_start, mode_scale;
-  size_t eps, ux, uy, partials, totals, twx, twy, z0, z1, bins, cols, total;
+  size_t eps, ux, uy, partials, totals, twx, twy, z0, z1, bins, cols, sync, total;
   long long plane;
   int pitch, xoff, Q, nrows, nmodes, max_bins, eyp;
   long long max_blocks;
@@ -101,7 +101,11 @@ Layout make_layout(const rlbm_config &c) {
   L.pop[0] = take(sb * L.Q * L.plane);
   L.pop[1] = take(sb * L.Q * L.plane);
   L.nbmask = take(needs_mask(c) ? 2 * ncell : 0);
+  // the error word and the small results lie together: one copy brings both to the host
   L.err = take(16);
+  L.totals = take(32);
+  L.cols = take(16 * (size_t)c.nx);  // column means j_x, j_y
+  L.bins = take(8 * (size_t)L.max_bins);
   L.ctr = take(16);  // tile counters of the step kernel (two, used by alternate launches)
   L.eyp = (c.ny + 7) / 8 * 8;  // EY rows padded to 8 entries (16-byte TMA strides)
   L.EY = take(2 * rb * (size_t)L.nrows * L.eyp);
@@ -116,13 +120,11 @@ Layout make_layout(const rlbm_config &c) {
   L.ux = take(8 * ncell);
   L.uy = take(8 * ncell);
   L.partials = take(32 * (size_t)std::max<long long>(L.max_blocks, c.nx));  // moments blocks, or one per k_x column
-  L.totals = take(32);
   L.twx = take(16 * (size_t)c.nx);
   L.twy = take(16 * (size_t)c.ny);
   L.z0 = take(16 * ncell);
   L.z1 = take(16 * ncell);
-  L.bins = take(8 * (size_t)L.max_bins);
-  L.cols = take(16 * (size_t)c.nx);  // column means j_x, j_y
+  L.sync = take(4 * (size_t)((c.nx + 31) / 32));  // counters of finished blocks of an observation
   L.total = off;
   return L;
 }
@@ -202,7 +204,7 @@ struct rlbm_ctx {
   std::string msg;
   HostGeom geom;
   HostPhys phys;
-  dim3 block{32, 8, 1};       // moments kernel
+  int sms = 0;                 // multiprocessors of the device
   int grid_limit = 0;          // step kernel: 0 = one wave of resident CTAs
   int stages = 2;              // shared-memory pipeline depth of the step kernel (1 or 2)
   int stir_rows = 1;           // stirring rows: 1 = staged with each tile, 2 = read from global memory
@@ -210,7 +212,7 @@ struct rlbm_ctx {
   int halo_faces = 0;          // a strip: faces whose ghost rows come from neighbours (bit 0 below, 1 above)
   int halo_pending = 0;        // faces not unpacked since the last step, set_state or init
   CUtensorMap tmap_in[2], tmap_G[2], tmap_EY;
-  std::vector<uint8_t> host_stage;
+  std::vector<uint8_t> host_stage, host_small;
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
 
@@ -358,22 +360,26 @@ std::string make_tensor_maps(rlbm_ctx *c) {
   return "";
 }
 
-cudaError_t dispatch_moments(rlbm_ctx *c) {
+// Observation of the current state (rlbm_kernels.cuh): mode 0 the wanted fields and the
+// totals, mode 1 the velocities into z0, mode 2 the column means into L.cols.
+cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = false, bool uy = false) {
   const void *fin = c->ws + c->L.pop[c->cur];
-  double *e = c->at<double>(c->L.eps), *ux = c->at<double>(c->L.ux), *uy = c->at<double>(c->L.uy);
-  double *part = c->at<double>(c->L.partials);
+  HostObs o{};
+  o.eps = eps ? c->at<double>(c->L.eps) : nullptr;
+  o.ux = ux ? c->at<double>(c->L.ux) : nullptr;
+  o.uy = uy ? c->at<double>(c->L.uy) : nullptr;
+  o.z = c->at<double2>(c->L.z0);
+  o.partials = c->at<double>(c->L.partials);
+  o.totals = mode == 2 ? c->at<double>(c->L.cols) : c->at<double>(c->L.totals);
+  o.sync = c->at<unsigned>(c->L.sync);
   unsigned *err = c->at<unsigned>(c->L.err);
-  const double e0 = c->cfg.eps0;
-  cudaError_t r;
+  const double e0 = c->cfg.eps0, vm = c->phys.vmax2;
   switch (c->cfg.precision) {
-    case RLBM_F64: r = launch_moments_f64(c->cfg.vset, fin, c->geom, e0, c->phys.vmax2, e, ux, uy, part, err, c->block, c->stream); break;
-    case RLBM_F32: r = launch_moments_f32(c->cfg.vset, fin, c->geom, e0, c->phys.vmax2, e, ux, uy, part, err, c->block, c->stream); break;
-    case RLBM_F16: r = launch_moments_f16(c->cfg.vset, fin, c->geom, e0, c->phys.vmax2, e, ux, uy, part, err, c->block, c->stream); break;
-    default: r = launch_moments_bf16(c->cfg.vset, fin, c->geom, e0, c->phys.vmax2, e, ux, uy, part, err, c->block, c->stream); break;
+    case RLBM_F64: return launch_observe_f64(c->cfg.vset, mode, fin, c->geom, e0, vm, o, err, c->sms, c->stream);
+    case RLBM_F32: return launch_observe_f32(c->cfg.vset, mode, fin, c->geom, e0, vm, o, err, c->sms, c->stream);
+    case RLBM_F16: return launch_observe_f16(c->cfg.vset, mode, fin, c->geom, e0, vm, o, err, c->sms, c->stream);
+    default: return launch_observe_bf16(c->cfg.vset, mode, fin, c->geom, e0, vm, o, err, c->sms, c->stream);
   }
-  if (r != cudaSuccess) return r;
-  const long long nblocks = (long long)((c->cfg.nx + c->block.x - 1) / c->block.x) * ((c->cfg.ny + c->block.y - 1) / c->block.y);
-  return launch_reduce_partials(part, nblocks, c->at<double>(c->L.totals), c->stream);
 }
 
 cudaError_t dispatch_init(rlbm_ctx *c, void *fout, const double *e, const double *ux, const double *uy) {
@@ -419,13 +425,17 @@ cudaError_t stir_prime(rlbm_ctx *c, int64_t n) {
   }
 }
 
-// Reads the device error word after a synchronisation and latches it.
-rlbm_status check_device(rlbm_ctx *c) {
-  cudaError_t e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return c->cuda_fail(e, "cudaStreamSynchronize");
+// Waits for the stream, reads the device error word and latches it.  The word comes in one
+// copy with the small results behind it (up to byte offset `end` of the workspace), which the
+// caller then finds through small(c, offset): a synchronisation, a copy of the results and a
+// copy of the word were three round trips of some 10 us each.
+rlbm_status check_device(rlbm_ctx *c, size_t end = 0) {
+  c->host_small.resize(std::max(end, c->L.err + sizeof(unsigned)) - c->L.err);
+  cudaError_t e = cudaMemcpyAsync(c->host_small.data(), c->ws + c->L.err, c->host_small.size(), cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return c->cuda_fail(e, "copy of the error word");
   unsigned w = 0;
-  e = cudaMemcpy(&w, c->at<unsigned>(c->L.err), sizeof(unsigned), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return c->cuda_fail(e, "cudaMemcpy(error word)");
+  std::memcpy(&w, c->host_small.data(), sizeof(w));
   if (w & ERR_UNSTABLE) {
     c->latched = RLBM_E_UNSTABLE;
     return c->fail(RLBM_E_UNSTABLE, "a cell became non-finite, eps <= 0 or |v| >= 1 (numerically unstable run)");
@@ -441,6 +451,9 @@ rlbm_status check_device(rlbm_ctx *c) {
   }
   return RLBM_OK;
 }
+
+// A small result after check_device(c, end): the host copy of byte offset `off`.
+const uint8_t *small(const rlbm_ctx *c, size_t off) { return c->host_small.data() + (off - c->L.err); }
 
 rlbm_status usable(rlbm_ctx *c) {
   if (c->latched != RLBM_OK) {
@@ -526,6 +539,7 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   c->ws = static_cast<char *>(dev_workspace);
   c->stream = static_cast<cudaStream_t>(cuda_stream);
   cudaGetDevice(&c->device);
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (c->cfg.fp64_landau_vmax == 0.0) c->cfg.fp64_landau_vmax = 0.5;
 
   auto bail = [&](rlbm_status s) { g_thread_error = c->msg; delete c; return s; };
@@ -643,6 +657,13 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
     std::vector<double> twx(2 * (size_t)cfg->nx), twy(2 * (size_t)cfg->ny);
     for (int t = 0; t < cfg->nx; ++t) { twx[2 * t] = std::cos(2.0 * M_PI * t / cfg->nx); twx[2 * t + 1] = -std::sin(2.0 * M_PI * t / cfg->nx); }
     for (int t = 0; t < cfg->ny; ++t) { twy[2 * t] = std::cos(2.0 * M_PI * t / cfg->ny); twy[2 * t + 1] = -std::sin(2.0 * M_PI * t / cfg->ny); }
+    if (cfg->precision != RLBM_F64)  // (re, im) as high parts, then low parts, in FP32
+      for (std::vector<double> *tw : {&twx, &twy})
+        for (size_t t = 0; t < tw->size(); t += 2) {
+          const double re = (*tw)[t], im = (*tw)[t + 1];
+          const float f[4] = {(float)re, (float)im, (float)(re - (float)re), (float)(im - (float)im)};
+          std::memcpy(&(*tw)[t], f, sizeof(f));
+        }
     keep.emplace_back(reinterpret_cast<uint8_t *>(twx.data()), reinterpret_cast<uint8_t *>(twx.data()) + 16 * (size_t)cfg->nx);
     keep.emplace_back(reinterpret_cast<uint8_t *>(twy.data()), reinterpret_cast<uint8_t *>(twy.data()) + 16 * (size_t)cfg->ny);
     if ((e = put(L.twx, keep[keep.size() - 2].data(), 16 * (size_t)cfg->nx)) != cudaSuccess ||
@@ -667,6 +688,7 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   }
   if ((e = cudaMemsetAsync(c->ws + L.err, 0, 16, c->stream)) != cudaSuccess) { c->cuda_fail(e, "cudaMemsetAsync"); return bail(RLBM_E_CUDA); }
   if ((e = cudaMemsetAsync(c->ws + L.ctr, 0, 16, c->stream)) != cudaSuccess) { c->cuda_fail(e, "cudaMemsetAsync"); return bail(RLBM_E_CUDA); }
+  if ((e = cudaMemsetAsync(c->ws + L.sync, 0, 4 * (size_t)((cfg->nx + 31) / 32), c->stream)) != cudaSuccess) { c->cuda_fail(e, "cudaMemsetAsync"); return bail(RLBM_E_CUDA); }
   if ((e = stir_prime(c, 0)) != cudaSuccess) { c->cuda_fail(e, "stirring set-up kernels"); return bail(RLBM_E_CUDA); }
   if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) { c->cuda_fail(e, "cudaStreamSynchronize"); return bail(RLBM_E_CUDA); }
   c->cur = 0;
@@ -702,13 +724,14 @@ rlbm_status rlbm_moments(rlbm_ctx *c, double *eps, double *ux, double *uy, doubl
   if (c->halo_pending) return c->fail(RLBM_E_STATE, "the strip's ghost rows are not unpacked since its last step");
   Scoped dev(c->device);
   const size_t n = (size_t)c->cfg.nx * c->cfg.ny * sizeof(double);
-  cudaError_t e = dispatch_moments(c);
+  cudaError_t e = dispatch_observe(c, 0, eps, ux, uy);
   if (e != cudaSuccess) return c->cuda_fail(e, "moments kernel launch");
   if (eps && (e = cudaMemcpyAsync(eps, c->ws + c->L.eps, n, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of eps");
   if (ux && (e = cudaMemcpyAsync(ux, c->ws + c->L.ux, n, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of ux");
   if (uy && (e = cudaMemcpyAsync(uy, c->ws + c->L.uy, n, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of uy");
-  if (totals && (e = cudaMemcpyAsync(totals, c->ws + c->L.totals, 32, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of totals");
-  return check_device(c);
+  const rlbm_status s = check_device(c, c->L.totals + 32);
+  if (totals && (s == RLBM_OK || c->latched == s)) std::memcpy(totals, small(c, c->L.totals), 32);
+  return s;
 }
 
 rlbm_status rlbm_spectrum(rlbm_ctx *c, int32_t nbins, double *E) {
@@ -717,16 +740,16 @@ rlbm_status rlbm_spectrum(rlbm_ctx *c, int32_t nbins, double *E) {
   if (is_strip(c->cfg)) return c->fail(RLBM_E_INVAL, "a strip has no spectrum of its own: it needs the whole lattice");
   if (nbins < 1 || !E) return c->fail(RLBM_E_INVAL, "nbins must be >= 1 and E non-NULL");
   Scoped dev(c->device);
-  cudaError_t e = dispatch_moments(c);
-  if (e != cudaSuccess) return c->cuda_fail(e, "moments kernel launch");
+  cudaError_t e = dispatch_observe(c, 1);
+  if (e != cudaSuccess) return c->cuda_fail(e, "velocity kernel launch");
   const int nb = std::min(nbins, c->L.max_bins);
-  e = launch_spectrum(c->at<double>(c->L.ux), c->at<double>(c->L.uy), c->cfg.nx, c->cfg.ny,
+  e = launch_spectrum(c->cfg.precision == RLBM_F64, c->cfg.nx, c->cfg.ny,
                       c->at<double2>(c->L.twx), c->at<double2>(c->L.twy), c->at<double2>(c->L.z0),
                       c->at<double2>(c->L.z1), c->at<double>(c->L.bins), nb, c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "spectrum kernels");
-  if ((e = cudaMemcpyAsync(E, c->ws + c->L.bins, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
-    return c->cuda_fail(e, "copy of the spectrum");
-  rlbm_status s = check_device(c);
+  const rlbm_status s = check_device(c, c->L.bins + 8 * (size_t)nb);
+  if (s != RLBM_OK && c->latched != s) return s;
+  std::memcpy(E, small(c, c->L.bins), sizeof(double) * nb);
   for (int i = nb; i < nbins; ++i) E[i] = 0.0;  // beyond the largest |k| of the lattice
   return s;
 }
@@ -781,17 +804,15 @@ rlbm_status rlbm_band_energy(rlbm_ctx *c, int64_t k2lo, int64_t k2hi, double *E)
   if (is_strip(c->cfg)) return c->fail(RLBM_E_INVAL, "a strip has no band energy of its own: it needs the whole lattice");
   if (!E || k2lo < 0) return c->fail(RLBM_E_INVAL, "E must be non-NULL and k2lo >= 0");
   Scoped dev(c->device);
-  cudaError_t e = dispatch_moments(c);
-  if (e != cudaSuccess) return c->cuda_fail(e, "moments kernel launch");
+  cudaError_t e = dispatch_observe(c, 1);
+  if (e != cudaSuccess) return c->cuda_fail(e, "velocity kernel launch");
   double *out = c->at<double>(c->L.totals);
-  e = launch_band_energy(c->at<double>(c->L.ux), c->at<double>(c->L.uy), c->cfg.nx, c->cfg.ny,
+  e = launch_band_energy(c->cfg.precision == RLBM_F64, c->cfg.nx, c->cfg.ny,
                          c->at<double2>(c->L.twx), c->at<double2>(c->L.twy), c->at<double2>(c->L.z0),
                          c->at<double2>(c->L.z1), k2lo, k2hi, c->at<double>(c->L.partials), out, c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "band energy kernels");
-  double host[4];
-  if ((e = cudaMemcpyAsync(host, out, 32, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of the band energy");
-  if (rlbm_status s = check_device(c)) return s;
-  *E = host[0];
+  if (rlbm_status s = check_device(c, c->L.totals + 32)) return s;
+  std::memcpy(E, small(c, c->L.totals), sizeof(double));
   return RLBM_OK;
 }
 
@@ -800,15 +821,14 @@ rlbm_status rlbm_column_means(rlbm_ctx *c, double *jx, double *jy) {
   if (rlbm_status s = usable(c)) return s;
   if (is_strip(c->cfg)) return c->fail(RLBM_E_INVAL, "a strip has no column means of its own: it needs the whole lattice");
   Scoped dev(c->device);
-  cudaError_t e = dispatch_moments(c);
-  if (e != cudaSuccess) return c->cuda_fail(e, "moments kernel launch");
-  double *d = c->at<double>(c->L.cols);
-  const int nx = c->cfg.nx;
-  if ((e = launch_column_means(c->at<double>(c->L.ux), c->at<double>(c->L.uy), nx, c->cfg.ny, d, d + nx, c->stream)) != cudaSuccess)
-    return c->cuda_fail(e, "column means kernel");
-  if (jx && (e = cudaMemcpyAsync(jx, d, 8 * (size_t)nx, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of j_x");
-  if (jy && (e = cudaMemcpyAsync(jy, d + nx, 8 * (size_t)nx, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return c->cuda_fail(e, "copy of j_y");
-  return check_device(c);
+  cudaError_t e = dispatch_observe(c, 2);
+  if (e != cudaSuccess) return c->cuda_fail(e, "column means kernel launch");
+  const size_t bytes = 8 * (size_t)c->cfg.nx;
+  const rlbm_status s = check_device(c, c->L.cols + 2 * bytes);
+  if (s != RLBM_OK && c->latched != s) return s;
+  if (jx) std::memcpy(jx, small(c, c->L.cols), bytes);
+  if (jy) std::memcpy(jy, small(c, c->L.cols) + bytes, bytes);
+  return s;
 }
 
 }  // extern "C"

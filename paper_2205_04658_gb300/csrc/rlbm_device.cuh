@@ -469,6 +469,41 @@ __device__ __forceinline__ F2 fmax(F2 a, F2 b) { return F2(fmaxf(a.v.x, b.v.x), 
 template <typename T> __device__ __forceinline__ T divide(T a, T b) { return a / b; }
 __device__ __forceinline__ F2 divide(F2 a, F2 b) { return F2(a.v.x / b.v.x, a.v.y / b.v.y); }
 
+// Numbers as unevaluated sums h + l of two FP32 values (about 48 bits), two to a packed pair: sums
+// and transforms of FP32 data that must not round at FP32, at FP32's rate (GB300's FP64 units run
+// at 1/64 of it).  The sum is Knuth's exact two-sum of the high parts with the low parts added
+// (Dekker 1971; error below 2^-46 (|a| + |b|)), the product an FMA-exact product of the high
+// parts plus the cross terms.
+struct DF2 {
+  F2 h, l;
+};
+__device__ __forceinline__ DF2 df_norm(F2 h, F2 l) {  // |h| >= |l|
+  const F2 s = h + l;
+  return DF2{s, l - (s - h)};
+}
+__device__ __forceinline__ DF2 df_add(const DF2 &a, const DF2 &b) {
+  const F2 s = a.h + b.h, bb = s - a.h;
+  const F2 e = (a.h - (s - bb)) + (b.h - bb);
+  return df_norm(s, e + (a.l + b.l));
+}
+__device__ __forceinline__ DF2 df_add(const DF2 &a, F2 b) {
+  const F2 s = a.h + b, bb = s - a.h;
+  const F2 e = (a.h - (s - bb)) + (b - bb);
+  return df_norm(s, e + a.l);
+}
+__device__ __forceinline__ DF2 df_neg(const DF2 &a) { return DF2{-a.h, -a.l}; }
+__device__ __forceinline__ DF2 df_mul(const DF2 &a, const DF2 &b) {
+  const F2 p = a.h * b.h;
+  return df_norm(p, fma(a.l, b.h, fma(a.h, b.l, fma(a.h, b.h, -p))));
+}
+// the two lanes exchanged
+__device__ __forceinline__ F2 swap(F2 a) { return F2(a.v.y, a.v.x); }
+__device__ __forceinline__ DF2 swap(const DF2 &a) { return DF2{swap(a.h), swap(a.l)}; }
+__device__ __forceinline__ F2 shfl_xor(F2 a, int off) {
+  return F2(__shfl_xor_sync(0xffffffffu, a.v.x, off), __shfl_xor_sync(0xffffffffu, a.v.y, off));
+}
+__device__ __forceinline__ DF2 df_shfl_xor(const DF2 &a, int off) { return DF2{shfl_xor(a.h, off), shfl_xor(a.l, off)}; }
+
 template <> struct FM<F2> {
   static __device__ __forceinline__ F2 rcp(F2 x) { return F2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
   static __device__ __forceinline__ F2 rsqrt(F2 x) { return F2(rsqrtf(x.v.x), rsqrtf(x.v.y)); }

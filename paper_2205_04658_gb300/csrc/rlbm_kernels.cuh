@@ -749,10 +749,38 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
 }
 
 // ---------------------------------------------------------------------------
-// Moments of the current state f_n = stream(f*_n) (procedure item 3) straight from
-// global memory (ghost-padded planes): eps, u^x, u^y per cell and per-block FP64
-// partial sums of T^00, T^0x, T^0y, 1/2 |v|^2.  Landau runs in FP64 here.
+// Observation of the current state f_n = stream(f*_n) (procedure item 3) straight from
+// global memory (ghost-padded planes), in one of three forms:
+//   OBS_FIELDS  eps, u^x, u^y per cell (each pointer may be NULL) and the totals T^00, T^0x,
+//               T^0y, 1/2 |v|^2 in `totals`;
+//   OBS_V       z = v_x + i v_y per cell, the input of the spectrum's transform;
+//   OBS_COLS    the column means of v in totals[0 .. nx) (x) and totals[nx .. 2 nx) (y).
+// FP64 storage matches and sums in FP64; the others (FP32 state) match in FP32, as the step
+// kernel does, on packed pairs of cells (x, y), (x, y + 1).
+//
+// What bounds it: DRAM at large sizes (17 planes read, 24 bytes of fields written per cell),
+// so no other pipe may come near that: GB300 runs FP64 and the FP32 -> FP64 conversions at
+// 1/64 of FP32's rate, and the former kernel's five FP64-pipe operations per cell alone took
+// as long as the memory.  The values are widened with integer operations instead (exact),
+// one FP64 addition per cell is left (eps = eps0 (1 + e)), and the totals and column sums of
+// FP32 states are carried in pairs of FP32 numbers (48 bits), FP64 from the block's sum on.
+// The last block to finish adds the blocks' partial sums in a fixed order; a second launch
+// with one serial block took 12-130 us for that.
 // ---------------------------------------------------------------------------
+constexpr int OBS_FIELDS = 0, OBS_V = 1, OBS_COLS = 2;
+// cells of a thread (rows y, y + 1) and rows of an observation tile (32 columns; 8 thread rows)
+template <typename S> constexpr int obs_cells() { return sizeof(S) == 8 ? 1 : 2; }
+template <typename S> constexpr int obs_rows() { return 8 * obs_cells<S>(); }
+
+// FP32 to FP64 by moving the fields of the IEEE formats (exact); zeros, subnormals,
+// infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a < 0x00800000u || a >= 0x7f800000u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 template <typename S, typename R, int VS, bool MASK>
 __device__ __forceinline__ void pull_global(const S *__restrict__ fin, const Geometry<R> &g, int x, int y,
                                             unsigned nb, R h[VSet<VS>::Q]) {
@@ -763,7 +791,7 @@ __device__ __forceinline__ void pull_global(const S *__restrict__ fin, const Geo
     const S *pl = fin + q * g.plane + o;
     const int sx = sgnx<VS>(q), sy = sgny<VS>(q);
     R acc = g.beta[q][0] * load_h<S, R>(pl);
-    const R own = load_h<S, R>(fin + VSet<VS>::opp(q) * g.plane + o);
+    const R own = MASK ? load_h<S, R>(fin + VSet<VS>::opp(q) * g.plane + o) : R(0);
     if (sx != 0) acc += g.beta[q][1] * ((MASK && ((nb >> (4 - sx)) & 1u)) ? own : load_h<S, R>(pl - sx));
     if (sy != 0) acc += g.beta[q][2] * ((MASK && ((nb >> (4 - 3 * sy)) & 1u)) ? own : load_h<S, R>(pl - (long long)sy * g.pitch));
     if (sx != 0 && sy != 0)
@@ -772,99 +800,241 @@ __device__ __forceinline__ void pull_global(const S *__restrict__ fin, const Geo
   }
 }
 
+// The pulls of the cells (x, y) and (x, y + 1) as a pair (lanes without fluid are not pulled).
 template <typename S, int VS, bool MASK>
+__device__ __forceinline__ void pull_global_pair(const S *__restrict__ fin, const Geometry<float> &g, int x, int y,
+                                                 unsigned nbA, unsigned nbB, bool flA, bool flB, F2 h[VSet<VS>::Q]) {
+  float a[VSet<VS>::Q], b[VSet<VS>::Q];
+#pragma unroll
+  for (int q = 0; q < VSet<VS>::Q; ++q) a[q] = b[q] = 0.0f;
+  if (flA) pull_global<S, float, VS, MASK>(fin, g, x, y, nbA, a);
+  if (flB) pull_global<S, float, VS, MASK>(fin, g, x, y + 1, nbB, b);
+#pragma unroll
+  for (int q = 0; q < VSet<VS>::Q; ++q) h[q] = F2(a[q], b[q]);
+}
+
+struct ObsOut {
+  double *eps, *ux, *uy;  // OBS_FIELDS (each may be NULL)
+  double2 *z;             // OBS_V (FP32 states: float4 v_x, v_y, 0, 0: high and low parts); OBS_COLS: the
+                          // blocks' partial column sums (the same two forms)
+  double *partials;       // [blocks][4]
+  double *totals;         // [4]; OBS_COLS: [2 nx]
+  unsigned *sync;         // zeroed counters of finished blocks: 1, or one per tile column (OBS_COLS)
+};
+
+template <typename S, int VS, bool MASK, int MODE>
 __global__ void __launch_bounds__(256)
-moments_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::type> g, double eps0, float vmax2,
-               double *__restrict__ eps, double *__restrict__ ux, double *__restrict__ uy,
-               double *__restrict__ partials, unsigned *__restrict__ err) {
+observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::type> g, double eps0, float vmax2,
+               const ObsOut out, unsigned *__restrict__ err) {
   using R = typename RealOf<S>::type;
   constexpr int Q = VSet<VS>::Q;
   constexpr bool F64 = sizeof(R) == 8;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  // Per-cell terms of the block totals: T^00, T^0x, T^0y, 1/2 |v|^2.  FP64 storage sums
-  // them in FP64.  The other storage types (FP32 state) match and sum in FP32, as the step
-  // kernel does (GB300's FP64 rate is 1/64 of FP32): the FP32 terms are the deviations
-  // e, m_x, m_y (order u), summed per warp, and the warps' sums are added in FP64 to the
-  // exact count of fluid cells (T^00 = eps0 (1 + e)).
+  constexpr int NC = obs_cells<S>(), OBS_ROWS = obs_rows<S>();
+  const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * 32 + lx;
+  const int ntx = (g.nx + 31) / 32, nty = (g.ny + OBS_ROWS - 1) / OBS_ROWS, ntiles = ntx * nty;
+  __shared__ double redd[8][4];
+  __shared__ float4 redf[8][4];         // FP32 state: the warps' sums (high x, y, low x, y) of the four terms
+  __shared__ double2 cols[8][32];
+  __shared__ int cnt[8];
+  __shared__ bool last;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  float accf[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  DF2 accf[4];
   int fluid = 0;
-  if (x < g.nx && y < g.ny) {
-    const long long c = (long long)y * g.nx + x;
-    unsigned nb = MASK ? g.nbmask[c] : 0u;
-    if (MASK && (nb & 16u)) {
-      eps[c] = 0.0; ux[c] = 0.0; uy[c] = 0.0;
-    } else {
-      R h[Q];
-      pull_global<S, R, VS, MASK>(fin, g, x, y, nb, h);
-      if constexpr (F64) {
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int tx = t % ntx, ty = t / ntx;
+    const int x = tx * 32 + lx, y = ty * OBS_ROWS + NC * ly;
+    unsigned nb[NC];
+    bool in[NC], fl[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      in[k] = x < g.nx && y + k < g.ny;
+      nb[k] = 0u;
+      if (MASK && in[k]) nb[k] = g.nbmask[(long long)(y + k) * g.nx + x];
+      fl[k] = in[k] && !(MASK && (nb[k] & 16u));
+    }
+    R e[NC], ux[NC], uy[NC], vx[NC], vy[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) e[k] = ux[k] = uy[k] = vx[k] = vy[k] = R(0);
+    if constexpr (F64) {
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        if (!fl[k]) continue;
+        R h[Q];
+        pull_global<S, R, VS, MASK>(fin, g, x, y + k, nb[k], h);
         const Mom<double> M = moments_of<double, R, VS, false>(h);
         const Macro<double> m = macro_from<double, VS>(M, 40, 1e-12);
         if (!m.ok) atomicOr(err, (1.0 + m.eps_m1 > 0.0 && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
-        eps[c] = eps0 * (1.0 + m.eps_m1);
-        ux[c] = m.ux;
-        uy[c] = m.uy;
-        acc[0] = eps0 * (1.0 + M.e);
-        acc[1] = eps0 * M.mx;
-        acc[2] = eps0 * M.my;
-        acc[3] = 0.5 * (m.vx * m.vx + m.vy * m.vy);
+        e[k] = m.eps_m1; ux[k] = m.ux; uy[k] = m.uy; vx[k] = m.vx; vy[k] = m.vy;
+        if (MODE == OBS_FIELDS) {
+          acc[0] += eps0 * (1.0 + M.e);
+          acc[1] += eps0 * M.mx;
+          acc[2] += eps0 * M.my;
+          acc[3] += 0.5 * (m.vx * m.vx + m.vy * m.vy);
+        }
+      }
+    } else {
+      if (fl[0] || fl[1]) {
+        F2 h[Q];
+        pull_global_pair<S, VS, MASK>(fin, g, x, y, nb[0], nb[1], fl[0], fl[1], h);
+        const Mom<F2> M = moments_of<F2, F2, VS, false>(h);
+        const Macro<F2> m = cell_macro_pair<VS>(h, M, vmax2);  // (a lane without fluid matches the rest state)
+        if (!m.ok) atomicOr(err, (isfinite(m.eps_m1.v.x) && isfinite(m.eps_m1.v.y)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+        e[0] = m.eps_m1.v.x; e[1] = m.eps_m1.v.y;
+        ux[0] = m.ux.v.x; ux[1] = m.ux.v.y; uy[0] = m.uy.v.x; uy[1] = m.uy.v.y;
+        vx[0] = m.vx.v.x; vx[1] = m.vx.v.y; vy[0] = m.vy.v.x; vy[1] = m.vy.v.y;
+        if (MODE == OBS_FIELDS) {
+          // the deviations e, m_x, m_y (order u) beside the exact count of fluid cells
+          // (T^00 = eps0 (1 + e))
+          fluid += (fl[0] ? 1 : 0) + (fl[1] ? 1 : 0);
+          accf[0] = df_add(accf[0], M.e);
+          accf[1] = df_add(accf[1], M.mx);
+          accf[2] = df_add(accf[2], M.my);
+          accf[3] = df_add(accf[3], F2(0.5f) * fma(m.vx, m.vx, m.vy * m.vy));
+        }
+      }
+    }
+    if (MODE == OBS_COLS) {
+      // column sums of the tile's rows, then (the last block of this tile column) of the row blocks
+      if constexpr (F64) {
+        cols[ly][lx] = make_double2(vx[0], vy[0]);
+        __syncthreads();
+        if (ly == 0 && x < g.nx) {
+          double2 a = cols[0][lx];
+          for (int j = 1; j < 8; ++j) { a.x += cols[j][lx].x; a.y += cols[j][lx].y; }
+          out.z[(long long)ty * g.nx + x] = a;
+        }
       } else {
-        // Landau in FP32, re-solved in FP64 where it has not converged or |v| > vmax
-        const Mom<float> M = moments_of<float, float, VS, false>(h);
-        const Macro<float> m = cell_macro<float, VS>(h, M, vmax2);
-        if (!m.ok) atomicOr(err, (1.0f + m.eps_m1 > 0.0f && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
-        eps[c] = eps0 * (1.0 + (double)m.eps_m1);
-        ux[c] = m.ux;
-        uy[c] = m.uy;
-        accf[0] = M.e;
-        accf[1] = M.mx;
-        accf[2] = M.my;
-        accf[3] = 0.5f * (m.vx * m.vx + m.vy * m.vy);
-        fluid = 1;
+        float4 *cf = reinterpret_cast<float4 *>(&cols[0][0]), *zf = reinterpret_cast<float4 *>(out.z);
+        DF2 a = df_add(DF2{F2(vx[0], vy[0]), F2(0.0f)}, F2(vx[NC - 1], vy[NC - 1]));
+        cf[ly * 32 + lx] = make_float4(a.h.v.x, a.h.v.y, a.l.v.x, a.l.v.y);
+        __syncthreads();
+        if (ly == 0 && x < g.nx) {
+          for (int j = 1; j < 8; ++j) {
+            const float4 v = cf[j * 32 + lx];
+            a = df_add(a, DF2{F2(v.x, v.y), F2(v.z, v.w)});
+          }
+          zf[(long long)ty * g.nx + x] = make_float4(a.h.v.x, a.h.v.y, a.l.v.x, a.l.v.y);
+        }
+      }
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) last = atomicInc(out.sync + tx, nty - 1) == (unsigned)(nty - 1);
+      __syncthreads();
+      if (last) {
+        __threadfence();
+        double2 a = make_double2(0.0, 0.0);
+        if constexpr (F64) {
+          if (x < g.nx)
+            for (int j = ly; j < nty; j += 8) {
+              const double2 v = __ldcg(&out.z[(long long)j * g.nx + x]);
+              a.x += v.x;
+              a.y += v.y;
+            }
+          cols[ly][lx] = a;
+          __syncthreads();
+          if (ly == 0)
+            for (int j = 1; j < 8; ++j) { a.x += cols[j][lx].x; a.y += cols[j][lx].y; }
+        } else {
+          float4 *cf = reinterpret_cast<float4 *>(&cols[0][0]);
+          const float4 *zf = reinterpret_cast<const float4 *>(out.z);
+          DF2 d;
+          if (x < g.nx)
+            for (int j = ly; j < nty; j += 8) {
+              const float4 v = __ldcg(&zf[(long long)j * g.nx + x]);
+              d = df_add(d, DF2{F2(v.x, v.y), F2(v.z, v.w)});
+            }
+          cf[ly * 32 + lx] = make_float4(d.h.v.x, d.h.v.y, d.l.v.x, d.l.v.y);
+          __syncthreads();
+          if (ly == 0) {
+            for (int j = 1; j < 8; ++j) {
+              const float4 v = cf[j * 32 + lx];
+              d = df_add(d, DF2{F2(v.x, v.y), F2(v.z, v.w)});
+            }
+            a = make_double2(widen(d.h.v.x) + widen(d.l.v.x), widen(d.h.v.y) + widen(d.l.v.y));
+          }
+        }
+        if (ly == 0 && x < g.nx) {
+          out.totals[x] = a.x / g.ny;
+          out.totals[g.nx + x] = a.y / g.ny;
+        }
+      }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      if (!in[k]) continue;
+      const long long c = (long long)(y + k) * g.nx + x;
+      if (MODE == OBS_FIELDS) {
+        if (out.eps) {
+          double v = 1.0 + widen(e[k]);
+          if (eps0 != 1.0) v *= eps0;
+          out.eps[c] = fl[k] ? v : 0.0;
+        }
+        if (out.ux) out.ux[c] = widen(ux[k]);  // (0 at solid cells)
+        if (out.uy) out.uy[c] = widen(uy[k]);
+      } else if constexpr (F64) {
+        out.z[c] = make_double2(vx[k], vy[k]);
+      } else {
+        reinterpret_cast<float4 *>(out.z)[c] = make_float4(vx[k], vy[k], 0.0f, 0.0f);
       }
     }
   }
-  __shared__ double red[4][32];
-  __shared__ int cnt[32];
-  const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
-  const int warp = (threadIdx.y * blockDim.x + threadIdx.x) >> 5;
+  if (MODE != OBS_FIELDS) return;
+  // this block's partial sums, then (the last block) those of all blocks in a fixed order
+  __syncthreads();
   if constexpr (F64) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       double v = acc[k];
       for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (lane == 0) red[k][warp] = v;
+      if (lx == 0) redd[ly][k] = v;
+    }
+    __syncthreads();
+    if (tid < 4) {
+      double v = 0.0;
+      for (int w = 0; w < 8; ++w) v += redd[w][tid];
+      out.partials[(long long)blockIdx.x * 4 + tid] = v;
     }
   } else {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      float v = accf[k];
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (lane == 0) red[k][warp] = (double)v;
-    }
-    const int nf = __popc(__ballot_sync(0xffffffffu, fluid));
-    if (lane == 0) cnt[warp] = nf;
-  }
-  __syncthreads();
-  const int nwarps = (blockDim.x * blockDim.y + 31) / 32;
-  if (warp == 0) {
-    double tot[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      double v = lane < nwarps ? red[k][lane] : 0.0;
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      tot[k] = v;
+      for (int off = 16; off > 0; off >>= 1) accf[k] = df_add(accf[k], df_shfl_xor(accf[k], off));
+      if (lx == 0) redf[ly][k] = make_float4(accf[k].h.v.x, accf[k].h.v.y, accf[k].l.v.x, accf[k].l.v.y);
     }
-    if (!F64) {
-      int nf = lane < nwarps ? cnt[lane] : 0;
-      for (int off = 16; off > 0; off >>= 1) nf += __shfl_down_sync(0xffffffffu, nf, off);
-      tot[0] = eps0 * ((double)nf + tot[0]);
-      tot[1] *= eps0;
-      tot[2] *= eps0;
+    for (int off = 16; off > 0; off >>= 1) fluid += __shfl_down_sync(0xffffffffu, fluid, off);
+    if (lx == 0) cnt[ly] = fluid;
+    __syncthreads();
+    if (ly == 0) {  // lane: term lx & 3 of warp lx >> 2
+      const float4 f = redf[lx >> 2][lx & 3];
+      double v = (widen(f.x) + widen(f.y)) + (widen(f.z) + widen(f.w));
+      for (int off = 16; off >= 4; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);  // lanes of a term are 4 apart
+      if (lx == 0) {
+        int n = 0;
+        for (int w = 0; w < 8; ++w) n += cnt[w];
+        v += (double)n;
+      }
+      if (lx < 4) out.partials[(long long)blockIdx.x * 4 + lx] = lx == 3 ? v : eps0 * v;
     }
-    if (lane == 0)
-      for (int k = 0; k < 4; ++k) partials[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 4 + k] = tot[k];
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicInc(out.sync, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  {  // term tid & 3; blocks tid >> 2, + 64, ...
+    double v = 0.0;
+    for (int i = tid >> 2; i < (int)gridDim.x; i += 64) v += __ldcg(&out.partials[(long long)i * 4 + (tid & 3)]);
+    for (int off = 16; off >= 4; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lx < 4) redd[ly][lx] = v;
+    __syncthreads();
+    if (tid < 4) {
+      double w = 0.0;
+      for (int j = 0; j < 8; ++j) w += redd[j][tid];
+      out.totals[tid] = w;
+    }
   }
 }
 
@@ -1170,23 +1340,37 @@ static cudaError_t launch_batch_t(int vset, const BatchTables &bt, const HostGeo
   return launch_batch_n<S, 2>(vset, bt, w, p, srows, amp, bstep, mask, force, grid_limit, ntiles, stream);
 }
 
+template <typename S, int VS, bool MASK, int MODE>
+static cudaError_t launch_observe_k(const S *fin, const Geometry<typename RealOf<S>::type> &g, double eps0, double vmax2,
+                                    const ObsOut &o, unsigned *err, int blocks, cudaStream_t stream) {
+  observe_kernel<S, VS, MASK, MODE><<<blocks, dim3(32, 8), 0, stream>>>(fin, g, eps0, (float)vmax2, o, err);
+  return cudaGetLastError();
+}
+
+template <typename S, int VS, bool MASK>
+static cudaError_t launch_observe_v(int mode, const S *fin, const Geometry<typename RealOf<S>::type> &g, double eps0,
+                                    double vmax2, const ObsOut &o, unsigned *err, int sms, cudaStream_t stream) {
+  const int ntiles = ((g.nx + 31) / 32) * ((g.ny + obs_rows<S>() - 1) / obs_rows<S>());
+  // the fields' totals: at most 6 blocks per SM, which add up their tiles (fewer partial sums)
+  if (mode == OBS_FIELDS) return launch_observe_k<S, VS, MASK, OBS_FIELDS>(fin, g, eps0, vmax2, o, err, ntiles < 6 * sms ? ntiles : 6 * sms, stream);
+  if (mode == OBS_V) return launch_observe_k<S, VS, MASK, OBS_V>(fin, g, eps0, vmax2, o, err, ntiles, stream);
+  return launch_observe_k<S, VS, MASK, OBS_COLS>(fin, g, eps0, vmax2, o, err, ntiles, stream);
+}
+
 template <typename S>
-static cudaError_t launch_moments_t(int vset, const void *fin, const HostGeom &hg, double eps0, double vmax2,
-                                    double *eps, double *ux, double *uy, double *partials, unsigned *err,
-                                    dim3 block, cudaStream_t stream) {
+static cudaError_t launch_observe_t(int vset, int mode, const void *fin, const HostGeom &hg, double eps0, double vmax2,
+                                    const HostObs &ho, unsigned *err, int sms, cudaStream_t stream) {
   using R = typename RealOf<S>::type;
   const Geometry<R> g = to_geom<S>(hg);
-  const dim3 grid((hg.nx + block.x - 1) / block.x, (hg.ny + block.y - 1) / block.y);
+  const ObsOut o{ho.eps, ho.ux, ho.uy, ho.z, ho.partials, ho.totals, ho.sync};
   const bool mask = hg.nbmask != nullptr;
   const S *a = (const S *)fin;
   if (vset == 3) {
-    if (mask) moments_kernel<S, 3, true><<<grid, block, 0, stream>>>(a, g, eps0, (float)vmax2, eps, ux, uy, partials, err);
-    else moments_kernel<S, 3, false><<<grid, block, 0, stream>>>(a, g, eps0, (float)vmax2, eps, ux, uy, partials, err);
-  } else {
-    if (mask) moments_kernel<S, 2, true><<<grid, block, 0, stream>>>(a, g, eps0, (float)vmax2, eps, ux, uy, partials, err);
-    else moments_kernel<S, 2, false><<<grid, block, 0, stream>>>(a, g, eps0, (float)vmax2, eps, ux, uy, partials, err);
+    if (mask) return launch_observe_v<S, 3, true>(mode, a, g, eps0, vmax2, o, err, sms, stream);
+    return launch_observe_v<S, 3, false>(mode, a, g, eps0, vmax2, o, err, sms, stream);
   }
-  return cudaGetLastError();
+  if (mask) return launch_observe_v<S, 2, true>(mode, a, g, eps0, vmax2, o, err, sms, stream);
+  return launch_observe_v<S, 2, false>(mode, a, g, eps0, vmax2, o, err, sms, stream);
 }
 
 template <typename S>
@@ -1255,10 +1439,9 @@ static cudaError_t launch_stir_prime_t(const HostStir &hs, void *coef_n, void *c
                                       int grid_limit, int ntiles, cudaStream_t st) {                        \
     return launch_batch_t<S>(vset, bt, w, p, srows, amp, bstep, mask, stages, grid_limit, ntiles, st);    \
   }                                                                                                      \
-  cudaError_t launch_moments_##SUF(int vset, const void *fin, const HostGeom &g, double eps0, double vmax2, \
-                                   double *e, double *ux, double *uy, double *part, unsigned *err,       \
-                                   dim3 b, cudaStream_t st) {                                            \
-    return launch_moments_t<S>(vset, fin, g, eps0, vmax2, e, ux, uy, part, err, b, st);                  \
+  cudaError_t launch_observe_##SUF(int vset, int mode, const void *fin, const HostGeom &g, double eps0,   \
+                                   double vmax2, const HostObs &o, unsigned *err, int sms, cudaStream_t st) { \
+    return launch_observe_t<S>(vset, mode, fin, g, eps0, vmax2, o, err, sms, st);                         \
   }                                                                                                      \
   cudaError_t launch_init_##SUF(int vset, void *fout, const HostGeom &g, double eps0, const double *e,  \
                                 const double *ux, const double *uy, cudaStream_t st) {                   \

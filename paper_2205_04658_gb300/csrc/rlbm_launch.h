@@ -46,6 +46,15 @@ struct HostStir {
   const double *mode_scale;  // device [nmodes]; NULL = all 1
 };
 
+// What an observation of a lattice writes (device memory; rlbm_kernels.cuh): fields and
+// totals (mode 0), velocities for the transform (mode 1) or column means (mode 2).
+struct HostObs {
+  double *eps, *ux, *uy;
+  double2 *z;
+  double *partials, *totals;
+  unsigned *sync;
+};
+
 // One lattice of a batch, as the batched step kernel sees it (device memory, written by
 // the host before the launches; 128-byte aligned so its tensor maps are 64-byte aligned).
 struct alignas(128) MemberDesc {
@@ -87,9 +96,8 @@ struct BatchTables {
   cudaError_t launch_batch_step_##SUF(int vset, const BatchTables &bt, const HostGeom &w, const HostPhys &p, \
                                       int srows, double amp, const long long *bstep, bool mask, int stages, \
                                       int grid_limit, int ntiles, cudaStream_t st);                       \
-  cudaError_t launch_moments_##SUF(int vset, const void *fin, const HostGeom &g, double eps0, double vmax2, \
-                                   double *e, double *ux, double *uy, double *part, unsigned *err,       \
-                                   dim3 b, cudaStream_t st);                                             \
+  cudaError_t launch_observe_##SUF(int vset, int mode, const void *fin, const HostGeom &g, double eps0,   \
+                                   double vmax2, const HostObs &o, unsigned *err, int sms, cudaStream_t st); \
   cudaError_t launch_init_##SUF(int vset, void *fout, const HostGeom &g, double eps0, const double *e,  \
                                 const double *ux, const double *uy, cudaStream_t st);                   \
   cudaError_t launch_open_ghosts_##SUF(int vset, void *f, const HostGeom &g, double ux_in, cudaStream_t st); \
@@ -151,13 +159,15 @@ cudaError_t launch_halo_copy(char *pop, const HaloRows &rows, long long row_byte
 // Reductions and spectrum (rlbm_aux.cu)
 cudaError_t launch_counter_inc(long long *counter, int *tile_ctr, cudaStream_t st);
 cudaError_t launch_reduce_partials(const double *partials, long long nblocks, double *totals, cudaStream_t st);
-cudaError_t launch_column_means(const double *ux, const double *uy, int nx, int ny, double *jx, double *jy,
-                                cudaStream_t st);
-cudaError_t launch_band_energy(const double *ux, const double *uy, int nx, int ny, const double2 *twx,
-                               const double2 *twy, double2 *z0, double2 *z1, long long k2lo, long long k2hi,
-                               double *partials, double *out4, cudaStream_t st);
-cudaError_t launch_spectrum(const double *ux, const double *uy, int nx, int ny, const double2 *twx,
-                            const double2 *twy, double2 *z0, double2 *z1, double *bins, int nbins,
-                            cudaStream_t st);
+
+// The velocity field z = v_x + i v_y (interleaved, [y][x]) of caller-provided u^x, u^y.
+cudaError_t launch_make_z(const double *ux, const double *uy, double2 *z, long long ncell, cudaStream_t st);
+// Spectrum and band energy of z0; both buffers hold nx * ny complex numbers of 16 bytes and are
+// overwritten.  f64: (re, im) in FP64; else high and low FP32 parts (re_h, im_h, re_l, im_l).
+// twx, twy: exp(-2 pi i t / n) in the same form.
+cudaError_t launch_band_energy(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, long long k2lo,
+                               long long k2hi, double *partials, double *out4, cudaStream_t st);
+cudaError_t launch_spectrum(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, double *bins,
+                            int nbins, cudaStream_t st);
 
 }  // namespace rlbm
