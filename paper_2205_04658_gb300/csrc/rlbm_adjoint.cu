@@ -24,7 +24,6 @@ namespace rlbm {
 
 template <typename R> struct AdjStir {
   int nrows;
-  const R4<R> *G;    // [nrows][nx] table of the step (Gx.re, Gx.im, Gy.re, Gy.im)
   const R2<R> *EY;   // [nrows][eyp] exp(i 2 pi k_y y / ny)
   int eyp;
 };
@@ -370,29 +369,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
         m = cell_macro<R, VS>(h, M, p.vmax2);
         if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
       }
-      if (FORCE && !LAM) {
-        // two rows per iteration, in two partial sums: both rows' loads are in flight at once
-        const R *ey = reinterpret_cast<const R *>(st.EY);
-        R Fx2 = R(0), Fy2 = R(0);
-        int r = 0;
-        for (; r + 1 < st.nrows; r += 2) {
-          const R4<R> G0 = st.G[(long long)r * g.nx + x], G1 = st.G[(long long)(r + 1) * g.nx + x];
-          const R2<R> E0 = ey_at<R>(ey + (long long)r * 2 * st.eyp, y);
-          const R2<R> E1 = ey_at<R>(ey + (long long)(r + 1) * 2 * st.eyp, y);
-          Fx = fma(G0.x, E0.x, fma(-G0.y, E0.y, Fx));
-          Fy = fma(G0.z, E0.x, fma(-G0.w, E0.y, Fy));
-          Fx2 = fma(G1.x, E1.x, fma(-G1.y, E1.y, Fx2));
-          Fy2 = fma(G1.z, E1.x, fma(-G1.w, E1.y, Fy2));
-        }
-        if (r < st.nrows) {
-          const R4<R> G0 = st.G[(long long)r * g.nx + x];
-          const R2<R> E0 = ey_at<R>(ey + (long long)r * 2 * st.eyp, y);
-          Fx = fma(G0.x, E0.x, fma(-G0.y, E0.y, Fx));
-          Fy = fma(G0.z, E0.x, fma(-G0.w, E0.y, Fy));
-        }
-        Fx += Fx2;
-        Fy += Fy2;
-      }
+      // (without kappa_{n+1}, the state's force meets a zero adjoint: the body force stands in)
       cell_adjoint<R, VS, FORCE>(h, lam, M, m, p.omega0, p.fpref, Fx, Fy, cj, kap, gom, gFx, gFy);
       jv = cj * R(0.5) * (m.vx * m.vx + m.vy * m.vy);
     }
@@ -908,7 +885,6 @@ static cudaError_t launch_adjoint_v(const AdjointArgs &a, const Geometry<typenam
   using R = typename RealOf<S>::type;
   AdjStir<R> s;
   s.nrows = FORCE ? a.nrows : 0;
-  s.G = (const R4<R> *)a.G;
   s.EY = (const R2<R> *)a.EY;
   s.eyp = a.eyp;
   if (a.kin) {

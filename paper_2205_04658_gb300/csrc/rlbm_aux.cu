@@ -162,7 +162,7 @@ struct SumD {
   __device__ __forceinline__ double value() const { return v; }
 };
 struct SumF {
-  DF2 v;
+  DF2 v{F2(0.0f), F2(0.0f)};
   __device__ __forceinline__ void add(Cf z) { const DF2 d = df_of(z); v = df_add(v, df_mul(d, d)); }
   __device__ __forceinline__ double value() const {
     return ((double)v.h.v.x + (double)v.h.v.y) + ((double)v.l.v.x + (double)v.l.v.y);

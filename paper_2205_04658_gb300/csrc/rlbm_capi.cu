@@ -73,7 +73,7 @@ int halo_faces(const rlbm_config &c) {
 bool needs_mask(const rlbm_config &c) { return c.solid || c.walls_y || (is_strip(c) && c.strip_solid_halo); }
 
 struct Layout {
-  size_t pop[2], nbmask, err, ctr, EY, G[2], coef[2], mode_kx, row_start, mode_scale;
+  size_t pop[2], nbmask, err, ctr, EY, G[2], tw, mode_kx, row_start, mode_scale;
   size_t eps, ux, uy, partials, totals, twx, twy, z0, z1, bins, cols, sync, total;
   long long plane;
   int pitch, xoff, Q, nrows, nmodes, max_bins, eyp;
@@ -111,8 +111,7 @@ Layout make_layout(const rlbm_config &c) {
   L.EY = take(2 * rb * (size_t)L.nrows * L.eyp);
   L.G[0] = take(4 * rb * (size_t)L.nrows * c.nx);
   L.G[1] = take(4 * rb * (size_t)L.nrows * c.nx);
-  L.coef[0] = take(4 * rb * L.nmodes);
-  L.coef[1] = take(4 * rb * L.nmodes);
+  L.tw = take(L.nmodes ? 2 * rb * (size_t)c.nx : 0);
   L.mode_kx = take(4 * L.nmodes);
   L.row_start = take(4 * (L.nrows + 1));
   L.mode_scale = take(8 * L.nmodes);
@@ -399,31 +398,33 @@ HostStir stir_for_step(rlbm_ctx *c, int64_t n) {
   if (L.nmodes == 0) return s;
   s.G_cur = c->ws + L.G[n & 1];
   s.G_next = c->ws + L.G[(n + 1) & 1];
-  s.coef_next = c->ws + L.coef[(n + 1) & 1];
-  s.coef_new = c->ws + L.coef[n & 1];
+  s.step_next = n + 1;
   s.EY = c->ws + L.EY;
   s.eyp = L.eyp;
   s.mode_kx = c->at<int>(L.mode_kx);
   s.row_start = c->at<int>(L.row_start);
+  s.tw = c->ws + L.tw;
   s.seed = c->cfg.seed;
-  s.step_new = n + 2;
   s.amp = c->cfg.force_amp;
   s.mode_scale = c->unit_scale ? nullptr : c->at<double>(L.mode_scale);
   return s;
 }
 
-// Coefficients of steps n and n+1 and the table of step n.
-cudaError_t stir_prime(rlbm_ctx *c, int64_t n) {
+// The stirring tables of steps n .. n + count - 1 at G, `table` bytes apart.
+cudaError_t stir_tables(rlbm_ctx *c, int64_t n, int count, void *G, size_t table) {
   if (c->L.nmodes == 0) return cudaSuccess;
-  HostStir s = stir_for_step(c, n);
-  void *cn = c->ws + c->L.coef[n & 1], *cn1 = c->ws + c->L.coef[(n + 1) & 1], *G = c->ws + c->L.G[n & 1];
+  const HostStir s = stir_for_step(c, n);
+  const long long entries = (long long)(table / (4 * real_bytes(c->cfg.precision)));
   switch (c->cfg.precision) {
-    case RLBM_F64: return launch_stir_prime_f64(s, cn, cn1, G, c->cfg.nx, n, c->stream);
-    case RLBM_F32: return launch_stir_prime_f32(s, cn, cn1, G, c->cfg.nx, n, c->stream);
-    case RLBM_F16: return launch_stir_prime_f16(s, cn, cn1, G, c->cfg.nx, n, c->stream);
-    default: return launch_stir_prime_bf16(s, cn, cn1, G, c->cfg.nx, n, c->stream);
+    case RLBM_F64: return launch_stir_tables_f64(s, G, entries, c->cfg.nx, n, count, c->stream);
+    case RLBM_F32: return launch_stir_tables_f32(s, G, entries, c->cfg.nx, n, count, c->stream);
+    case RLBM_F16: return launch_stir_tables_f16(s, G, entries, c->cfg.nx, n, count, c->stream);
+    default: return launch_stir_tables_bf16(s, G, entries, c->cfg.nx, n, count, c->stream);
   }
 }
+
+// The table of step n (each step's launch builds the next one's).
+cudaError_t stir_prime(rlbm_ctx *c, int64_t n) { return stir_tables(c, n, 1, c->ws + c->L.G[n & 1], 0); }
 
 // Waits for the stream, reads the device error word and latches it.  The word comes in one
 // copy with the small results behind it (up to byte offset `end` of the workspace), which the
@@ -620,31 +621,35 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   // stirring tables (library's own; FP64-built, stored in the compute type)
   if (L.nmodes) {
     const Modes m = shell_modes(cfg->kmin, cfg->kmax);
-    // phase rows in the layout of ey_index: per row 2 eyp reals, blocks of 8 lattice rows,
-    // entry k of a block = (Re y, Re y+1, Im y, Im y+1) for y = 8 b + 2 k
-    // (the phase of lattice row y0 + y for a strip starting at row y0 of ny_t rows)
+    // phase rows of eyp entries (re, im): the phase of lattice row y0 + y for a strip starting at
+    // row y0 of ny_t rows
     std::vector<double> ey((size_t)L.nrows * 2 * L.eyp, 0.0);
     const long long y0 = is_strip(*cfg) ? cfg->strip_y0 : 0, nyt = total_rows(*cfg);
     for (int r = 0; r < L.nrows; ++r)
       for (int y = 0; y < cfg->ny; ++y) {
         const long long j = ((long long)m.row_ky[r] * (y0 + y)) % nyt;
-        const size_t i = (size_t)r * 2 * L.eyp + ey_index(y);
+        const size_t i = (size_t)r * 2 * L.eyp + 2 * y;
         ey[i] = std::cos(2.0 * M_PI * (double)j / (double)nyt);
-        ey[i + 2] = std::sin(2.0 * M_PI * (double)j / (double)nyt);
+        ey[i + 1] = std::sin(2.0 * M_PI * (double)j / (double)nyt);
       }
-    keep.emplace_back();
-    if (cfg->precision == RLBM_F64) {
-      keep.back().resize(ey.size() * sizeof(double));
-      std::memcpy(keep.back().data(), ey.data(), ey.size() * sizeof(double));
-    } else {
-      keep.back().resize(ey.size() * sizeof(float));
-      float *pf = reinterpret_cast<float *>(keep.back().data());
-      for (size_t i = 0; i < ey.size(); ++i) pf[i] = (float)ey[i];
+    std::vector<double> tw(2 * (size_t)cfg->nx);
+    for (int j = 0; j < cfg->nx; ++j) { tw[2 * j] = std::cos(2.0 * M_PI * j / cfg->nx); tw[2 * j + 1] = std::sin(2.0 * M_PI * j / cfg->nx); }
+    for (const std::vector<double> *v : {&tw, &ey}) {  // in the compute type
+      keep.emplace_back();
+      if (cfg->precision == RLBM_F64) {
+        keep.back().resize(v->size() * sizeof(double));
+        std::memcpy(keep.back().data(), v->data(), v->size() * sizeof(double));
+      } else {
+        keep.back().resize(v->size() * sizeof(float));
+        float *pf = reinterpret_cast<float *>(keep.back().data());
+        for (size_t i = 0; i < v->size(); ++i) pf[i] = (float)(*v)[i];
+      }
     }
     const std::vector<double> ones(L.nmodes, 1.0);
     keep.emplace_back(reinterpret_cast<const uint8_t *>(ones.data()), reinterpret_cast<const uint8_t *>(ones.data()) + 8 * ones.size());
     if ((e = put(L.mode_scale, keep.back().data(), keep.back().size())) != cudaSuccess ||
         (e = put(L.EY, keep[keep.size() - 2].data(), keep[keep.size() - 2].size())) != cudaSuccess ||
+        (e = put(L.tw, keep[keep.size() - 3].data(), keep[keep.size() - 3].size())) != cudaSuccess ||
         (e = put(L.mode_kx, m.kx.data(), 4 * m.kx.size())) != cudaSuccess ||
         (e = put(L.row_start, m.row_start.data(), 4 * m.row_start.size())) != cudaSuccess) {
       c->cuda_fail(e, "upload of the stirring tables");
@@ -1004,8 +1009,8 @@ struct rlbm_batch {
   cudaStream_t stream = nullptr;
   int device = 0;
   MemberDesc *d_mem = nullptr;
-  int *d_tile0 = nullptr, *d_draw0 = nullptr;
-  long long *d_entry0 = nullptr, *d_bstep = nullptr;
+  int *d_tile0 = nullptr, *d_prep0 = nullptr;
+  long long *d_bstep = nullptr;
   int *d_tctr = nullptr;  // the batched kernel's tile counter
   std::vector<MemberDesc> h_mem;
   int ntiles = 0, srows = 0, stages = 2, grid_limit = 0;
@@ -1019,7 +1024,7 @@ struct rlbm_batch {
 
 namespace {
 
-struct BatchLayout { size_t mem, tile0, entry0, draw0, bstep, tctr, total; };
+struct BatchLayout { size_t mem, tile0, prep0, bstep, tctr, total; };
 
 BatchLayout batch_layout(int n) {
   BatchLayout L{};
@@ -1027,8 +1032,7 @@ BatchLayout batch_layout(int n) {
   auto take = [&](size_t b) { size_t o = off; off += align_up(std::max<size_t>(b, 1)); return o; };
   L.mem = take(sizeof(MemberDesc) * (size_t)n);
   L.tile0 = take(sizeof(int) * (size_t)(n + 1));
-  L.entry0 = take(sizeof(long long) * (size_t)(n + 1));
-  L.draw0 = take(sizeof(int) * (size_t)(n + 1));
+  L.prep0 = take(sizeof(int) * (size_t)(n + 1));
   L.bstep = take(sizeof(long long));
   L.tctr = take(sizeof(int));
   L.total = off;
@@ -1048,6 +1052,7 @@ cudaError_t batch_prepare(rlbm_batch *b) {
   for (size_t i = 0; i < b->members.size(); ++i) {
     b->h_mem[i].cur0 = b->members[i]->cur;
     b->h_mem[i].step0 = b->members[i]->step;
+    b->h_mem[i].mode_scale = b->members[i]->unit_scale ? nullptr : b->members[i]->at<double>(b->members[i]->L.mode_scale);
   }
   cudaError_t e = cudaMemcpyAsync(b->d_mem, b->h_mem.data(), sizeof(MemberDesc) * b->h_mem.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bstep, 0, sizeof(long long), b->stream);
@@ -1057,7 +1062,7 @@ cudaError_t batch_prepare(rlbm_batch *b) {
 
 cudaError_t batch_launch_one(rlbm_batch *b) {
   rlbm_ctx *c0 = b->members[0];
-  BatchTables bt{b->d_mem, b->d_tile0, b->d_entry0, b->d_draw0, b->d_tctr, (int)b->members.size()};
+  BatchTables bt{b->d_mem, b->d_tile0, b->d_prep0, b->d_tctr, (int)b->members.size()};
   cudaError_t e;
   const double amp = c0->cfg.force_amp;
   switch (c0->cfg.precision) {
@@ -1105,15 +1110,13 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
   b->device = members[0]->device;
   b->d_mem = reinterpret_cast<MemberDesc *>(b->ws + L.mem);
   b->d_tile0 = reinterpret_cast<int *>(b->ws + L.tile0);
-  b->d_entry0 = reinterpret_cast<long long *>(b->ws + L.entry0);
-  b->d_draw0 = reinterpret_cast<int *>(b->ws + L.draw0);
+  b->d_prep0 = reinterpret_cast<int *>(b->ws + L.prep0);
   b->d_bstep = reinterpret_cast<long long *>(b->ws + L.bstep);
   b->d_tctr = reinterpret_cast<int *>(b->ws + L.tctr);
   b->stages = members[0]->stages;
   const int nrows = members[0]->L.nrows;
   b->srows = (nrows > 0 && nrows <= 16) ? nrows : 0;
-  std::vector<int> tile0(nmembers + 1, 0), draw0(nmembers + 1, 0);
-  std::vector<long long> entry0(nmembers + 1, 0);
+  std::vector<int> tile0(nmembers + 1, 0), prep0(nmembers + 1, 0);
   b->h_mem.resize(nmembers);
   for (int i = 0; i < nmembers; ++i) {
     rlbm_ctx *c = members[i];
@@ -1124,25 +1127,24 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
     d.f[0] = c->ws + c->L.pop[0]; d.f[1] = c->ws + c->L.pop[1];
     d.nbmask = c->geom.nbmask;
     d.nx = c->cfg.nx; d.ny = c->cfg.ny; d.pitch = c->L.pitch; d.walls = c->cfg.walls_y; d.plane = c->L.plane;
-    d.nrows = c->L.nrows; d.nmodes = c->L.nmodes; d.eyp = c->L.eyp;
+    d.nrows = c->L.nrows; d.eyp = c->L.eyp;
     d.G[0] = c->ws + c->L.G[0]; d.G[1] = c->ws + c->L.G[1]; d.EY = c->ws + c->L.EY;
-    d.coef[0] = c->ws + c->L.coef[0]; d.coef[1] = c->ws + c->L.coef[1];
+    d.tw = c->ws + c->L.tw;
     d.mode_kx = c->at<int>(c->L.mode_kx); d.row_start = c->at<int>(c->L.row_start);
     d.seed = c->cfg.seed; d.round_key = c->phys.round_key; d.err = c->at<unsigned>(c->L.err);
     d.ntx = (c->cfg.nx + 31) / 32;
     d.rcp_ntx = 1.0f / (float)d.ntx;
     const int nt = d.ntx * ((c->cfg.ny + 7) / 8);
     tile0[i + 1] = tile0[i] + nt;
-    entry0[i + 1] = entry0[i] + (c->L.nmodes ? (long long)c->L.nrows * c->cfg.nx : 0);
-    draw0[i + 1] = draw0[i] + c->L.nmodes;
+    const int chunk = c->cfg.precision == RLBM_F64 ? stir_chunk<double>() : stir_chunk<float>();
+    prep0[i + 1] = prep0[i] + c->L.nrows * ((c->cfg.nx + chunk - 1) / chunk);
     if (c->geom.nbmask) b->mask = true;
   }
   b->ntiles = tile0[nmembers];
   Scoped dev(b->device);
   cudaError_t e;
   if ((e = cudaMemcpyAsync(b->d_tile0, tile0.data(), sizeof(int) * (nmembers + 1), cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(b->d_entry0, entry0.data(), sizeof(long long) * (nmembers + 1), cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(b->d_draw0, draw0.data(), sizeof(int) * (nmembers + 1), cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(b->d_prep0, prep0.data(), sizeof(int) * (nmembers + 1), cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
       (e = batch_prepare(b)) != cudaSuccess || (e = cudaStreamSynchronize(b->stream)) != cudaSuccess) {
     g_thread_error = std::string("batch tables upload: ") + cudaGetErrorString(e);
     delete b;
@@ -1171,7 +1173,7 @@ rlbm_status rlbm_batch_autotune(rlbm_batch *b, int32_t reps, double *ms_out) {
   if (cudaError_t e0_ = batch_prepare(b); e0_ != cudaSuccess) return b->cuda_fail(e0_, "batch descriptor upload");
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-  BatchTables bt{b->d_mem, b->d_tile0, b->d_entry0, b->d_draw0, b->d_tctr, (int)b->members.size()};
+  BatchTables bt{b->d_mem, b->d_tile0, b->d_prep0, b->d_tctr, (int)b->members.size()};
   rlbm_ctx *c0 = b->members[0];
   const double amp = c0->cfg.force_amp;
   // one batched step without advancing the step counter: every member's next buffer and
@@ -1280,7 +1282,7 @@ struct GradLayout {
   int64_t N;
   int seg, K, nslots;
   size_t state_bytes, kap_bytes, table_bytes, zpart_bytes;
-  size_t ckpt, slots, kap[2], acc, gst, zpart, zsum, tw, twf, gstep, gsig, out, macro, scratch, gscratch, total;
+  size_t ckpt, slots, kap[2], acc, gst, zpart, zsum, tw, twf, gstep, gsig, out, macro, scratch, total;
   size_t macro_bytes;
   long long nblocks;
   int nby;
@@ -1321,7 +1323,6 @@ GradLayout grad_layout(const rlbm_ctx *c, int64_t N, int32_t segment) {
   G.macro_bytes = align_up((5 + (size_t)c->L.Q) * rb * (size_t)c->cfg.nx * c->cfg.ny);
   G.macro = take(G.macro_bytes * G.seg);
   G.scratch = take(G.state_bytes);   // output of the last recomputed step of a segment (unused)
-  G.gscratch = take(G.table_bytes);  // and the stirring rows it prepares for the next step
   G.total = off;
   return G;
 }
@@ -1485,14 +1486,9 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
   // states B_lo .. B_{hi-2} alternate between the two ping-pong slots (B_{hi-1} goes to the
   // scratch state)
   auto recompute = [&](int k, int64_t lo, int64_t hi) -> cudaError_t {
-    cudaError_t e2;
-    if (c->L.nmodes) {
-      HostStir sp = stir_for_step(c, s0 + lo);
-      void *cn = c->ws + c->L.coef[(s0 + lo) & 1], *cn1 = c->ws + c->L.coef[(s0 + lo + 1) & 1];
-      e2 = c->cfg.precision == RLBM_F64 ? launch_stir_prime_f64(sp, cn, cn1, gtab(0), c->cfg.nx, s0 + lo, c->stream)
-                                        : launch_stir_prime_f32(sp, cn, cn1, gtab(0), c->cfg.nx, s0 + lo, c->stream);
-      if (e2 != cudaSuccess) return e2;
-    }
+    // (all tables of the segment in one launch: the steps then build none)
+    cudaError_t e2 = stir_tables(c, s0 + lo, (int)(hi - lo), gtab(0), G.table_bytes);
+    if (e2 != cudaSuccess) return e2;
     // steps lo .. hi-1 again, each keeping its cells' Landau solution, force and streamed h
     // for the reverse step of the same index (the last one's state and next rows are not needed)
     for (int64_t n = lo; n <= hi - 1; ++n) {
@@ -1500,7 +1496,7 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
       HostStir st = stir_for_step(c, s0 + n);
       if (c->L.nmodes) {
         st.G_cur = gtab((int)(n - lo));
-        st.G_next = n == hi - 1 ? w + G.gscratch : gtab((int)(n - lo + 1));
+        st.G_next = nullptr;
       }
       c->phys.step = s0 + n;
       void *fout = n == hi - 1 ? w + G.scratch : slot((int)((n - lo) & 1));
@@ -1536,7 +1532,6 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
   a.macro = nullptr;  // S_N is no step's input: matched and forced here
   a.kout = w + G.kap[kc];
   a.cj = cj;
-  a.G = c->ws + c->L.G[0];
   a.zpart = w + G.zpart;
   if ((e = dispatch_adjoint(c, a)) != cudaSuccess) return c->cuda_fail(e, "adjoint kernel launch");
   for (int k = G.K - 1; k >= 0; --k) {
@@ -1552,7 +1547,6 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
       a.tK = &mkap[kc];
       a.kout = w + G.kap[kc ^ 1];
       a.cj = n >= 1 ? cj : 0.0;
-      a.G = gtab((int)(n - lo));
       a.zpart = w + G.zpart + G.zpart_bytes * (size_t)(n - lo);
       a.macro = w + G.macro + G.macro_bytes * (size_t)(n - lo);
       a.chained = n < hi - 1;  // the first reverse step of a segment follows its recomputation

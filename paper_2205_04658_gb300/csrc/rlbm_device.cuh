@@ -216,22 +216,24 @@ __device__ __forceinline__ uint32_t round_pair_f16_rn(float a, float b) {
   return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// The stirring modes of a lattice, grouped in rows of equal k_y (device pointers).
+struct StirModes {
+  const int *kx;          // [nmodes]
+  const int *row_start;   // [nrows + 1] mode range of each row (modes sorted by k_y)
+  const void *tw;         // [nx] R2: exp(i 2 pi j / nx)
+  const double *scale;    // [nmodes] amplitude multipliers sigma_m; NULL = all 1
+  unsigned long long seed;
+  double amp;
+};
+
 template <typename R> struct Stir {
   int nrows;               // distinct k_y of the shell (0 = no stirring)
-  int nmodes;
-  const R4<R> *G_cur;      // [nrows][nx]: (Gx.re, Gx.im, Gy.re, Gy.im) of this step
+  const R4<R> *G_cur;      // [nrows][nx]: (Gx.re, -Gx.im, Gy.re, -Gy.im) of this step
   const R2<R> *EY;         // [nrows][eyp]: exp(i 2 pi k_y(row) y / ny), rows padded to eyp
   int eyp;
-  // pipelined preparation of the next steps (done by the same launch)
-  R4<R> *G_next;           // [nrows][nx] of step n+1
-  const R4<R> *coef_next;  // [nmodes]: (cx.re, cx.im, cy.re, cy.im) of step n+1
-  R4<R> *coef_new;         // [nmodes] of step n+2 (written)
-  const int *mode_kx;      // [nmodes]
-  const int *row_start;    // [nrows+1] mode range of each row (modes sorted by k_y)
-  unsigned long long seed;
-  long long step_new;      // n + 2
-  double amp;
-  const double *mode_scale;  // [nmodes] amplitude multipliers sigma_m; NULL = all 1
+  R4<R> *G_next;           // the table of step step_next, built by the same launch (NULL: none)
+  long long step_next;
+  StirModes modes;
 };
 
 // ---------------------------------------------------------------------------
@@ -264,135 +266,6 @@ __device__ inline void stir_draw(unsigned long long seed, long long n, int m, do
   out[2] = a * spsi * cphi; out[3] = a * spsi * sphi;
 }
 
-// exp(i pi a) for the stirring phases: FP64 in the FP64 path, FP32 (about 1 ulp) in the
-// others.
-template <typename R> __device__ __forceinline__ void sincospi_R(R a, R *s, R *c);
-template <> __device__ __forceinline__ void sincospi_R<double>(double a, double *s, double *c) { sincospi(a, s, c); }
-template <> __device__ __forceinline__ void sincospi_R<float>(float a, float *s, float *c) { sincospif(a, s, c); }
-
-// One entry of the per-row stirring table of a step:
-//   G_r(x) = sum_{m in row r} (cx_m, cy_m) exp(i 2 pi k_x,m x / nx),
-// the phase evaluated from the exact integer residue k_x,m x mod nx.  The modes of a row
-// are summed in four interleaved parts (m = first + l, l + 4, ...), combined as
-// (p0 + p1) + (p2 + p3): the table builders that split an entry over four lanes and those
-// that do not then give the same bits.  `coef`, `kx` and `row_start` may live in shared
-// memory.
-template <typename R>
-__device__ inline R4<R> stir_entry_part(const R4<R> *coef, const int *kx, const int *row_start, int r, int x, int nx,
-                                        int l4) {
-  R4<R> g{R(0), R(0), R(0), R(0)};
-  const int m1 = row_start[r + 1];
-  for (int m = row_start[r] + l4; m < m1; m += 4) {
-    int j = (kx[m] * x) % nx;  // |k_x| < nx / 2 and x < nx <= 32768: no 32-bit overflow
-    if (j < 0) j += nx;
-    R sn, cs;
-    sincospi_R<R>(R(2 * j) / R(nx), &sn, &cs);
-    const R4<R> c = coef[m];
-    g.x = fma(c.x, cs, fma(-c.y, sn, g.x));
-    g.y = fma(c.x, sn, fma(c.y, cs, g.y));
-    g.z = fma(c.z, cs, fma(-c.w, sn, g.z));
-    g.w = fma(c.z, sn, fma(c.w, cs, g.w));
-  }
-  return g;
-}
-
-template <typename R> __device__ __forceinline__ R4<R> r4_sum(const R4<R> &a, const R4<R> &b) {
-  return R4<R>{a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
-}
-
-template <typename R>
-__device__ inline R4<R> stir_row_entry(const R4<R> *coef, const int *kx, const int *row_start, int r, int x, int nx) {
-  const R4<R> p0 = stir_entry_part<R>(coef, kx, row_start, r, x, nx, 0);
-  const R4<R> p1 = stir_entry_part<R>(coef, kx, row_start, r, x, nx, 1);
-  const R4<R> p2 = stir_entry_part<R>(coef, kx, row_start, r, x, nx, 2);
-  const R4<R> p3 = stir_entry_part<R>(coef, kx, row_start, r, x, nx, 3);
-  return r4_sum<R>(r4_sum<R>(p0, p1), r4_sum<R>(p2, p3));
-}
-
-template <typename R>
-__device__ inline R4<R> stir_row_entry(const Stir<R> &s, const R4<R> *coef, int r, int x, int nx) {
-  return stir_row_entry<R>(coef, s.mode_kx, s.row_start, r, x, nx);
-}
-
-// The table of step n+1 by `ncta` CTAs of a launch (this one has rank `rank`), with the
-// mode coefficients, k_x and row ranges first copied to shared memory `sm` when they fit
-// in `sm_bytes`.  Entry e goes to CTA e mod ncta, thread (e div ncta) mod nthr.
-template <typename R>
-__device__ inline void stir_table_part(const Stir<R> &s, int rank, int ncta, int tid, int nthr, int nx,
-                                       unsigned char *sm, int sm_bytes) {
-  if (s.nrows == 0) return;
-  const R4<R> *coef = s.coef_next;
-  const int *kx = s.mode_kx, *rs = s.row_start;
-  const int need = s.nmodes * (int)(sizeof(R4<R>) + sizeof(int)) + (s.nrows + 1) * (int)sizeof(int);
-  if (sm && need <= sm_bytes) {
-    R4<R> *c2 = reinterpret_cast<R4<R> *>(sm);
-    int *k2 = reinterpret_cast<int *>(c2 + s.nmodes);
-    int *r2 = k2 + s.nmodes;
-    for (int i = tid; i < s.nmodes; i += nthr) { c2[i] = coef[i]; k2[i] = kx[i]; }
-    for (int i = tid; i <= s.nrows; i += nthr) r2[i] = rs[i];
-    __syncthreads();
-    coef = c2; kx = k2; rs = r2;
-  }
-  const long long entries = (long long)s.nrows * nx;
-  for (long long e = rank + (long long)ncta * tid; e < entries; e += (long long)ncta * nthr)
-    s.G_next[e] = stir_row_entry<R>(coef, kx, rs, (int)(e / nx), (int)(e % nx), nx);
-}
-
-// The per-row phase table EY_r(y) = exp(i 2 pi k_y(r) y / ny): each k_y row holds 2 eyp
-// reals in blocks of 8 lattice rows; entry k (0..3) of block b holds
-// (Re y, Re y+1, Im y, Im y+1) for y = 8b + 2k.  One 16-byte load then gives a thread of the
-// paired step kernels (cells y and y + 1) both phases as register pairs.
-__host__ __device__ __forceinline__ int ey_index(int y) { return (y >> 3) * 16 + ((y >> 1) & 3) * 4 + (y & 1); }
-template <typename R> __device__ __forceinline__ R2<R> ey_at(const R *row, int y) {
-  const int i = ey_index(y);
-  return R2<R>{row[i], row[i + 2]};
-}
-
-// Byte sizes of the mode data a step launch copies to shared memory for the table of the
-// next step: coefficients (16-byte R4 per mode for FP32, 32 for FP64), k_x and the row
-// ranges, each part padded to 16 bytes (the copies are untiled bulk copies).
-__host__ __device__ inline int mode_coef_bytes(int nmodes, int rbytes) { return nmodes * 4 * rbytes; }
-__host__ __device__ inline int mode_kx_bytes(int nmodes) { return (nmodes * 4 + 15) / 16 * 16; }
-__host__ __device__ inline int mode_rows_bytes(int nrows) { return ((nrows + 1) * 4 + 15) / 16 * 16; }
-
-// This CTA's share of the table of step n+1 from mode data already in shared memory.
-// Entry e goes to CTA e mod ncta.  Within the CTA, quads of lanes take the entries (dealt
-// round-robin over the warps) and split each entry's modes four ways, summing with two
-// shuffles: a row of the shell holds up to a dozen modes, and the longest entry, not the
-// number of entries, sets the time.  Every thread reaches the shuffles the same number of
-// times (all lanes of a warp take part).
-template <typename R>
-__device__ inline void stir_table_staged(const Stir<R> &s, int rank, int ncta, int tid, int nthr, int nx,
-                                         const R4<R> *coef, const int *kx, const int *rs) {
-  const int nwarps = nthr >> 5, nquads = nthr >> 2;
-  const int lane = tid & 31, warp = tid >> 5, l4 = tid & 3;
-  const int quad = warp + nwarps * (lane >> 2);  // quads of one warp are nwarps apart
-  const long long entries = (long long)s.nrows * nx;
-  const long long mine = entries > rank ? (entries - 1 - rank) / ncta + 1 : 0;  // this CTA's entries
-  for (long long base = 0; base < mine; base += nquads) {
-    const long long i = base + quad;
-    R4<R> g{R(0), R(0), R(0), R(0)};
-    int r = 0, x = 0;
-    if (i < mine) {
-      const long long e = rank + i * ncta;
-      r = (int)(e / nx);
-      x = (int)(e % nx);
-      g = stir_entry_part<R>(coef, kx, rs, r, x, nx, l4);
-    }
-    // lane 0 of the quad ends with (p0 + p1) + (p2 + p3), as stir_row_entry
-#pragma unroll
-    for (int off = 1; off < 4; off <<= 1) {
-      R4<R> o;
-      o.x = __shfl_xor_sync(0xffffffffu, g.x, off);
-      o.y = __shfl_xor_sync(0xffffffffu, g.y, off);
-      o.z = __shfl_xor_sync(0xffffffffu, g.z, off);
-      o.w = __shfl_xor_sync(0xffffffffu, g.w, off);
-      g = r4_sum<R>(g, o);
-    }
-    if (i < mine && l4 == 0) s.G_next[(long long)r * nx + x] = g;
-  }
-}
-
 // Mode m of step n in FP32 (the draws of the FP32-compute paths; the uniform u_j and
 // the Box-Muller transform in single precision, about 1e-7 relative).
 __device__ inline void stir_draw_f32(unsigned long long seed, long long n, int m, float amp, float out[4]) {
@@ -409,40 +282,147 @@ __device__ inline void stir_draw_f32(unsigned long long seed, long long n, int m
   out[2] = a * spsi * cphi; out[3] = a * spsi * sphi;
 }
 
-// Philox draws of step n+2: mode m by one thread of the CTA of rank m, m + ncta, ...
-// (FP64 arithmetic in the FP64 path, FP32 in the others: GB300's FP64 rate is 1/64 of
-// FP32, and the draws sit on the critical path of the CTAs that make them).
 template <typename R>
-__device__ inline void stir_draws_part(const Stir<R> &s, int rank, int ncta) {
-  for (int m = rank; m < s.nmodes; m += ncta) {
-    if constexpr (sizeof(R) == 8) {
-      double c[4];
-      stir_draw(s.seed, s.step_new, m, s.mode_scale ? s.amp * s.mode_scale[m] : s.amp, c);
-      s.coef_new[m] = R4<R>{(R)c[0], (R)c[1], (R)c[2], (R)c[3]};
-    } else {
-      float c[4];
-      stir_draw_f32(s.seed, s.step_new, m, (float)(s.mode_scale ? s.amp * s.mode_scale[m] : s.amp), c);
-      s.coef_new[m] = R4<R>{c[0], c[1], c[2], c[3]};
+__device__ __forceinline__ R4<R> stir_draw_r(unsigned long long seed, long long n, int m, double amp) {
+  if constexpr (sizeof(R) == 8) {
+    double c[4];
+    stir_draw(seed, n, m, amp, c);
+    return R4<R>{c[0], c[1], c[2], c[3]};
+  } else {
+    float c[4];
+    stir_draw_f32(seed, n, m, (float)amp, c);
+    return R4<R>{c[0], c[1], c[2], c[3]};
+  }
+}
+
+// One row of a step's stirring table for the columns of one chunk, by one warp:
+//   G_r(x) = sum_{m in row r} (cx_m, cy_m) exp(i 2 pi k_x,m x / nx),
+// kept as (Re, -Im) of both components.  F = Re[G_r(x) exp(i 2 pi k_y y / ny)] is then a sum of
+// products of parts that lie side by side, as packed multiply-adds take them.  Each lane draws
+// modes of the row (Philox is counter-based: no state is kept between steps) and every lane
+// adds all of them for its columns x0 + lane, + 32, ...; the phase is read from the table of
+// the nx roots of unity at the exact residue k_x x mod nx (a sine and cosine per mode and
+// column, as the table was built before, took three times the instructions).
+template <typename R> constexpr int stir_chunk() { return 32 * (sizeof(R) == 8 ? 4 : 8); }
+
+template <typename R>
+__device__ __forceinline__ void stir_row_chunk(const StirModes &s, long long step, int r, int chunk, int nx, int lane,
+                                               R4<R> *row) {
+  constexpr int NCOL = stir_chunk<R>() / 32;
+  const int x0 = chunk * stir_chunk<R>() + lane;
+  const int m1 = s.row_start[r + 1];
+  R4<R> g[NCOL];
+#pragma unroll
+  for (int i = 0; i < NCOL; ++i) g[i] = R4<R>{R(0), R(0), R(0), R(0)};
+  for (int m0 = s.row_start[r]; m0 < m1; m0 += 32) {
+    R4<R> c{R(0), R(0), R(0), R(0)};
+    int kx = 0;
+    if (m0 + lane < m1) {
+      kx = s.kx[m0 + lane];
+      c = stir_draw_r<R>(s.seed, step, m0 + lane, s.scale ? s.amp * s.scale[m0 + lane] : s.amp);
+    }
+    // residues of the lane's first column and of 32 columns (|k_x| < nx / 2, x < 2^15 + 2^8: no overflow)
+    int d = (32 * kx) % nx;
+    if (d < 0) d += nx;
+    const int cnt = m1 - m0 < 32 ? m1 - m0 : 32;
+    for (int k = 0; k < cnt; ++k) {
+      const R4<R> a{__shfl_sync(0xffffffffu, c.x, k), __shfl_sync(0xffffffffu, c.y, k),
+                    __shfl_sync(0xffffffffu, c.z, k), __shfl_sync(0xffffffffu, c.w, k)};
+      const int kk = __shfl_sync(0xffffffffu, kx, k), dd = __shfl_sync(0xffffffffu, d, k);
+      int j = (kk * x0) % nx;
+      if (j < 0) j += nx;
+#pragma unroll
+      for (int i = 0; i < NCOL; ++i) {
+        R2<R> e;
+        if constexpr (sizeof(R) == 8) {
+          const double2 v = __ldg(reinterpret_cast<const double2 *>(s.tw) + j);
+          e = R2<R>{v.x, v.y};
+        } else {
+          const float2 v = __ldg(reinterpret_cast<const float2 *>(s.tw) + j);
+          e = R2<R>{v.x, v.y};
+        }
+        g[i].x = fma(a.x, e.x, fma(-a.y, e.y, g[i].x));
+        g[i].y = fma(-a.x, e.y, fma(-a.y, e.x, g[i].y));
+        g[i].z = fma(a.z, e.x, fma(-a.w, e.y, g[i].z));
+        g[i].w = fma(-a.z, e.y, fma(-a.w, e.x, g[i].w));
+        j += dd;
+        if (j >= nx) j -= nx;
+      }
     }
   }
+#pragma unroll
+  for (int i = 0; i < NCOL; ++i)
+    if (x0 + 32 * i < nx) row[x0 + 32 * i] = g[i];
+}
+
+// The phase table EY_r(y) = exp(i 2 pi k_y(r) y / ny): rows of eyp entries (re, im).
+template <typename R> __device__ __forceinline__ R2<R> ey_at(const R *row, int y) {
+  return R2<R>{row[2 * y], row[2 * y + 1]};
 }
 
 // ---------------------------------------------------------------------------
 // Arithmetic helpers: exact in FP64, hardware approximations (<= 2 ulp) in FP32.
 // ---------------------------------------------------------------------------
 template <typename T> struct FM;
+// FP64 roots by Newton's method from the FP32 approximation (1e-7), two steps (1e-14, rounding):
+// 8 to 10 FP64 operations where the library functions take about 30, and on GB300 a warp's FP64
+// instruction occupies its quarter of the SM for 64 cycles.  Arguments beyond FP32's range take
+// the library functions.
 template <> struct FM<double> {
+  static __device__ __forceinline__ bool in_range(double x) { return x > 1e-30 && x < 1e30; }
   static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double rsqrt(double x) { return 1.0 / sqrt(x); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-  static __device__ __forceinline__ double qroot(double x) { return sqrt(sqrt(x)); }
-  static __device__ __forceinline__ double croot(double x) { return cbrt(x); }
+  static __device__ __forceinline__ double rsqrt(double x) {
+    if (!in_range(x)) return 1.0 / sqrt(x);
+    double y = (double)rsqrtf((float)x);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    return y;
+  }
+  static __device__ __forceinline__ double qroot(double x) {  // x^(1/4): q += (x - q^4) / (4 q^3)
+    if (!in_range(x)) return sqrt(sqrt(x));
+    const float f = rsqrtf(rsqrtf((float)x));
+    const double c = (double)__fdividef(0.25f, f * f * f);
+    double q = (double)f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const double q2 = q * q;
+      q = fma(c, fma(-q2, q2, x), q);
+    }
+    return q;
+  }
+  static __device__ __forceinline__ double croot(double x) {  // x^(1/3): q += (x - q^3) / (3 q^2)
+    if (!in_range(x)) return cbrt(x);
+    const float f = cbrtf((float)x);
+    const double c = (double)__fdividef(1.0f, 3.0f * f * f);
+    double q = (double)f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) q = fma(c, fma(-q * q, q, x), q);
+    return q;
+  }
 };
+// The .ftz forms are one instruction each; the others bring the scaling of subnormal arguments
+// along (a compare, a select and two multiplications per call, a twentieth of the step
+// kernel's instructions), and no argument here comes near those: T^00, determinants near
+// -(1 + 1/D_p)^2 to -1, 1 - v^2, eps^ > 0 (an eps^ or 1 - v^2 so close to zero is reported as
+// unstable or re-solved in FP64).
 template <> struct FM<float> {
-  static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
-  static __device__ __forceinline__ float rsqrt(float x) { return rsqrtf(x); }
-  static __device__ __forceinline__ float sqrt_(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
-  static __device__ __forceinline__ float qroot(float x) { return rsqrtf(rsqrtf(x)); }
+  static __device__ __forceinline__ float rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+  }
+  static __device__ __forceinline__ float rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+  }
+  static __device__ __forceinline__ float sqrt_(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+  }
+  static __device__ __forceinline__ float qroot(float x) { return rsqrt(rsqrt(x)); }
   static __device__ __forceinline__ float croot(float x) { return cbrtf(x); }
 };
 
@@ -450,7 +430,7 @@ template <> struct FM<float> {
 // add/multiply/FMA (__fadd2_rn, __fmul2_rn, __ffma2_rn) do both in one instruction.
 struct F2 {
   float2 v;
-  __device__ __forceinline__ F2() : v(make_float2(0.0f, 0.0f)) {}
+  F2() = default;  // (uninitialised)
   __device__ __forceinline__ explicit F2(float s) : v(make_float2(s, s)) {}
   __device__ __forceinline__ explicit F2(double s) : v(make_float2((float)s, (float)s)) {}
   __device__ __forceinline__ explicit F2(int s) : v(make_float2((float)s, (float)s)) {}
@@ -505,8 +485,8 @@ __device__ __forceinline__ F2 shfl_xor(F2 a, int off) {
 __device__ __forceinline__ DF2 df_shfl_xor(const DF2 &a, int off) { return DF2{shfl_xor(a.h, off), shfl_xor(a.l, off)}; }
 
 template <> struct FM<F2> {
-  static __device__ __forceinline__ F2 rcp(F2 x) { return F2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
-  static __device__ __forceinline__ F2 rsqrt(F2 x) { return F2(rsqrtf(x.v.x), rsqrtf(x.v.y)); }
+  static __device__ __forceinline__ F2 rcp(F2 x) { return F2(FM<float>::rcp(x.v.x), FM<float>::rcp(x.v.y)); }
+  static __device__ __forceinline__ F2 rsqrt(F2 x) { return F2(FM<float>::rsqrt(x.v.x), FM<float>::rsqrt(x.v.y)); }
   static __device__ __forceinline__ F2 sqrt_(F2 x) { return F2(FM<float>::sqrt_(x.v.x), FM<float>::sqrt_(x.v.y)); }
   static __device__ __forceinline__ F2 qroot(F2 x) { return F2(FM<float>::qroot(x.v.x), FM<float>::qroot(x.v.y)); }
   static __device__ __forceinline__ F2 croot(F2 x) { return F2(cbrtf(x.v.x), cbrtf(x.v.y)); }
@@ -520,23 +500,28 @@ template <> struct FM<F2> {
 // ---------------------------------------------------------------------------
 template <typename T> struct Mom { T e, mx, my, txx, txy, tyy, wxxx, wxxy, wxyy, wyyy; };
 
-// Generic sum over classes with compile-time coefficients.
+// Generic sum over classes with compile-time coefficients.  (The packed intrinsics are never
+// contracted by the compiler, so the multiply-adds are written out.)
 template <typename T, typename R, int VS, bool THIRD>
 __device__ __forceinline__ Mom<T> moments_generic(const R h[VSet<VS>::Q]) {
   using V = VSet<VS>;
-  Mom<T> M{};
+  const T z = T(0);
+  Mom<T> M{z, z, z, z, z, z, z, z, z, z};
 #pragma unroll
   for (int q = 0; q < V::Q; ++q) {
     const double w = V::w(q), vx = V::vx(q), vy = V::vy(q);
     const T hq = (T)h[q];
-    M.e += T(w) * hq;
-    if (vx != 0.0) { M.mx += T(w * vx) * hq; M.txx += T(w * vx * vx) * hq; }
-    if (vy != 0.0) { M.my += T(w * vy) * hq; M.tyy += T(w * vy * vy) * hq; }
-    if (vx != 0.0 && vy != 0.0) M.txy += T(w * vx * vy) * hq;
+    M.e = fma(T(w), hq, M.e);
+    if (vx != 0.0) { M.mx = fma(T(w * vx), hq, M.mx); M.txx = fma(T(w * vx * vx), hq, M.txx); }
+    if (vy != 0.0) { M.my = fma(T(w * vy), hq, M.my); M.tyy = fma(T(w * vy * vy), hq, M.tyy); }
+    if (vx != 0.0 && vy != 0.0) M.txy = fma(T(w * vx * vy), hq, M.txy);
     if (THIRD) {
-      if (vx != 0.0) M.wxxx += T(w * vx * vx * vx) * hq;
-      if (vx != 0.0 && vy != 0.0) { M.wxxy += T(w * vx * vx * vy) * hq; M.wxyy += T(w * vx * vy * vy) * hq; }
-      if (vy != 0.0) M.wyyy += T(w * vy * vy * vy) * hq;
+      if (vx != 0.0) M.wxxx = fma(T(w * vx * vx * vx), hq, M.wxxx);
+      if (vx != 0.0 && vy != 0.0) {
+        M.wxxy = fma(T(w * vx * vx * vy), hq, M.wxxy);
+        M.wxyy = fma(T(w * vx * vy * vy), hq, M.wxyy);
+      }
+      if (vy != 0.0) M.wyyy = fma(T(w * vy * vy * vy), hq, M.wyyy);
     }
   }
   return M;
@@ -545,34 +530,39 @@ __device__ __forceinline__ Mom<T> moments_generic(const R h[VSet<VS>::Q]) {
 // The 17 folded classes of the paper's set come in four sign-symmetric groups
 // {(+a,+b), (-a,+b), (-a,-b), (+a,-b)} (diagonals) or {(+a,0), (0,+a), (-a,0), (0,-a)}
 // (axes).  Sums and differences within a group (a butterfly) give each moment from one
-// product per group instead of one per class.
-template <typename T, typename R, bool THIRD>
+// multiply-add per group instead of one per class.
+template <typename T, bool THIRD>
 __device__ __forceinline__ void moments_axis_group(Mom<T> &M, double w, double a, T h0, T h1, T h2, T h3) {
   // classes (+a,0), (0,+a), (-a,0), (0,-a)
   const T sx = h0 + h2, dx = h0 - h2, sy = h1 + h3, dy = h1 - h3;
-  M.e += T(w) * (sx + sy);
-  M.mx += T(w * a) * dx;
-  M.my += T(w * a) * dy;
-  M.txx += T(w * a * a) * sx;
-  M.tyy += T(w * a * a) * sy;
-  if (THIRD) { M.wxxx += T(w * a * a * a) * dx; M.wyyy += T(w * a * a * a) * dy; }
+  M.e = fma(T(w), sx + sy, M.e);
+  M.mx = fma(T(w * a), dx, M.mx);
+  M.my = fma(T(w * a), dy, M.my);
+  M.txx = fma(T(w * a * a), sx, M.txx);
+  M.tyy = fma(T(w * a * a), sy, M.tyy);
+  if (THIRD) { M.wxxx = fma(T(w * a * a * a), dx, M.wxxx); M.wyyy = fma(T(w * a * a * a), dy, M.wyyy); }
 }
-template <typename T, typename R, bool THIRD>
-__device__ __forceinline__ void moments_diag_group(Mom<T> &M, double w, double a, T h0, T h1, T h2, T h3) {
+// The diagonal groups (a, w) and (b, u) together: they alone reach t_xy, w_xxy and w_xyy.
+template <typename T, bool THIRD>
+__device__ __forceinline__ void moments_diag_groups(Mom<T> &M, double w, double a, T h0, T h1, T h2, T h3, double u,
+                                                    double b, T g0, T g1, T g2, T g3) {
   // classes (+a,+a), (-a,+a), (-a,-a), (+a,-a)
   const T s02 = h0 + h2, d02 = h0 - h2, s13 = h1 + h3, d31 = h3 - h1;
   const T P0 = s02 + s13, Pxy = s02 - s13, Px = d02 + d31, Py = d02 - d31;
-  M.e += T(w) * P0;
-  M.txx += T(w * a * a) * P0;
-  M.tyy += T(w * a * a) * P0;
-  M.mx += T(w * a) * Px;
-  M.my += T(w * a) * Py;
-  M.txy += T(w * a * a) * Pxy;
+  const T r02 = g0 + g2, c02 = g0 - g2, r13 = g1 + g3, c31 = g3 - g1;
+  const T Q0 = r02 + r13, Qxy = r02 - r13, Qx = c02 + c31, Qy = c02 - c31;
+  M.e = fma(T(u), Q0, fma(T(w), P0, M.e));
+  const T t2 = fma(T(u * b * b), Q0, T(w * a * a) * P0);
+  M.txx += t2;
+  M.tyy += t2;
+  M.mx = fma(T(u * b), Qx, fma(T(w * a), Px, M.mx));
+  M.my = fma(T(u * b), Qy, fma(T(w * a), Py, M.my));
+  M.txy = fma(T(u * b * b), Qxy, T(w * a * a) * Pxy);
   if (THIRD) {
-    M.wxxx += T(w * a * a * a) * Px;
-    M.wxyy += T(w * a * a * a) * Px;
-    M.wxxy += T(w * a * a * a) * Py;
-    M.wyyy += T(w * a * a * a) * Py;
+    M.wxyy = fma(T(u * b * b * b), Qx, T(w * a * a * a) * Px);
+    M.wxxy = fma(T(u * b * b * b), Qy, T(w * a * a * a) * Py);
+    M.wxxx += M.wxyy;
+    M.wyyy += M.wxxy;
   }
 }
 
@@ -580,12 +570,21 @@ template <typename T, typename R, int VS, bool THIRD>
 __device__ __forceinline__ Mom<T> moments_of(const R h[VSet<VS>::Q]) {
   if constexpr (VS == 3) {
     using V = VSet<3>;
-    Mom<T> M{};
-    M.e = T(V::w(0)) * (T)h[0];
-    moments_axis_group<T, R, THIRD>(M, V::w(1), 1.0, (T)h[1], (T)h[2], (T)h[3], (T)h[4]);
-    moments_diag_group<T, R, THIRD>(M, V::w(5), RLBM_S2, (T)h[5], (T)h[6], (T)h[7], (T)h[8]);
-    moments_axis_group<T, R, THIRD>(M, V::w(9), RLBM_S2, (T)h[9], (T)h[10], (T)h[11], (T)h[12]);
-    moments_diag_group<T, R, THIRD>(M, V::w(13), RLBM_S3, (T)h[13], (T)h[14], (T)h[15], (T)h[16]);
+    Mom<T> M;
+    {  // the unit axes start the sums
+      const T sx = (T)h[1] + (T)h[3], dx = (T)h[1] - (T)h[3], sy = (T)h[2] + (T)h[4], dy = (T)h[2] - (T)h[4];
+      constexpr double w = V::w(1);
+      M.e = fma(T(w), sx + sy, T(V::w(0)) * (T)h[0]);
+      M.mx = T(w) * dx;
+      M.my = T(w) * dy;
+      M.txx = T(w) * sx;
+      M.tyy = T(w) * sy;
+      M.wxxx = M.mx;
+      M.wyyy = M.my;
+    }
+    moments_axis_group<T, THIRD>(M, V::w(9), RLBM_S2, (T)h[9], (T)h[10], (T)h[11], (T)h[12]);
+    moments_diag_groups<T, THIRD>(M, V::w(5), RLBM_S2, (T)h[5], (T)h[6], (T)h[7], (T)h[8],
+                                  V::w(13), RLBM_S3, (T)h[13], (T)h[14], (T)h[15], (T)h[16]);
     return M;
   } else {
     return moments_generic<T, R, VS, THIRD>(h);
@@ -641,6 +640,39 @@ __device__ __forceinline__ bool landau(const Mom<T> &M, int maxit, T tol, T &vx,
   return (v2 < T(1)) && (T00 - (M.mx * vx + M.my * vy) > T(0)) && (d2 <= tol * lim);
 }
 
+// The FP64 solution from the FP32 one: the residual R(v) in FP64, the correction -J^{-1} R in FP32
+// with the FP32 Jacobian, whose relative error (about 1e-6) is the factor by which a step reduces
+// the error: two steps from FP32's 1e-7 to rounding, some 30 FP64 operations in place of four
+// full Newton steps with an FP64 division each.  False when it has not converged (the full FP64
+// iteration decides then).
+template <int VS> __device__ __forceinline__ bool landau_refined(const Mom<double> &M, double &vx, double &vy) {
+  Mom<float> f;
+  f.e = (float)M.e; f.mx = (float)M.mx; f.my = (float)M.my;
+  f.txx = (float)M.txx; f.txy = (float)M.txy; f.tyy = (float)M.tyy;
+  float x, y;
+  if (!landau<float, VS>(f, 4, 3e-4f, x, y)) return false;
+  const float dinvf = 1.0f / VSet<VS>::DP;
+  const float E = 1.0f + f.e - (f.mx * x + f.my * y);
+  const float jxx = x * f.mx - (dinvf + f.txx) - E, jxy = x * f.my - f.txy;
+  const float jyx = y * f.mx - f.txy, jyy = y * f.my - (dinvf + f.tyy) - E;
+  const float idet = __fdividef(1.0f, jxx * jyy - jxy * jyx);
+  constexpr double dinv = 1.0 / VSet<VS>::DP;
+  const double nxx = -(dinv + M.txx), nyy = -(dinv + M.tyy), n00 = -(1.0 + M.e);
+  vx = (double)x;
+  vy = (double)y;
+  for (int it = 0; it < 4; ++it) {
+    const double nE = fma(M.mx, vx, fma(M.my, vy, n00));
+    const float rx = (float)fma(nxx + nE, vx, fma(-M.txy, vy, M.mx));
+    const float ry = (float)fma(nyy + nE, vy, fma(-M.txy, vx, M.my));
+    const float dx = (jxy * ry - jyy * rx) * idet, dy = (jyx * rx - jxx * ry) * idet;
+    vx += (double)dx;
+    vy += (double)dy;
+    // after a step of 1e-11 |v| the error is below rounding (the factor 1e-6 above)
+    if (fabsf(dx) + fabsf(dy) <= 1e-11f * (fabsf(x) + fabsf(y))) return vx * vx + vy * vy < 1.0;
+  }
+  return false;
+}
+
 // Macroscopic result of one cell (eps^ = eps / eps0, u^mu = gamma (1, v)).
 template <typename T> struct Macro { T eps_m1, u0, ux, uy, vx, vy; bool ok; };
 
@@ -648,7 +680,13 @@ template <typename T, int VS>
 __device__ __forceinline__ Macro<T> macro_from(const Mom<T> &M, int maxit, T tol) {
   Macro<T> r;
   T vx, vy;
-  const bool ok = landau<T, VS>(M, maxit, tol, vx, vy);
+  bool ok;
+  if constexpr (sizeof(T) == 8) {
+    ok = landau_refined<VS>(M, vx, vy);
+    if (!ok) ok = landau<T, VS>(M, maxit, tol, vx, vy);
+  } else {
+    ok = landau<T, VS>(M, maxit, tol, vx, vy);
+  }
   const T v2 = vx * vx + vy * vy;
   const T gam = FM<T>::rsqrt(T(1) - v2);
   r.eps_m1 = M.e - (M.mx * vx + M.my * vy);
@@ -692,30 +730,32 @@ __device__ __forceinline__ Macro<F2> cell_macro_pair(const F2 h[VSet<VS>::Q], co
   if (VS == 3) c = F2(3.0f) * FM<F2>::rcp(F2(2.0f) + FM<F2>::sqrt_(fmax(fma(F2(-3.0f), m2, F2(4.0f)), F2(0.0f))));
   else c = F2(4.0f) * FM<F2>::rcp(F2(3.0f) + FM<F2>::sqrt_(fmax(fma(F2(-8.0f), m2, F2(9.0f)), F2(0.0f))));
   F2 vx = c * ax, vy = c * ay;
-  const F2 Txx = F2(dinv) + M.txx, Txy = M.txy, Tyy = F2(dinv) + M.tyy;
+  // -T^{ab} and -T^00: the residual and its Jacobian then take one multiply-add per term
+  const F2 nxx = fma(M.txx, F2(-1.0f), F2(-dinv)), nxy = -M.txy, nyy = fma(M.tyy, F2(-1.0f), F2(-dinv));
+  const F2 n00 = -T00;
   bool convA = false, convB = false;
   for (int it = 0; it < 4; ++it) {
-    const F2 E = T00 - fma(M.mx, vx, M.my * vy);
-    const F2 rx = M.mx - fma(Txx, vx, Txy * vy) - E * vx;
-    const F2 ry = M.my - fma(Txy, vx, Tyy * vy) - E * vy;
-    const F2 jxx = fma(vx, M.mx, -Txx) - E, jxy = fma(vx, M.my, -Txy);
-    const F2 jyx = fma(vy, M.mx, -Txy), jyy = fma(vy, M.my, -Tyy) - E;
+    const F2 nE = fma(M.mx, vx, fma(M.my, vy, n00));  // -(T^00 - m.v)
+    const F2 bx = nxx + nE, by = nyy + nE;
+    const F2 rx = fma(bx, vx, fma(nxy, vy, M.mx)), ry = fma(by, vy, fma(nxy, vx, M.my));
+    const F2 jxx = fma(vx, M.mx, bx), jxy = fma(vx, M.my, nxy);
+    const F2 jyx = fma(vy, M.mx, nxy), jyy = fma(vy, M.my, by);
     const F2 idet = FM<F2>::rcp(jxx * jyy - jxy * jyx);
     const F2 dx = (jxy * ry - jyy * rx) * idet;
     const F2 dy = (jyx * rx - jxx * ry) * idet;
     vx += F2(convA ? 0.0f : dx.v.x, convB ? 0.0f : dx.v.y);
     vy += F2(convA ? 0.0f : dy.v.x, convB ? 0.0f : dy.v.y);
-    const F2 d2 = fma(dx, dx, dy * dy), lim = F2(tol * tol) * (F2(1e-6f) + fma(vx, vx, vy * vy));
+    const F2 d2 = fma(dx, dx, dy * dy), lim = fma(F2(tol * tol), fma(vx, vx, vy * vy), F2(tol * tol * 1e-6f));
     convA = convA || d2.v.x <= lim.v.x;
     convB = convB || d2.v.y <= lim.v.y;
     if (convA && convB) break;
   }
-  const F2 v2 = fma(vx, vx, vy * vy);
-  const F2 E = T00 - fma(M.mx, vx, M.my * vy);
+  const F2 v2 = fma(vx, vx, vy * vy), mv = fma(M.mx, vx, M.my * vy);
+  const F2 E = T00 - mv;
   const bool okA = convA && v2.v.x < vmax2 && E.v.x > 0.0f, okB = convB && v2.v.y < vmax2 && E.v.y > 0.0f;
   Macro<F2> r;
   const F2 gam = FM<F2>::rsqrt(one - v2);
-  r.eps_m1 = M.e - fma(M.mx, vx, M.my * vy);
+  r.eps_m1 = M.e - mv;
   r.u0 = gam; r.ux = gam * vx; r.uy = gam * vy; r.vx = vx; r.vy = vy;
   r.ok = true;
   if (!okA || !okB) {
@@ -764,28 +804,30 @@ __device__ __forceinline__ Coll<R> coll_coeffs(const Mom<R> &M, const Macro<R> &
   Coll<R> c;
   const R epsh = R(1) + m.eps_m1;
   const R om = VS == 3 ? omega0 * FM<R>::qroot(epsh) : omega0 * FM<R>::croot(epsh);
-  const R u2 = m.ux * m.ux + m.uy * m.uy;
-  const R ca = R(V::CA) * epsh * m.u0, cb = R(V::CB) * epsh, cc = m.eps_m1 - R(V::CC) * epsh * u2;
+  const R u2 = fma(m.ux, m.ux, m.uy * m.uy);
+  const R ca = R(V::CA) * epsh * m.u0, cb = R(V::CB) * epsh, cc = fma(R(-V::CC) * epsh, u2, m.eps_m1);
+  const R omu = om * m.u0;
   c.ux = m.ux; c.uy = m.uy; c.om = om;
-  c.k0 = one - om * m.u0;
-  c.p0 = om * m.u0 * cc;
-  c.p1 = om * (m.u0 * ca - cc);
-  c.p2 = om * (m.u0 * cb - ca);
-  c.p3 = -om * cb;
+  c.k0 = one - omu;
+  c.p0 = omu * cc;
+  c.p1 = om * fma(m.u0, ca, -cc);
+  c.p2 = om * fma(m.u0, cb, -ca);
+  c.p3 = R(-V::CB) * om * epsh;
   c.s0 = c.s1x = c.s1y = c.sxx = c.sxy2 = c.syy = c.szz = R(0);
   if (FORCE) {
-    const R FM1 = Fx * M.mx + Fy * M.my, M0 = R(1) + M.e;
-    const R Bxx = Fx * M.wxxx + Fy * M.wxxy;
-    const R Bxy = Fx * M.wxxy + Fy * M.wxyy;
-    const R Byy = Fx * M.wxyy + Fy * M.wyyy;
+    const R FM1 = fma(Fx, M.mx, Fy * M.my), M0 = R(1) + M.e;
+    const R Bxx = fma(Fx, M.wxxx, Fy * M.wxxy);
+    const R Bxy = fma(Fx, M.wxxy, Fy * M.wxyy);
+    const R Byy = fma(Fx, M.wxyy, Fy * M.wyyy);
     const R Bzz = FM1 - Bxx - Byy;
-    const R f54 = R(1.25) * fpref;
+    const R f54 = R(1.25) * fpref, h = R(-0.5) * fpref * M0;
+    const R Fx2 = R(-2) * Fx, Fy2 = R(-2) * Fy;
     c.s0 = R(0.25) * fpref * FM1;
-    c.s1x = R(-0.5) * fpref * M0 * Fx;
-    c.s1y = R(-0.5) * fpref * M0 * Fy;
-    c.sxx = f54 * (Bxx - R(2) * Fx * M.mx);
-    c.sxy2 = R(2) * f54 * (Bxy - Fx * M.my - Fy * M.mx);
-    c.syy = f54 * (Byy - R(2) * Fy * M.my);
+    c.s1x = h * Fx;
+    c.s1y = h * Fy;
+    c.sxx = f54 * fma(Fx2, M.mx, Bxx);
+    c.sxy2 = f54 * fma(Fx2, M.my, fma(Fy2, M.mx, R(2) * Bxy));
+    c.syy = f54 * fma(Fy2, M.my, Byy);
     c.szz = f54 * Bzz;
   }
   c.s0 += c.p0;
@@ -813,44 +855,45 @@ __device__ __forceinline__ R collide_class(const Coll<R> &c, int q, R h) {
   return fma(h, k, acc);
 }
 
-// All classes of a cell.  For the paper's set the classes of a sign group
-// {(+a,+b), (-a,+b), (-a,-b), (+a,-b)} share a u-projection pair (a u^x, b u^y) and the
-// even part of the force polynomial; only signs differ between the four members.
+// Two opposite classes at once, t = u.v of the first: the polynomial's even part (with the
+// force's even part e) and odd part (with the force's odd part x) are formed once.
+template <typename R>
+__device__ __forceinline__ void collide_opposite(const Coll<R> &c, R t, R e, R x, R hp, R hm, R &op, R &om) {
+  const R t2 = t * t, ot = c.om * t;
+  const R even = fma(t2, c.p2, e), odd = fma(t, fma(t2, c.p3, c.p1), x);
+  op = fma(hp, c.k0 + ot, even + odd);
+  om = fma(hm, c.k0 - ot, even - odd);
+}
+
+// The classes of a sign group {(+a,+b), (-a,+b), (-a,-b), (+a,-b)} share a u-projection pair
+// (a u^x, b u^y) and the even part of the force polynomial; only signs differ between them.
 template <typename R, bool FORCE>
 __device__ __forceinline__ void collide_group(const Coll<R> &c, double a, double b, double vz2, R h0, R h1, R h2,
                                               R h3, R &o0, R &o1, R &o2, R &o3) {
-  const R A = c.ux * R(a), B = c.uy * R(b);
-  R even = c.s0, X = R(0), Y = R(0), XY = R(0);
-  if (FORCE) {
-    even = fma(c.sxx, R(a * a), even);
-    if (b != 0.0) even = fma(c.syy, R(b * b), even);
-    if (vz2 != 0.0) even = fma(c.szz, R(vz2), even);
-    X = c.s1x * R(a);
-    if (b != 0.0) { Y = c.s1y * R(b); XY = c.sxy2 * R(a * b); }
-  }
-  auto one = [&](R t, R force, R hq) {
-    const R acc = fma(t, fma(t, fma(t, c.p3, c.p2), c.p1), force);
-    return fma(hq, fma(c.om, t, c.k0), acc);
-  };
   if (b != 0.0) {  // diagonal group: (+a,+b), (-a,+b), (-a,-b), (+a,-b)
-    const R e0 = even + XY, e1 = even - XY;
-    o0 = one(A + B, e0 + (X + Y), h0);
-    o1 = one(B - A, e1 + (Y - X), h1);
-    o2 = one(-(A + B), e0 - (X + Y), h2);
-    o3 = one(A - B, e1 + (X - Y), h3);
-  } else {  // axis group: (+a,0), (0,+a), (-a,0), (0,-a)
-    R evx = even, evy = c.s0;
-    R Yv = R(0);
+    const R A = c.ux * R(a), B = c.uy * R(b);
+    R even = c.s0, X = R(0), Y = R(0), e0 = c.s0, e1 = c.s0;
     if (FORCE) {
-      evy = fma(c.syy, R(a * a), c.s0);
-      if (vz2 != 0.0) evy = fma(c.szz, R(vz2), evy);
-      Yv = c.s1y * R(a);
+      even = fma(c.syy, R(b * b), fma(c.sxx, R(a * a), even));
+      if (vz2 != 0.0) even = fma(c.szz, R(vz2), even);
+      X = c.s1x * R(a);
+      Y = c.s1y * R(b);
+      e0 = fma(c.sxy2, R(a * b), even);
+      e1 = fma(c.sxy2, R(-a * b), even);
     }
-    const R By = c.uy * R(a);
-    o0 = one(A, evx + X, h0);
-    o1 = one(By, evy + Yv, h1);
-    o2 = one(-A, evx - X, h2);
-    o3 = one(-By, evy - Yv, h3);
+    collide_opposite<R>(c, A + B, e0, X + Y, h0, h2, o0, o2);
+    collide_opposite<R>(c, B - A, e1, Y - X, h1, h3, o1, o3);
+  } else {  // axis group: (+a,0), (0,+a), (-a,0), (0,-a)
+    R ex = c.s0, ey = c.s0, X = R(0), Y = R(0);
+    if (FORCE) {
+      const R ez = vz2 != 0.0 ? fma(c.szz, R(vz2), c.s0) : c.s0;
+      ex = fma(c.sxx, R(a * a), ez);
+      ey = fma(c.syy, R(a * a), ez);
+      X = c.s1x * R(a);
+      Y = c.s1y * R(a);
+    }
+    collide_opposite<R>(c, c.ux * R(a), ex, X, h0, h2, o0, o2);
+    collide_opposite<R>(c, c.uy * R(a), ey, Y, h1, h3, o1, o3);
   }
 }
 

@@ -34,8 +34,8 @@ template <typename S, int VS> struct Tile {
   static constexpr int TYB = TILE_Y + 2;             // staged rows (one halo row each side)
   static constexpr int IN_BYTES = Q * TYB * TXB * (int)sizeof(S);
   static constexpr int IN_STRIDE = (IN_BYTES + 127) / 128 * 128;
-  // stirring tables of the tile (at most MAX_SROWS k_y rows): G[row][TILE_X] (R4) and
-  // EY[row][TILE_Y] (R2) after the populations; their size follows the shell at run time
+  // stirring rows of the tile (at most MAX_SROWS k_y rows): G[row][TILE_X] (R4) and EY[row][TILE_Y]
+  // (R2) after the populations; their size follows the shell at run time
   using R = typename RealOf<S>::type;
   static constexpr int MAX_SROWS = 16;
   static constexpr int G_ROW = TILE_X * 4 * (int)sizeof(R);
@@ -96,38 +96,25 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
       const Macro<R> m = cell_macro<R, VS>(h, M, p.vmax2);
       if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
       R Fx = p.body_x, Fy = p.body_y;
-      if (FORCE) {
-        if (staged) {
-          const R4<R> *Gs = reinterpret_cast<const R4<R> *>(stg + TL::IN_STRIDE) + lx;
-          const R *Er = reinterpret_cast<const R *>(stg + ey_off) + ey_index(ly);
-          // F = sum_r Re[G_r(x) EY_r(y)], two rows per iteration (staged phase rows: 16 reals)
-          R Fx2 = R(0), Fy2 = R(0);
-          int r = 0;
-#pragma unroll 1
-          for (; r + 1 < st.nrows; r += 2) {
-            const R4<R> G0 = Gs[r * TILE_X], G1 = Gs[(r + 1) * TILE_X];
-            const R2<R> E0{Er[r * 16], Er[r * 16 + 2]}, E1{Er[(r + 1) * 16], Er[(r + 1) * 16 + 2]};
-            Fx = fma(G0.x, E0.x, fma(-G0.y, E0.y, Fx));
-            Fy = fma(G0.z, E0.x, fma(-G0.w, E0.y, Fy));
-            Fx2 = fma(G1.x, E1.x, fma(-G1.y, E1.y, Fx2));
-            Fy2 = fma(G1.z, E1.x, fma(-G1.w, E1.y, Fy2));
+      if (FORCE) {  // F = sum_r Re[G_r(x) EY_r(y)], the table holding (Re, -Im)
+        R Fx2 = R(0), Fy2 = R(0);
+        for (int r = 0; r < st.nrows; ++r) {
+          R4<R> G;
+          R2<R> E;
+          if (staged) {
+            G = reinterpret_cast<const R4<R> *>(stg + TL::IN_STRIDE)[r * TILE_X + lx];
+            E = reinterpret_cast<const R2<R> *>(stg + ey_off)[r * TILE_Y + ly];
+          } else {
+            G = st.G_cur[(long long)r * g.nx + x];
+            E = st.EY[(long long)r * st.eyp + y];
           }
-          if (r < st.nrows) {
-            const R4<R> G0 = Gs[r * TILE_X];
-            const R2<R> E0{Er[r * 16], Er[r * 16 + 2]};
-            Fx = fma(G0.x, E0.x, fma(-G0.y, E0.y, Fx));
-            Fy = fma(G0.z, E0.x, fma(-G0.w, E0.y, Fy));
-          }
-          Fx += Fx2;
-          Fy += Fy2;
-        } else {
-          for (int r = 0; r < st.nrows; ++r) {
-            const R4<R> G = st.G_cur[(long long)r * g.nx + x];
-            const R2<R> E = ey_at<R>(reinterpret_cast<const R *>(st.EY) + (long long)r * 2 * st.eyp, y);
-            Fx += G.x * E.x - G.y * E.y;
-            Fy += G.z * E.x - G.w * E.y;
-          }
+          Fx = fma(G.x, E.x, Fx);
+          Fx2 = fma(G.y, E.y, Fx2);
+          Fy = fma(G.z, E.x, Fy);
+          Fy2 = fma(G.w, E.y, Fy2);
         }
+        Fx += Fx2;
+        Fy += Fy2;
       }
       if (macro_out) {  // the cell's Landau solution, force and streamed h, kept for the reverse sweep
         const long long nc = (long long)g.nx * g.ny, c = (long long)y * g.nx + x;
@@ -191,7 +178,36 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
   const bool flA = inA && !(MASK && (nbA & 16u)), flB = inB && !(MASK && (nbB & 16u));
   const bool both = flA && flB;
   T hn[Q];
-  if (flA || flB) {
+  {
+    T Fx(p.body_x), Fy(p.body_y);
+    if (FORCE) {
+      // (before the pull: four rows of loads in flight need registers that h and its moments take later)
+      // F = sum_r Re[G_r(x) EY_r(y)]: the pairs are (Re, -Im) of the table and (Re, Im) of the phase as
+      // they lie in memory, so a row costs four multiply-adds and two 16-byte loads for both cells
+      // (pairs over the two cells took a copy of each table value into both lanes and two negations)
+      T axA(0.0f), ayA(0.0f), axB(0.0f), ayB(0.0f);
+      auto add = [&](const float4 &G, const float4 &E) {
+        const T gx(G.x, G.y), gy(G.z, G.w), eA(E.x, E.y), eB(E.z, E.w);
+        axA = fma(gx, eA, axA);
+        ayA = fma(gy, eA, ayA);
+        axB = fma(gx, eB, axB);
+        ayB = fma(gy, eB, ayB);
+      };
+      if (staged) {
+        const float4 *Gs = reinterpret_cast<const float4 *>(stg + TL::IN_STRIDE) + lx;
+        const float4 *Es = reinterpret_cast<const float4 *>(stg + ey_off) + ly;
+#pragma unroll 4
+        for (int r = 0; r < st.nrows; ++r) add(Gs[r * TILE_X], Es[r * (TILE_Y / 2)]);
+      } else if (flA || flB) {
+        // (yA is even: yA and yA + 1 share 16 bytes of the phase table)
+        const float4 *Gg = reinterpret_cast<const float4 *>(st.G_cur) + x;
+        const float4 *Eg = reinterpret_cast<const float4 *>(st.EY) + yA / 2;
+        for (int r = 0; r < st.nrows; ++r) add(Gg[(long long)r * g.nx], Eg[(long long)r * (st.eyp / 2)]);
+      }
+      Fx += T(axA.v.x + axA.v.y, axB.v.x + axB.v.y);
+      Fy += T(ayA.v.x + ayA.v.y, ayB.v.x + ayB.v.y);
+    }
+    // (lanes without fluid, outside the lattice or solid, pull what the stage holds there and drop it)
     const int b0 = (2 * ly + 1) * TL::TXB + lx + TL::V;
     T h[Q];
 #pragma unroll
@@ -227,57 +243,6 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     const Mom<T> M = moments_of<T, T, VS, FORCE>(h);
     const Macro<T> m = cell_macro_pair<VS>(h, M, p.vmax2);
     if (!m.ok) atomicOr(err, (isfinite(m.eps_m1.v.x) && isfinite(m.eps_m1.v.y)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
-    T Fx(p.body_x), Fy(p.body_y);
-    if (FORCE) {
-      if (staged) {
-        const R4<float> *Gs = reinterpret_cast<const R4<float> *>(stg + TL::IN_STRIDE) + lx;
-        // (Re yA, Re yB, Im yA, Im yB) of each staged phase row: the pairs load as they are used.
-        // Two rows per iteration into two partial sums, so that both rows' loads and FMA chains
-        // are in flight at once (the synthesis is latency-bound when it runs one row at a time).
-        const R4<float> *Es = reinterpret_cast<const R4<float> *>(stg + ey_off) + ly;
-        T Fx2(0.0f), Fy2(0.0f);
-        int r = 0;
-#pragma unroll 1
-        for (; r + 1 < st.nrows; r += 2) {
-          const R4<float> G = Gs[r * TILE_X], G1 = Gs[(r + 1) * TILE_X];
-          const R4<float> E = Es[r * 4], E1 = Es[(r + 1) * 4];
-          const T Ere(E.x, E.y), Eim(E.z, E.w), Ere1(E1.x, E1.y), Eim1(E1.z, E1.w);
-          Fx = fma(T(G.x), Ere, fma(T(-G.y), Eim, Fx));
-          Fy = fma(T(G.z), Ere, fma(T(-G.w), Eim, Fy));
-          Fx2 = fma(T(G1.x), Ere1, fma(T(-G1.y), Eim1, Fx2));
-          Fy2 = fma(T(G1.z), Ere1, fma(T(-G1.w), Eim1, Fy2));
-        }
-        if (r < st.nrows) {
-          const R4<float> G = Gs[r * TILE_X];
-          const R4<float> E = Es[r * 4];
-          const T Ere(E.x, E.y), Eim(E.z, E.w);
-          Fx = fma(T(G.x), Ere, fma(T(-G.y), Eim, Fx));
-          Fy = fma(T(G.z), Ere, fma(T(-G.w), Eim, Fy));
-        }
-        Fx += Fx2;
-        Fy += Fy2;
-      } else {
-        // the same sums in the same order as the staged path (even rows into Fx, Fy, odd rows
-        // into Fx2, Fy2), so the two give the same bits
-        T Fx2(0.0f), Fy2(0.0f);
-        for (int r = 0; r < st.nrows; ++r) {
-          const R4<float> G = st.G_cur[(long long)r * g.nx + x];
-          // yA = y0 + 2 ly (even): yA and yB = yA + 1 share one entry of the phase table
-          const R4<float> E = *reinterpret_cast<const R4<float> *>(reinterpret_cast<const float *>(st.EY) +
-                                                                   (long long)r * 2 * st.eyp + ey_index(yA));
-          const T Ere(E.x, E.y), Eim(E.z, E.w);
-          if (r & 1) {
-            Fx2 = fma(T(G.x), Ere, fma(T(-G.y), Eim, Fx2));
-            Fy2 = fma(T(G.z), Ere, fma(T(-G.w), Eim, Fy2));
-          } else {
-            Fx = fma(T(G.x), Ere, fma(T(-G.y), Eim, Fx));
-            Fy = fma(T(G.z), Ere, fma(T(-G.w), Eim, Fy));
-          }
-        }
-        Fx += Fx2;
-        Fy += Fy2;
-      }
-    }
     if (macro_out) {  // the cells' Landau solutions, forces and streamed h, kept for the reverse sweep
       const long long nc = (long long)g.nx * g.ny;
       if (flA) {
@@ -392,8 +357,8 @@ __global__ void __launch_bounds__(NTHREADS / CPT)
 step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tG,
             const __grid_constant__ CUtensorMap tEY, S *__restrict__ fout,
             const Geometry<typename RealOf<S>::type> g, const Physics<typename RealOf<S>::type> p,
-            const Stir<typename RealOf<S>::type> st, int prep_bytes, int srows_in, int *__restrict__ tile_ctr,
-            unsigned seq, unsigned *__restrict__ err, typename RealOf<S>::type *__restrict__ macro_out) {
+            const Stir<typename RealOf<S>::type> st, int srows_in, int *__restrict__ tile_ctr, unsigned seq,
+            unsigned *__restrict__ err, typename RealOf<S>::type *__restrict__ macro_out) {
   using R = typename RealOf<S>::type;
   using TL = Tile<S, VS>;
   constexpr int NT = NTHREADS / CPT;
@@ -405,48 +370,57 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
   const bool staged = FORCE && srows_in > 0;
   const int srows = staged ? srows_in : 0;
   const int stage_stride = TL::stage(srows), ey_off = TL::IN_STRIDE + TL::g_bytes(srows);
-  // barriers: one per stage, then one for the mode data; then the tile of each stage
+  // barriers, one per stage; then the work item of each stage and the tile's column | row << 16
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + NST * stage_stride);
-  int *tile_of = reinterpret_cast<int *>(smem + NST * stage_stride + 32);
-  int *tile_xy = tile_of + NST;  // the stage's tile column | row << 16, set with tile_of
+  int *item_of = reinterpret_cast<int *>(smem + NST * stage_stride + 32);
+  int *tile_xy = item_of + NST;
 
   const int tid = threadIdx.x;
   const int ntx = (g.nx + TILE_X - 1) / TILE_X, nty = (g.ny + TILE_Y - 1) / TILE_Y;
   const int ntiles = ntx * nty;
   const float rcp_ntx = 1.0f / (float)ntx;
   const uint32_t stage_bytes = TL::IN_BYTES + srows * (TL::G_ROW + TL::EY_ROW);
-  // The mode data of step n+1 (coefficients, k_x, row ranges), copied on its own barrier
-  // when it fits in the `prep` area past the barriers.
-  constexpr int RB = (int)sizeof(R);
-  const int cb = mode_coef_bytes(st.nmodes, RB), kb = mode_kx_bytes(st.nmodes), rb_ = mode_rows_bytes(st.nrows);
-  const bool prep_copy = FORCE && st.nrows > 0 && cb + kb + rb_ <= prep_bytes;
-  unsigned char *prep = smem + NST * stage_stride + 64;
-  // Tiles are handed out by a counter of this launch (launches alternate between two; the
-  // first CTA clears the other one for the next launch).  Every tile is computed the same
-  // way by whichever CTA takes it, so the results do not depend on the order.
+  // Work items: the chunks of the next step's stirring table, one per warp, then the tiles.  On
+  // small lattices CTAs of their own build the table while the others compute.  (A share of the
+  // table for every CTA, in the shadow of its first copy, was longer than the copy and cost about
+  // 1 us of every step; chunks behind the tiles made the launch's end 1.5 us longer at 1024^2.)
+  const int chunks = (g.nx + stir_chunk<R>() - 1) / stir_chunk<R>();
+  const int nprep = FORCE && st.G_next ? st.nrows * chunks : 0;
+  const int tile0 = (nprep + NT / 32 - 1) / (NT / 32), nitems = tile0 + ntiles;
+  // Items are handed out by a counter of this launch (launches alternate between two; the first
+  // CTA clears the other one for the next launch).  Every item is computed the same way by whichever
+  // CTA takes it, so the results do not depend on it.  With a CTA for every item its number is
+  // the item, without the counter's round trip before the first copy (0.7 us).  (Larger grids
+  // started that way were 3 % slower at 4096^2.)
   int *ctr = tile_ctr + (seq & 1u);
+  const bool one_each = nitems <= nworkers;
 
   if (tid == 0) {
-    for (int s = 0; s <= NST; ++s) mbar_init(&bar[s], 1);
+    for (int s = 0; s < NST; ++s) mbar_init(&bar[s], 1);
     fence_mbar_init();
+    prefetch_map(&tin);
+    if (staged) {
+      prefetch_map(&tG);
+      prefetch_map(&tEY);
+    }
   }
   // A launch chained to the previous step (programmatic dependent launch) may start while
-  // that step's grid drains: the state, the stirring tables, the mode data and the tile
-  // counters it wrote are touched only after it has completed and its writes are visible.
+  // that step's grid drains: the state, the stirring tables and the counters it wrote are
+  // touched only after it has completed and its writes are visible.
   griddep_wait();
   if (tid == 0 && wid == 0) tile_ctr[(seq + 1u) & 1u] = 0;
-  __syncthreads();
-  // thread 0: stage s takes tile t (or, with t past the end, only completes its barrier:
-  // this CTA takes no further tile, and the next step's grid, when chained, may be
-  // scheduled once every CTA has come this far)
+  // thread 0: stage s takes item t (only tiles are copied; the barrier of another item, or of
+  // none, completes at once: with t past the end this CTA takes nothing further, and the next
+  // step's grid, when chained, may be scheduled once every CTA has come this far)
   auto fill = [&](int s, int t) {
     uint64_t *b = &bar[s];
-    tile_of[s] = t < ntiles ? t : -1;
-    if (t >= ntiles) {
+    item_of[s] = t < nitems ? t : -1;
+    if (t < tile0 || t >= nitems) {
       mbar_arrive(b);
-      griddep_launch_dependents();
+      if (t >= nitems) griddep_launch_dependents();
       return;
     }
+    t -= tile0;
     // row = t / ntx, column = t mod ntx: the float quotient corrected exactly (t < 2^24)
     int row = (int)((float)t * rcp_ntx), col = t - row * ntx;
     while (col < 0) { --row; col += ntx; }
@@ -461,56 +435,41 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
       tma_load_2d(st0 + ey_off, &tEY, b, 2 * y0, 0);
     }
   };
-  int pending = 0;  // thread 0: the tile the next refill will stage (fetched one tile ahead)
+  int pending = 0;  // thread 0: the item the next refill will take (fetched one ahead)
   if (tid == 0) {
-    if (prep_copy) {
-      mbar_expect_tx(&bar[NST], cb + kb + rb_);
-      bulk_load(prep, st.coef_next, cb, &bar[NST]);
-      bulk_load(prep + cb, st.mode_kx, kb, &bar[NST]);
-      bulk_load(prep + cb + kb, st.row_start, rb_, &bar[NST]);
-    }
-    for (int s = 0; s < NST; ++s) fill(s, atomicAdd(ctr, 1));
-    pending = atomicAdd(ctr, 1);
+    for (int s = 0; s < NST; ++s) fill(s, one_each ? wid + s * nworkers : atomicAdd(ctr, 1));
+    pending = one_each ? nitems : atomicAdd(ctr, 1);
   }
-
-  // While the first tiles are in flight: for the CTAs of highest index, one Philox draw
-  // of step n+2 (pure arithmetic; the multipliers are read only when they differ from 1),
-  // and this CTA's share of the table of step n+1 (entry e to CTA e mod nworkers).
-  if (FORCE && st.nrows && tid == 32) stir_draws_part<R>(st, nworkers - 1 - wid, nworkers);
-  bool alive = true;
-  if (FORCE && st.nrows) {
-    if (prep_copy) {
-      const bool ok = mbar_wait_bounded(&bar[NST], 0, WAIT_CYCLES);
-      if (__syncthreads_or(!ok)) alive = false;
-      if (alive) {
-        const R4<R> *cs = reinterpret_cast<const R4<R> *>(prep);
-        const int *ks = reinterpret_cast<const int *>(prep + cb), *rs = reinterpret_cast<const int *>(prep + cb + kb);
-        stir_table_staged<R>(st, wid, nworkers, tid, NT, g.nx, cs, ks, rs);
-      }
-    } else {
-      stir_table_part<R>(st, wid, nworkers, tid, NT, g.nx, nullptr, 0);
-    }
-  }
+  __syncthreads();
 
   // Every thread waits for the staged tile (bounded); the vote in the barrier makes the
   // whole CTA wind down together if a copy never lands.
-  if (alive) {
+  bool alive = true;
+  {
     const bool ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
   for (int k = 0; alive; ++k) {
     const int s = k % NST;
-    const int t = tile_of[s];
+    const int t = item_of[s];
     if (t < 0) break;
-    const int xy = tile_xy[s];
-    tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, fout, (xy & 0xffff) * TILE_X,
-                                        (xy >> 16) * TILE_Y, tid, g, g, p, st, staged, err,
-                                        STORE ? macro_out : static_cast<R *>(nullptr));
+    if (t >= tile0) {
+      const int xy = tile_xy[s];
+      tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, fout, (xy & 0xffff) * TILE_X,
+                                          (xy >> 16) * TILE_Y, tid, g, g, p, st, staged, err,
+                                          STORE ? macro_out : static_cast<R *>(nullptr));
+    } else if (FORCE) {
+      const int i = t * (NT / 32) + tid / 32;
+      if (i < nprep) {
+        const int r = i / chunks;
+        stir_row_chunk<R>(st.modes, st.step_next, r, i - r * chunks, g.nx, tid & 31, st.G_next + (long long)r * g.nx);
+      }
+    }
     if (NST == 1) {  // the only stage is free once every thread is done with it
       __syncthreads();
       if (tid == 0) {
         fill(0, pending);
-        pending = atomicAdd(ctr, 1);
+        if (!one_each) pending = atomicAdd(ctr, 1);
       }
     }
     // the next stage's barrier completes with its tile, or at once when it has none
@@ -522,14 +481,14 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     }
     if (NST >= 2 && tid == 0) {
       fill(s, pending);
-      pending = atomicAdd(ctr, 1);
+      if (!one_each) pending = atomicAdd(ctr, 1);
     }
   }
   if (!alive && tid == 0) {
     // a staged copy did not land in time: latch the error and wait (bounded) once more
     // for this CTA's copies still in flight before returning
     atomicOr(err, ERR_TIMEOUT);
-    for (int s2 = 0; s2 <= NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
+    for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
   }
 }
 
@@ -563,25 +522,14 @@ struct alignas(16) TileInfo {
   unsigned round_key;
 };
 
-__device__ __forceinline__ int find_member(const int *prefix, int n, int t) {
-  int lo = 0, hi = n;  // prefix[lo] <= t < prefix[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (prefix[mid] <= t) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-template <typename R> __device__ __forceinline__ Stir<R> member_stir(const MemberDesc &d, long long n) {
+template <typename R> __device__ __forceinline__ Stir<R> member_stir(const MemberDesc &d, long long n, double amp) {
   Stir<R> s;
-  s.nrows = d.nrows; s.nmodes = d.nmodes; s.eyp = d.eyp;
+  s.nrows = d.nrows; s.eyp = d.eyp;
   s.G_cur = (const R4<R> *)d.G[n & 1];
   s.EY = (const R2<R> *)d.EY;
   s.G_next = (R4<R> *)d.G[(n + 1) & 1];
-  s.coef_next = (const R4<R> *)d.coef[(n + 1) & 1];
-  s.coef_new = (R4<R> *)d.coef[n & 1];
-  s.mode_kx = d.mode_kx; s.row_start = d.row_start;
-  s.seed = d.seed; s.step_new = n + 2; s.amp = 0.0; s.mode_scale = nullptr;
+  s.step_next = n + 1;
+  s.modes = StirModes{d.mode_kx, d.row_start, d.tw, d.mode_scale, d.seed, amp};
   return s;
 }
 
@@ -672,7 +620,7 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     // staged stirring rows need only their count (the shell is shared by all members)
     Stir<R> st{};
     if (FORCE && staged) st.nrows = srows;
-    else if (FORCE) st = member_stir<R>(bt.mem[ti.m], ti.n);
+    else if (FORCE) st = member_stir<R>(bt.mem[ti.m], ti.n, amp);
     tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, (S *)ti.fout, ti.x0, ti.y0, tid, ti.dims,
                                         wts, p, st, staged, ti.err, static_cast<R *>(nullptr));
     if (NST == 1) {  // the only stage is free once every thread is done with it
@@ -699,51 +647,18 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
   }
   if (!alive) return;  // copies may still be in flight: stage 0 is not free
-  // The stirring work of the following steps, after the tiles: table entries of step n+1,
-  // then the draws of step n+2, of every member.  Each CTA takes a contiguous range of the
-  // entries (members in order, entry = row * nx + x) and builds it member by member, the
-  // member's mode data (coefficients of step n+1, k_x, row ranges) first copied into the
-  // free stage 0; consecutive threads take consecutive entries.
-  if (FORCE && srows_in >= 0 && bt.mem[0].nrows) {
-    const long long entries = bt.entry0[bt.n];
-    const long long per = (entries + nworkers - 1) / nworkers;
-    long long e0 = (long long)wid * per;
-    const long long e1 = e0 + per < entries ? e0 + per : entries;
-    while (e0 < e1) {
-      int m = 0, hi = bt.n;  // entry0[m] <= e0 < entry0[hi]
-      while (hi - m > 1) { const int mid = (m + hi) >> 1; if (bt.entry0[mid] <= e0) m = mid; else hi = mid; }
+  // The stirring tables of the next step, after the tiles: chunks of rows, members in order, one
+  // per warp.
+  if (FORCE && bt.mem[0].nrows) {
+    const int total = bt.prep0[bt.n], warps = nworkers * (NT / 32);
+    int m = 0;
+    for (int e = wid * (NT / 32) + tid / 32; e < total; e += warps) {
+      while (bt.prep0[m + 1] <= e) ++m;  // prep0[n] = total > e ends the search
       const MemberDesc &d = bt.mem[m];
-      const long long mlo = bt.entry0[m], mend = bt.entry0[m + 1] < e1 ? bt.entry0[m + 1] : e1;
-      const Stir<R> st = member_stir<R>(d, d.step0 + bstep);
-      const int need = st.nmodes * (int)(sizeof(R4<R>) + sizeof(int)) + (st.nrows + 1) * (int)sizeof(int);
-      const R4<R> *coef = st.coef_next;
-      const int *kx = st.mode_kx, *rs = st.row_start;
-      if (need <= (int)TL::IN_STRIDE) {
-        R4<R> *c2 = reinterpret_cast<R4<R> *>(smem);
-        int *k2 = reinterpret_cast<int *>(c2 + st.nmodes);
-        int *r2 = k2 + st.nmodes;
-        for (int i = tid; i < st.nmodes; i += NT) { c2[i] = coef[i]; k2[i] = kx[i]; }
-        for (int i = tid; i <= st.nrows; i += NT) r2[i] = rs[i];
-        __syncthreads();
-        coef = c2; kx = k2; rs = r2;
-      }
-      const int nx = d.nx;
-      for (long long e = e0 + tid; e < mend; e += NT) {
-        const int le = (int)(e - mlo);  // < nrows * nx
-        st.G_next[le] = stir_row_entry<R>(coef, kx, rs, le / nx, le % nx, nx);
-      }
-      __syncthreads();  // the staged mode data is replaced by the next member's
-      e0 = mend;
-    }
-    const int draws = bt.draw0[bt.n];
-    const int dper = (draws + nworkers - 1) / nworkers;
-    const int d1 = (wid + 1) * dper < draws ? (wid + 1) * dper : draws;
-    for (int e = wid * dper + tid; e < d1; e += NT) {
-      const int m = find_member(bt.draw0, bt.n, e);
-      const MemberDesc &d = bt.mem[m];
-      Stir<R> st = member_stir<R>(d, d.step0 + bstep);
-      st.amp = amp;
-      stir_draws_part<R>(st, e - bt.draw0[m], st.nmodes);
+      const Stir<R> st = member_stir<R>(d, d.step0 + bstep, amp);
+      const int chunks = (d.nx + stir_chunk<R>() - 1) / stir_chunk<R>();
+      const int i = e - bt.prep0[m], r = i / chunks;
+      stir_row_chunk<R>(st.modes, st.step_next, r, i - r * chunks, d.nx, tid & 31, st.G_next + (long long)r * d.nx);
     }
   }
 }
@@ -838,7 +753,8 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
   __shared__ int cnt[8];
   __shared__ bool last;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  DF2 accf[4];
+  const DF2 zero{F2(0.0f), F2(0.0f)};
+  DF2 accf[4] = {zero, zero, zero, zero};
   int fluid = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int tx = t % ntx, ty = t / ntx;
@@ -937,7 +853,7 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
         } else {
           float4 *cf = reinterpret_cast<float4 *>(&cols[0][0]);
           const float4 *zf = reinterpret_cast<const float4 *>(out.z);
-          DF2 d;
+          DF2 d = zero;
           if (x < g.nx)
             for (int j = ly; j < nty; j += 8) {
               const float4 v = __ldcg(&zf[(long long)j * g.nx + x]);
@@ -1103,31 +1019,15 @@ __global__ void open_ghosts_kernel(S *__restrict__ f, const Geometry<typename Re
   pl[-1] = store_h<S, R>((R)(wall_row ? 0.0 : heq));
 }
 
-// Stirring pipeline start at step n: coefficients of steps n and n+1, table of step n.
+// The stirring tables of steps n .. n + count - 1, one after the other at G (one warp per chunk of a
+// row, as the step launches build the next step's).
 template <typename R>
-__global__ void stir_draw_kernel(R4<R> *coef_a, R4<R> *coef_b, int nmodes, unsigned long long seed,
-                                 long long n, double amp, const double *__restrict__ scale) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * nmodes) return;
-  const int m = t % nmodes;
-  if (scale) amp *= scale[m];
-  // same arithmetic as the draws a step launch makes for later steps
-  if constexpr (sizeof(R) == 8) {
-    double c[4];
-    stir_draw(seed, n + t / nmodes, m, amp, c);
-    (t < nmodes ? coef_a : coef_b)[m] = R4<R>{(R)c[0], (R)c[1], (R)c[2], (R)c[3]};
-  } else {
-    float c[4];
-    stir_draw_f32(seed, n + t / nmodes, m, (float)amp, c);
-    (t < nmodes ? coef_a : coef_b)[m] = R4<R>{c[0], c[1], c[2], c[3]};
-  }
-}
-
-template <typename R>
-__global__ void stir_table_kernel(const Stir<R> st, R4<R> *G, const R4<R> *coef, int nx) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)st.nrows * nx) return;
-  G[t] = stir_row_entry<R>(st, coef, (int)(t / nx), (int)(t % nx), nx);
+__global__ void stir_tables_kernel(const StirModes sm, R4<R> *G, long long table, int nrows, int nx, long long n, int count) {
+  const int chunks = (nx + stir_chunk<R>() - 1) / stir_chunk<R>();
+  const long long i = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (i >= (long long)count * nrows * chunks) return;
+  const int j = (int)(i / (nrows * chunks)), r = (int)(i / chunks) % nrows, chunk = (int)(i % chunks);
+  stir_row_chunk<R>(sm, n + j, r, chunk, nx, threadIdx.x & 31, G + j * table + (long long)r * nx);
 }
 
 // ---------------------------------------------------------------------------
@@ -1148,13 +1048,17 @@ template <typename S> static Geometry<typename RealOf<S>::type> to_geom(const Ho
   return g;
 }
 
+static StirModes to_modes(const HostStir &h) {
+  return StirModes{h.mode_kx, h.row_start, h.tw, h.mode_scale, h.seed, h.amp};
+}
+
 template <typename R> static Stir<R> to_stir(const HostStir &h) {
   Stir<R> s;
-  s.nrows = h.nrows; s.nmodes = h.nmodes;
+  s.nrows = h.nrows;
   s.G_cur = (const R4<R> *)h.G_cur; s.EY = (const R2<R> *)h.EY; s.G_next = (R4<R> *)h.G_next;
-  s.coef_next = (const R4<R> *)h.coef_next; s.coef_new = (R4<R> *)h.coef_new;
-  s.mode_kx = h.mode_kx; s.row_start = h.row_start; s.eyp = h.eyp;
-  s.seed = h.seed; s.step_new = h.step_new; s.amp = h.amp; s.mode_scale = h.mode_scale;
+  s.eyp = h.eyp;
+  s.step_next = h.step_next;
+  s.modes = to_modes(h);
   return s;
 }
 
@@ -1173,13 +1077,7 @@ static cudaError_t launch_step_k(const CUtensorMap &tin, const CUtensorMap &tG, 
   constexpr int NT = NTHREADS / CPT;
   auto kern = step_kernel<S, VS, MASK, FORCE, CPT, NST, STORE>;
   const int srows = (FORCE && s.nrows > 0 && s.nrows <= TL::MAX_SROWS && stir_rows != 2) ? s.nrows : 0;
-  // room to stage the stirring modes of the next step (coefficients, k_x, row ranges)
-  const int prep_bytes =
-      (FORCE && s.nrows && s.nmodes <= 1024)
-          ? (mode_coef_bytes(s.nmodes, (int)sizeof(typename RealOf<S>::type)) + mode_kx_bytes(s.nmodes) +
-             mode_rows_bytes(s.nrows) + 127) / 128 * 128
-          : 0;
-  const int smem = TL::smem(NST, srows) + prep_bytes;
+  const int smem = TL::smem(NST, srows);
   static int configured_dev = -1, configured_smem = -1, max_blocks = 0, sms = 0;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1193,10 +1091,11 @@ static cudaError_t launch_step_k(const CUtensorMap &tin, const CUtensorMap &tG, 
     configured_dev = dev;
     configured_smem = smem;
   }
-  const int ntiles = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  int items = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  if (FORCE && s.G_next) items += (s.nrows * ((g.nx + stir_chunk<R>() - 1) / stir_chunk<R>()) + NT / 32 - 1) / (NT / 32);
   int workers = max_blocks * sms;
   if (grid_limit > 0 && grid_limit < workers) workers = grid_limit;
-  if (workers > ntiles) workers = ntiles;
+  if (workers > items) workers = items;
   if (workers < 1) workers = 1;
   if (chained) {
     // a step right after the previous one on the same stream: programmatic dependent
@@ -1211,10 +1110,10 @@ static cudaError_t launch_step_k(const CUtensorMap &tin, const CUtensorMap &tG, 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, tin, tG, tEY, (S *)fout, g, p, s, prep_bytes, srows, tile_ctr, seq, err,
+    return cudaLaunchKernelEx(&cfg, kern, tin, tG, tEY, (S *)fout, g, p, s, srows, tile_ctr, seq, err,
                               static_cast<R *>(macro_out));
   }
-  kern<<<workers, NT, smem, stream>>>(tin, tG, tEY, (S *)fout, g, p, s, prep_bytes, srows, tile_ctr, seq, err,
+  kern<<<workers, NT, smem, stream>>>(tin, tG, tEY, (S *)fout, g, p, s, srows, tile_ctr, seq, err,
                                       static_cast<R *>(macro_out));
   return cudaGetLastError();
 }
@@ -1409,17 +1308,13 @@ static cudaError_t launch_open_ghosts_t(int vset, void *f, const HostGeom &hg, d
 }
 
 template <typename S>
-static cudaError_t launch_stir_prime_t(const HostStir &hs, void *coef_n, void *coef_n1, void *G_n, int nx,
-                                       long long n, cudaStream_t stream) {
+static cudaError_t launch_stir_tables_t(const HostStir &hs, void *G, long long table, int nx, long long n, int count,
+                                        cudaStream_t stream) {
   using R = typename RealOf<S>::type;
-  if (hs.nmodes == 0) return cudaSuccess;
-  const Stir<R> s = to_stir<R>(hs);
-  stir_draw_kernel<R><<<(2 * hs.nmodes + 127) / 128, 128, 0, stream>>>((R4<R> *)coef_n, (R4<R> *)coef_n1,
-                                                                        hs.nmodes, hs.seed, n, hs.amp,
-                                                                        hs.mode_scale);
-  const long long entries = (long long)hs.nrows * nx;
-  stir_table_kernel<R><<<(unsigned)((entries + 255) / 256), 256, 0, stream>>>(s, (R4<R> *)G_n,
-                                                                             (const R4<R> *)coef_n, nx);
+  const int chunks = (nx + stir_chunk<R>() - 1) / stir_chunk<R>();
+  const long long warps = (long long)count * hs.nrows * chunks;
+  if (warps == 0) return cudaSuccess;
+  stir_tables_kernel<R><<<(unsigned)((warps + 3) / 4), 128, 0, stream>>>(to_modes(hs), (R4<R> *)G, table, hs.nrows, nx, n, count);
   return cudaGetLastError();
 }
 
@@ -1453,8 +1348,8 @@ static cudaError_t launch_stir_prime_t(const HostStir &hs, void *coef_n, void *c
   cudaError_t launch_open_ghosts_##SUF(int vset, void *f, const HostGeom &g, double ux_in, cudaStream_t st) { \
     return launch_open_ghosts_t<S>(vset, f, g, ux_in, st);                                               \
   }                                                                                                      \
-  cudaError_t launch_stir_prime_##SUF(const HostStir &s, void *cn, void *cn1, void *G, int nx,          \
-                                      long long n, cudaStream_t st) {                                    \
-    return launch_stir_prime_t<S>(s, cn, cn1, G, nx, n, st);                                             \
+  cudaError_t launch_stir_tables_##SUF(const HostStir &s, void *G, long long table, int nx, long long n,  \
+                                       int count, cudaStream_t st) {                                     \
+    return launch_stir_tables_t<S>(s, G, table, nx, n, count, st);                                        \
   }                                                                                                      \
   }

@@ -32,16 +32,16 @@ struct HostPhys {
   int y_off;               // lattice row of the context's row 0 (a strip of a larger lattice; else 0)
 };
 
+// A lattice's stirring: modes and phase tables (device pointers) and the tables of a step.
 struct HostStir {
   int nrows, nmodes;
   const void *G_cur, *EY;
   int eyp;
-  void *G_next;
-  const void *coef_next;
-  void *coef_new;
+  void *G_next;              // the table of step_next, built by the launch (NULL: none)
+  long long step_next;
   const int *mode_kx, *row_start;
+  const void *tw;            // [nx] exp(i 2 pi j / nx), (re, im) in the compute type
   unsigned long long seed;
-  long long step_new;
   double amp;
   const double *mode_scale;  // device [nmodes]; NULL = all 1
 };
@@ -66,10 +66,12 @@ struct alignas(128) MemberDesc {
   int nx, ny, pitch, walls;
   long long plane;
   int cur0;                // buffer holding f*_n at batch step 0
-  int nrows, nmodes, eyp;
+  int nrows, eyp;
   long long step0;         // the member's step index at batch step 0
-  const void *G[2], *EY, *coef[2];
+  void *G[2];              // stirring tables of even and odd steps
+  const void *EY, *tw;
   const int *mode_kx, *row_start;
+  const double *mode_scale;
   unsigned long long seed;
   unsigned round_key;
   unsigned *err;
@@ -77,12 +79,11 @@ struct alignas(128) MemberDesc {
   float rcp_ntx;           // 1 / ntx (tile index -> row and column with one correction)
 };
 
-// Prefix tables of a batch (device): tiles, stirring-table entries and draws per member.
+// Prefix tables of a batch (device): tiles and chunks of stirring tables per member.
 struct BatchTables {
   const MemberDesc *mem;
   const int *tile0;        // [n + 1]
-  const long long *entry0; // [n + 1]
-  const int *draw0;        // [n + 1]
+  const int *prep0;        // [n + 1]
   int *tile_ctr;           // tiles handed out so far in this launch (0 before each launch)
   int n;
 };
@@ -101,8 +102,8 @@ struct BatchTables {
   cudaError_t launch_init_##SUF(int vset, void *fout, const HostGeom &g, double eps0, const double *e,  \
                                 const double *ux, const double *uy, cudaStream_t st);                   \
   cudaError_t launch_open_ghosts_##SUF(int vset, void *f, const HostGeom &g, double ux_in, cudaStream_t st); \
-  cudaError_t launch_stir_prime_##SUF(const HostStir &s, void *cn, void *cn1, void *G, int nx,          \
-                                      long long n, cudaStream_t st);
+  cudaError_t launch_stir_tables_##SUF(const HostStir &s, void *G, long long table, int nx, long long n,  \
+                                       int count, cudaStream_t st);
 
 RLBM_DECLARE_LAUNCHERS(f64)
 RLBM_DECLARE_LAUNCHERS(f32)
@@ -123,7 +124,7 @@ struct AdjointArgs {
   double cj;               // objective weight of the state S_n
   double *acc;             // [blocks][4] FP64 accumulators
   void *zpart;             // [block rows][nrows][nx] R4 of the compute type (this step's slot)
-  const void *G, *EY;      // stirring tables of step n
+  const void *EY;          // phase rows of the stirring tables
   int nrows, eyp;
   unsigned *err;
 };
