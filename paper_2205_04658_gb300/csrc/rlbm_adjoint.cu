@@ -89,10 +89,72 @@ __device__ __forceinline__ void pull_staged_pair(const float *tile, int plane, i
   }
 }
 
+// Sums over the classes of l times monomials of v (no weights), third order with THIRD:
+// e = sum l, m = sum l v, t = sum l v v, w = sum l v v v, zz = sum l v_z^2.
+template <typename T> struct PlainSums { T e, mx, my, txx, txy, tyy, wxxx, wxxy, wxyy, wyyy, zz; };
+
+template <typename T, int VS, bool THIRD>
+__device__ __forceinline__ PlainSums<T> plain_sums(const T l[VSet<VS>::Q]) {
+  PlainSums<T> s;
+  if constexpr (VS == 3) {
+    // the four sign groups, as in moments_of: axes a = 1 (v_z = 0) and 1/sqrt 2 (v_z^2 = 1/2),
+    // diagonals a = 1/sqrt 2 (v_z = 0) and 1/sqrt 3 (v_z^2 = 1/3)
+    const T ux = l[1] + l[3], vx = l[1] - l[3], uy = l[2] + l[4], vy = l[2] - l[4];
+    const T rx = l[9] + l[11], qx = l[9] - l[11], ry = l[10] + l[12], qy = l[10] - l[12];
+    const T a02 = l[5] + l[7], b02 = l[5] - l[7], a13 = l[6] + l[8], b31 = l[8] - l[6];
+    const T A0 = a02 + a13, Axy = a02 - a13, Ax = b02 + b31, Ay = b02 - b31;
+    const T c02 = l[13] + l[15], d02 = l[13] - l[15], c13 = l[14] + l[16], d31 = l[16] - l[14];
+    const T C0 = c02 + c13, Cxy = c02 - c13, Cx = d02 + d31, Cy = d02 - d31;
+    const T r = rx + ry;
+    s.e = (l[0] + (ux + uy)) + ((r + A0) + C0);
+    s.mx = fma(T(RLBM_S3), Cx, fma(T(RLBM_S2), qx + Ax, vx));
+    s.my = fma(T(RLBM_S3), Cy, fma(T(RLBM_S2), qy + Ay, vy));
+    const T tt = fma(T(0.5), A0, T(1.0 / 3.0) * C0);
+    s.txx = fma(T(0.5), rx, ux + tt);
+    s.tyy = fma(T(0.5), ry, uy + tt);
+    s.txy = fma(T(0.5), Axy, T(1.0 / 3.0) * Cxy);
+    s.zz = fma(T(0.5), r, fma(T(1.0 / 3.0), C0, l[0]));
+    if (THIRD) {
+      constexpr double s23 = RLBM_S2 * 0.5, s33 = RLBM_S3 / 3.0;
+      s.wxyy = fma(T(s23), Ax, T(s33) * Cx);
+      s.wxxy = fma(T(s23), Ay, T(s33) * Cy);
+      s.wxxx = fma(T(s23), qx, vx + s.wxyy);
+      s.wyyy = fma(T(s23), qy, vy + s.wxxy);
+    }
+  } else {
+    using V = VSet<VS>;
+    const T z = T(0);
+    s = PlainSums<T>{z, z, z, z, z, z, z, z, z, z, z};
+#pragma unroll
+    for (int q = 0; q < V::Q; ++q) {
+      const double x = V::vx(q), y = V::vy(q);
+      s.e += l[q];
+      s.mx = fma(T(x), l[q], s.mx);
+      s.my = fma(T(y), l[q], s.my);
+      s.txx = fma(T(x * x), l[q], s.txx);
+      s.txy = fma(T(x * y), l[q], s.txy);
+      s.tyy = fma(T(y * y), l[q], s.tyy);
+      if (THIRD) {
+        s.wxxx = fma(T(x * x * x), l[q], s.wxxx);
+        s.wxxy = fma(T(x * x * y), l[q], s.wxxy);
+        s.wxyy = fma(T(x * y * y), l[q], s.wxyy);
+        s.wyyy = fma(T(y * y * y), l[q], s.wyyy);
+      }
+    }
+  }
+  return s;
+}
+
 // Reverse of one cell's collision and force (coll_coeffs / collide_all) and of its
 // objective term cj |v|^2 / 2, given the cell's post-streaming deviations h, their
 // moments M and Landau solution m, and the adjoint lam of the cell's output.  Returns
 // the adjoint of h in kap, d/d(ln omega0) in gom and the adjoint of F in gFx, gFy.
+//
+// Every class's output is h (k0 + om t) + p(t) + S(v), t = u.v: polynomials in v.  So the sums over
+// classes that the coefficients' adjoints need are combinations of the plain moments of lam (up
+// to third order) and of lam h (first order), and the adjoint of the moments comes back as one
+// even and one odd polynomial per pair of opposite classes.  (Class by class, with t and its
+// powers in each, the reverse took twice the arithmetic: 946 thread instructions per cell.)
 template <typename R, int VS, bool FORCE>
 __device__ __forceinline__ void cell_adjoint(const R h[VSet<VS>::Q], const R lam[VSet<VS>::Q], const Mom<R> &M,
                                              const Macro<R> &m, R omega0, R fpref, R Fx, R Fy, R cj,
@@ -102,54 +164,50 @@ __device__ __forceinline__ void cell_adjoint(const R h[VSet<VS>::Q], const R lam
   const R epsh = R(1) + m.eps_m1;
   const R om = VS == 3 ? omega0 * FM<R>::qroot(epsh) : omega0 * FM<R>::croot(epsh);
   const R u0 = m.u0, ux = m.ux, uy = m.uy;
-  const R u2 = ux * ux + uy * uy;
-  const R ca = R(V::CA) * epsh * u0, cb = R(V::CB) * epsh, cc = m.eps_m1 - R(V::CC) * epsh * u2;
-  const R p1 = om * (u0 * ca - cc), p2 = om * (u0 * cb - ca), p3 = -om * cb;
-  const R k0 = R(1) - om * u0;
+  const R u2 = fma(ux, ux, uy * uy);
+  const R ca = R(V::CA) * epsh * u0, cb = R(V::CB) * epsh, cc = fma(R(-V::CC) * epsh, u2, m.eps_m1);
+  const R c1 = fma(u0, ca, -cc), c2 = fma(u0, cb, -ca);
+  const R p1 = om * c1, p2 = om * c2, p3 = -om * cb;
+  const R k0 = fma(-om, u0, R(1));
 
-  // h*_q = h_q (k0 + om t_q) + p0 + p1 t + p2 t^2 + p3 t^3 + S_q,  t_q = u . v_q
-  R om_b = R(0), u0_b = R(0), ux_b = R(0), uy_b = R(0);
-  R P0 = R(0), P1 = R(0), P2 = R(0), P3 = R(0);
-  R S1x = R(0), S1y = R(0), Sxx = R(0), Sxy = R(0), Syy = R(0), Szz = R(0);
+  // moments of lam and of lam h
+  const PlainSums<R> L = plain_sums<R, VS, true>(lam);
+  R lh0, lhx, lhy;
+  {
+    R lh[Q];
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const R vx = R(V::vx(q)), vy = R(V::vy(q));
-    const R t = ux * vx + uy * vy;
-    const R lq = lam[q];
-    kap[q] = lq * (k0 + om * t);
-    const R lh = lq * h[q];
-    om_b += lh * (t - u0);
-    u0_b -= om * lh;
-    const R tb = om * lh + lq * (p1 + t * (R(2) * p2 + R(3) * p3 * t));
-    ux_b += tb * vx;
-    uy_b += tb * vy;
-    P0 += lq;
-    P1 += lq * t;
-    P2 += lq * t * t;
-    P3 += lq * t * t * t;
-    if (FORCE) {
-      S1x += lq * vx;
-      S1y += lq * vy;
-      Sxx += lq * vx * vx;
-      Sxy += lq * vx * vy;
-      Syy += lq * vy * vy;
-      Szz += lq * R(V::vz2(q));
-    }
+    for (int q = 0; q < Q; ++q) lh[q] = lam[q] * h[q];
+    const PlainSums<R> s = plain_sums<R, VS, false>(lh);
+    lh0 = s.e;
+    lhx = s.mx;
+    lhy = s.my;
   }
+  // P_j = sum lam t^j;  sum lam t v and sum lam t^2 v
+  const R tx = fma(ux, L.txx, uy * L.txy), ty = fma(ux, L.txy, uy * L.tyy);
+  const R wxx = fma(ux, L.wxxx, uy * L.wxxy), wxy = fma(ux, L.wxxy, uy * L.wxyy), wyy = fma(ux, L.wxyy, uy * L.wyyy);
+  const R wx2 = fma(ux, wxx, uy * wxy), wy2 = fma(ux, wxy, uy * wyy);
+  const R P0 = L.e, P1 = fma(ux, L.mx, uy * L.my), P2 = fma(ux, tx, uy * ty), P3 = fma(ux, wx2, uy * wy2);
+
+  // h*_q = h_q (k0 + om t_q) + p0 + p1 t + p2 t^2 + p3 t^3 + S_q with
   // p0 = om u0 cc, p1 = om (u0 ca - cc), p2 = om (u0 cb - ca), p3 = -om cb
-  om_b += P0 * u0 * cc + P1 * (u0 * ca - cc) + P2 * (u0 * cb - ca) - P3 * cb;
-  u0_b += om * (P0 * cc + P1 * ca + P2 * cb);
-  const R cc_b = om * (P0 * u0 - P1);
-  const R ca_b = om * (P1 * u0 - P2);
-  const R cb_b = om * (P2 * u0 - P3);
+  R om_b = fma(ux, lhx, fma(uy, lhy, -u0 * lh0));
+  om_b = fma(P0, u0 * cc, fma(P1, c1, fma(P2, c2, fma(-P3, cb, om_b))));
+  R u0_b = om * (fma(P0, cc, fma(P1, ca, P2 * cb)) - lh0);
+  const R p2b = R(2) * p2, p3b = R(3) * p3;
+  R ux_b = fma(om, lhx, fma(p1, L.mx, fma(p2b, tx, p3b * wx2)));
+  R uy_b = fma(om, lhy, fma(p1, L.my, fma(p2b, ty, p3b * wy2)));
+  const R cc_b = om * fma(P0, u0, -P1);
+  const R ca_b = om * fma(P1, u0, -P2);
+  const R cb_b = om * fma(P2, u0, -P3);
   // ca = CA eps^ u0, cb = CB eps^, cc = (eps^ - 1) - CC eps^ |u|^2
-  R epsh_b = ca_b * R(V::CA) * u0 + cb_b * R(V::CB) + cc_b * (R(1) - R(V::CC) * u2);
-  u0_b += ca_b * R(V::CA) * epsh;
-  ux_b -= cc_b * R(2 * V::CC) * epsh * ux;
-  uy_b -= cc_b * R(2 * V::CC) * epsh * uy;
+  R epsh_b = fma(ca_b, R(V::CA) * u0, fma(cb_b, R(V::CB), cc_b * fma(R(-V::CC), u2, R(1))));
+  u0_b = fma(ca_b, R(V::CA) * epsh, u0_b);
+  const R cce = cc_b * (R(-2 * V::CC) * epsh);
+  ux_b = fma(cce, ux, ux_b);
+  uy_b = fma(cce, uy, uy_b);
   // om = omega0 eps^(1/4) (D_p = 3) or omega0 eps^(1/3) (D_p = 2)
-  epsh_b += divide(om_b * om, R(VS == 3 ? 4 : 3) * epsh);
   gom = om_b * om;
+  epsh_b += divide(gom, R(VS == 3 ? 4 : 3) * epsh);
 
   R e_b = R(0), mx_b = R(0), my_b = R(0), txx_b = R(0), txy_b = R(0), tyy_b = R(0);
   R wxxx_b = R(0), wxxy_b = R(0), wxyy_b = R(0), wyyy_b = R(0);
@@ -157,86 +215,99 @@ __device__ __forceinline__ void cell_adjoint(const R h[VSet<VS>::Q], const R lam
   gFy = R(0);
   if (FORCE) {
     // s0 = fpref F.m / 4;  s1 = -fpref (1 + e) F / 2;  quadratic form with B and F m^T
-    const R M0 = R(1) + M.e;
-    const R f54 = R(1.25) * fpref;
-    R FM1_b = R(0.25) * fpref * P0;
-    e_b += R(-0.5) * fpref * (Fx * S1x + Fy * S1y);
-    gFx += R(-0.5) * fpref * M0 * S1x;
-    gFy += R(-0.5) * fpref * M0 * S1y;
-    R Bxx_b = f54 * Sxx, Bxy_b = R(2) * f54 * Sxy, Byy_b = f54 * Syy;
-    gFx -= R(2) * f54 * (M.mx * Sxx + M.my * Sxy);
-    gFy -= R(2) * f54 * (M.mx * Sxy + M.my * Syy);
-    mx_b -= R(2) * f54 * (Fx * Sxx + Fy * Sxy);
-    my_b -= R(2) * f54 * (Fx * Sxy + Fy * Syy);
+    const R f54 = R(1.25) * fpref, f2 = R(-2) * f54, fh = R(-0.5) * fpref;
+    const R M0 = fh * (R(1) + M.e);
     // szz = f54 Bzz, Bzz = F.m - Bxx - Byy
-    const R Bzz_b = f54 * Szz;
-    FM1_b += Bzz_b;
-    Bxx_b -= Bzz_b;
-    Byy_b -= Bzz_b;
+    const R Bzz_b = f54 * L.zz;
+    const R FM1_b = fma(R(0.25) * fpref, P0, Bzz_b);
+    const R Bxx_b = fma(f54, L.txx, -Bzz_b), Bxy_b = R(2) * f54 * L.txy, Byy_b = fma(f54, L.tyy, -Bzz_b);
+    e_b = fh * fma(Fx, L.mx, Fy * L.my);
     // Bxx = Fx wxxx + Fy wxxy, Bxy = Fx wxxy + Fy wxyy, Byy = Fx wxyy + Fy wyyy
-    gFx += Bxx_b * M.wxxx + Bxy_b * M.wxxy + Byy_b * M.wxyy;
-    gFy += Bxx_b * M.wxxy + Bxy_b * M.wxyy + Byy_b * M.wyyy;
-    wxxx_b += Bxx_b * Fx;
-    wxxy_b += Bxx_b * Fy + Bxy_b * Fx;
-    wxyy_b += Bxy_b * Fy + Byy_b * Fx;
-    wyyy_b += Byy_b * Fy;
-    gFx += FM1_b * M.mx;
-    gFy += FM1_b * M.my;
-    mx_b += FM1_b * Fx;
-    my_b += FM1_b * Fy;
+    gFx = fma(M0, L.mx, fma(f2, fma(M.mx, L.txx, M.my * L.txy),
+                            fma(Bxx_b, M.wxxx, fma(Bxy_b, M.wxxy, fma(Byy_b, M.wxyy, FM1_b * M.mx)))));
+    gFy = fma(M0, L.my, fma(f2, fma(M.mx, L.txy, M.my * L.tyy),
+                            fma(Bxx_b, M.wxxy, fma(Bxy_b, M.wxyy, fma(Byy_b, M.wyyy, FM1_b * M.my)))));
+    mx_b = fma(f2, fma(Fx, L.txx, Fy * L.txy), FM1_b * Fx);
+    my_b = fma(f2, fma(Fx, L.txy, Fy * L.tyy), FM1_b * Fy);
+    wxxx_b = Bxx_b * Fx;
+    wxxy_b = fma(Bxx_b, Fy, Bxy_b * Fx);
+    wxyy_b = fma(Bxy_b, Fy, Byy_b * Fx);
+    wyyy_b = Byy_b * Fy;
   }
 
   // objective and the macroscopic map: u0 = gamma, u = gamma v, eps^ = 1 + e - m.v
   const R vx = m.vx, vy = m.vy;
-  R vx_b = cj * vx, vy_b = cj * vy;
   const R gam = u0;
-  const R gam_b = u0_b + ux_b * vx + uy_b * vy;
-  vx_b += ux_b * gam;
-  vy_b += uy_b * gam;
-  const R g3 = gam * gam * gam;
-  vx_b += gam_b * g3 * vx;
-  vy_b += gam_b * g3 * vy;
+  const R gam_b = fma(ux_b, vx, fma(uy_b, vy, u0_b));
+  const R g3 = gam * gam * gam * gam_b + cj;
+  R vx_b = fma(ux_b, gam, fma(g3, vx, -epsh_b * M.mx));
+  R vy_b = fma(uy_b, gam, fma(g3, vy, -epsh_b * M.my));
   e_b += epsh_b;
-  mx_b -= epsh_b * vx;
-  my_b -= epsh_b * vy;
-  vx_b -= epsh_b * M.mx;
-  vy_b -= epsh_b * M.my;
+  mx_b = fma(-epsh_b, vx, mx_b);
+  my_b = fma(-epsh_b, vy, my_b);
 
   // Landau: J = dR/dv = -T + v m^T - eps^ I;  J^T w = vbar;  pbar -= (dR/dp)^T w
   const R dinv = R(1.0 / V::DP);
-  const R Txx = dinv + M.txx, Txy = M.txy, Tyy = dinv + M.tyy;
-  const R jxx = -Txx + vx * M.mx - epsh, jxy = -Txy + vx * M.my;
-  const R jyx = -Txy + vy * M.mx, jyy = -Tyy + vy * M.my - epsh;
-  const R idet = divide(R(1), jxx * jyy - jxy * jyx);
-  const R wx = (jyy * vx_b - jyx * vy_b) * idet;
-  const R wy = (jxx * vy_b - jxy * vx_b) * idet;
-  const R wv = wx * vx + wy * vy;
+  const R nxx = -(dinv + M.txx), nyy = -(dinv + M.tyy);
+  const R jxx = fma(vx, M.mx, nxx) - epsh, jxy = fma(vx, M.my, -M.txy);
+  const R jyx = fma(vy, M.mx, -M.txy), jyy = fma(vy, M.my, nyy) - epsh;
+  const R idet = divide(R(1), fma(jxx, jyy, -jxy * jyx));
+  const R wx = fma(jyy, vx_b, -jyx * vy_b) * idet;
+  const R wy = fma(jxx, vy_b, -jxy * vx_b) * idet;
+  const R wv = fma(wx, vx, wy * vy);
   e_b += wv;
-  mx_b -= wx + vx * wv;
-  my_b -= wy + vy * wv;
-  txx_b += wx * vx;
-  tyy_b += wy * vy;
-  txy_b += wx * vy + wy * vx;
+  mx_b -= fma(vx, wv, wx);
+  my_b -= fma(vy, wv, wy);
+  txx_b = wx * vx;
+  tyy_b = wy * vy;
+  txy_b = fma(wx, vy, wy * vx);
 
-  // moments: e = sum w h, m = sum w h v, t = sum w h v v, third moments sum w h v v v
+  // kap_q = lam_q (k0 + om t_q) + w_q a(v_q), a the adjoint of the moments
+  // (e = sum w h, m = sum w h v, t = sum w h v v, third moments sum w h v v v)
+  auto opposite = [&](R t, double w, R even, R odd, R lp, R lm, R &kp, R &km) {
+    const R ot = om * t;
+    kp = fma(R(w), even + odd, lp * (k0 + ot));
+    km = fma(R(w), even - odd, lm * (k0 - ot));
+  };
+  if constexpr (VS == 3) {
+    kap[0] = fma(R(V::w(0)), e_b, lam[0] * k0);
+    auto axes = [&](int q, double a) {
+      R X = R(a) * mx_b, Y = R(a) * my_b;
+      if (FORCE) {
+        X = fma(R(a * a * a), wxxx_b, X);
+        Y = fma(R(a * a * a), wyyy_b, Y);
+      }
+      opposite(R(a) * ux, V::w(q), fma(R(a * a), txx_b, e_b), X, lam[q], lam[q + 2], kap[q], kap[q + 2]);
+      opposite(R(a) * uy, V::w(q), fma(R(a * a), tyy_b, e_b), Y, lam[q + 1], lam[q + 3], kap[q + 1], kap[q + 3]);
+    };
+    auto diagonals = [&](int q, double a) {
+      const R even = fma(R(a * a), txx_b + tyy_b, e_b), A = R(a) * ux, B = R(a) * uy;
+      R X = R(a) * mx_b, Y = R(a) * my_b;
+      if (FORCE) {
+        X = fma(R(a * a * a), wxxx_b + wxyy_b, X);
+        Y = fma(R(a * a * a), wyyy_b + wxxy_b, Y);
+      }
+      opposite(A + B, V::w(q), fma(R(a * a), txy_b, even), X + Y, lam[q], lam[q + 2], kap[q], kap[q + 2]);
+      opposite(B - A, V::w(q), fma(R(-a * a), txy_b, even), Y - X, lam[q + 1], lam[q + 3], kap[q + 1], kap[q + 3]);
+    };
+    axes(1, 1.0);
+    diagonals(5, RLBM_S2);
+    axes(9, RLBM_S2);
+    diagonals(13, RLBM_S3);
+  } else {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const double qx = V::vx(q), qy = V::vy(q);
-    R a = e_b;
-    if (qx != 0.0) a += mx_b * R(qx) + txx_b * R(qx * qx);
-    if (qy != 0.0) a += my_b * R(qy) + tyy_b * R(qy * qy);
-    if (qx != 0.0 && qy != 0.0) a += txy_b * R(qx * qy);
-    if (FORCE) {
-      if (qx != 0.0) a += wxxx_b * R(qx * qx * qx);
-      if (qx != 0.0 && qy != 0.0) a += wxxy_b * R(qx * qx * qy) + wxyy_b * R(qx * qy * qy);
-      if (qy != 0.0) a += wyyy_b * R(qy * qy * qy);
+    for (int q = 0; q < Q / 2; ++q) {  // (class q + 4 is opposite to class q)
+      const double qx = V::vx(q), qy = V::vy(q);
+      const R t = fma(ux, R(qx), uy * R(qy));
+      const R even = fma(R(qx * qx), txx_b, fma(R(qx * qy), txy_b, fma(R(qy * qy), tyy_b, e_b)));
+      const R odd = fma(R(qx), mx_b, R(qy) * my_b);
+      opposite(t, V::w(q), even, odd, lam[q], lam[q + Q / 2], kap[q], kap[q + Q / 2]);
     }
-    kap[q] += R(V::w(q)) * a;
   }
 }
 
-// One adjoint step over the lattice.  Persistent CTAs of 256 threads (one cell each) walk
-// the 32 x 8 tiles (tile t to CTA t mod grid); per tile one TMA box stages kappa_{n+1} (LAM)
+// One adjoint step over the lattice (FP64).  Persistent CTAs of a thread per cell walk the
+// tiles (tile t to CTA t mod grid); per tile one TMA box stages kappa_{n+1} (LAM)
 // or, for the last state, B_{n-1}, with its one-cell halo, two stages rotating on mbarriers
 // with bounded waits, as in the forward step kernel.
 //   tB    load map of the post-collision buffer B_{n-1} of the forward run (used when LAM is
@@ -245,12 +316,12 @@ __device__ __forceinline__ void cell_adjoint(const R h[VSet<VS>::Q], const R lam
 //   kout  kappa_n; ghost cells are written like the forward's (periodic copies)
 //   cj    objective weight of S_n (1 / (N N_fluid), or 0 for the first state)
 //   acc   per-tile FP64 sums, accumulated over steps: d/d(ln omega0), F adjoint x, y, J
-//   zpart per tile row and k_y row r: sum over the tile's 8 rows of gF(x, y) EY_r(y)
+//   zpart per tile row and k_y row r: sum over the tile's rows of gF(x, y) EY_r(y)
 //   macro (LAM) the step's eps/eps0 - 1, v_x, v_y, F_x, F_y and streamed h per cell (5 + Q
 //         planes of nx * ny) as the forward step kernel computed them when it recomputed the
 //         step; without LAM, Landau matching and the force synthesis are done here
 template <typename S, int VS, bool MASK, bool FORCE, bool LAM, int NST>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(TILE_THREADS)
 adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ CUtensorMap tK,
                typename RealOf<S>::type *__restrict__ kout, const Geometry<typename RealOf<S>::type> g,
                const Physics<typename RealOf<S>::type> p, const AdjStir<typename RealOf<S>::type> st,
@@ -262,15 +333,17 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
   constexpr int Q = VSet<VS>::Q;
   constexpr int PL = TL::TYB * TL::TXB;  // elements of a staged plane
   constexpr int STAGE = TL::IN_STRIDE;  // kappa_{n+1} (LAM) or B_{n-1}
+  constexpr int TY = TL::TY, NWARP = TILE_THREADS / 32;
+  static_assert(TY == NWARP, "a warp per row of the tile");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + NST * STAGE);
-  __shared__ R2<R> sF[8][32];
-  __shared__ R2<R> sE[32][8];  // the tile's phase rows EY_r(y0 + j) of the force adjoint's projections
-  __shared__ double red[8][4];
+  __shared__ R2<R> sF[TY][32];
+  __shared__ R2<R> sE[32][TY];  // the tile's phase rows EY_r(y0 + j) of the force adjoint's projections
+  __shared__ double red[NWARP][4];
   const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5, lane = tid & 31, warp = tid >> 5;
   const int wid = blockIdx.x, nworkers = gridDim.x;
-  const int ntx = (g.nx + 31) / 32, ntiles = ntx * ((g.ny + 7) / 8);
+  const int ntx = (g.nx + 31) / 32, ntiles = ntx * ((g.ny + TY - 1) / TY);
   const int my_tiles = wid < ntiles ? (ntiles - 1 - wid) / nworkers + 1 : 0;
   const uint32_t stage_bytes = TL::IN_BYTES;
   if (tid == 0) {
@@ -282,7 +355,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
   auto issue_B = [&](int k) {
     if (LAM) return;
     const int t = wid + k * nworkers;
-    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TILE_Y;
+    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TY;
     uint64_t *b = &bar[k % NST];
     mbar_expect_tx(b, stage_bytes);
     tma_load_3d(smem + (k % NST) * STAGE, &tB, b, x0 + TL::XOFF - TL::V, y0, 0);
@@ -290,7 +363,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
   auto issue_K = [&](int k) {
     if (!LAM) return;
     const int t = wid + k * nworkers;
-    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TILE_Y;
+    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TY;
     uint64_t *b = &bar[k % NST];
     mbar_expect_tx(b, stage_bytes);
     tma_load_3d(smem + (k % NST) * STAGE, &tK, b, x0 + TL::XOFF - TL::V, y0, 0);
@@ -314,7 +387,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
     if (tid == 0 && k == my_tiles - 1) griddep_launch_dependents();
     const int t = wid + k * nworkers;
     const int tx = t % ntx, ty = t / ntx;
-    const int x = tx * TILE_X + lx, y = ty * TILE_Y + ly;
+    const int x = tx * TILE_X + lx, y = ty * TY + ly;
     const S *tileB = reinterpret_cast<const S *>(smem + (k % NST) * STAGE);  // without LAM
     const R *tileK = reinterpret_cast<const R *>(smem + (k % NST) * STAGE);  // LAM
     const int b0 = (ly + 1) * TL::TXB + lx + TL::V;
@@ -326,13 +399,13 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
     R gom = R(0), gFx = R(0), gFy = R(0), jv = R(0);
 #pragma unroll
     for (int q = 0; q < Q; ++q) kap[q] = R(0);
-    // phase rows of the projections below, loaded now (one entry per thread: k_y row tid / 8,
-    // tile row tid % 8) so that the loads complete while the cell's reverse runs
+    // phase rows of the projections below, loaded now (one entry per thread: k_y row tid / TY,
+    // tile row tid % TY) so that the loads complete while the cell's reverse runs
     R2<R> eyv{R(0), R(0)};
     const bool ey_shared = st.nrows <= 32;  // wider shells read the phase rows from global memory below
-    const bool ey_loader = FORCE && ey_shared && tid < st.nrows * 8;
-    if (ey_loader && ty * TILE_Y + (tid & 7) < g.ny)
-      eyv = ey_at<R>(reinterpret_cast<const R *>(st.EY) + (long long)(tid >> 3) * 2 * st.eyp, ty * TILE_Y + (tid & 7));
+    const bool ey_loader = FORCE && ey_shared && tid < st.nrows * TY;
+    if (ey_loader && ty * TY + (tid % TY) < g.ny)
+      eyv = ey_at<R>(reinterpret_cast<const R *>(st.EY) + (long long)(tid / TY) * 2 * st.eyp, ty * TY + (tid % TY));
     if (fluid) {
       R h[Q], lam[Q];
       // the forward's Landau solution, force and streamed h of this cell, loaded first so
@@ -392,17 +465,17 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
     // projections of the force adjoint on the k_y rows of the stirring tables
     if (FORCE && st.nrows > 0) {
       sF[ly][lx] = R2<R>{gFx, gFy};
-      if (ey_loader) sE[tid >> 3][tid & 7] = eyv;
+      if (ey_loader) sE[tid / TY][tid % TY] = eyv;
       __syncthreads();
-      const int jmax = g.ny - ty * TILE_Y;  // rows of this tile inside the lattice (>= 1)
-      for (int r = ly; r < st.nrows; r += 8) {
+      const int jmax = g.ny - ty * TY;  // rows of this tile inside the lattice (>= 1)
+      for (int r = ly; r < st.nrows; r += NWARP) {
         R4<R> z{R(0), R(0), R(0), R(0)};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < TY; ++j) {
           if (j < jmax) {
             const R2<R> E = ey_shared ? sE[r][j]
                                       : ey_at<R>(reinterpret_cast<const R *>(st.EY) + (long long)r * 2 * st.eyp,
-                                                 ty * TILE_Y + j);
+                                                 ty * TY + j);
             const R2<R> F = sF[j][lx];
             z.x += F.x * E.x;
             z.y += F.x * E.y;
@@ -424,7 +497,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
     __syncthreads();
     if (tid < 4) {
       double sum = 0.0;
-      for (int w8 = 0; w8 < 8; ++w8) sum += red[w8][tid];
+      for (int wp = 0; wp < NWARP; ++wp) sum += red[wp][tid];
       // one update of this slot per launch, launches in stream order: the same sum as a
       // plain read-add-write, without waiting for the read
       atomicAdd(&acc[(long long)t * 4 + tid], sum);
@@ -452,8 +525,11 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
 // the 32 x 8 tile, the pulls, moments, the cell's reverse and the objective on packed FP32
 // pairs, as the forward step kernel computes its FP32 paths.  Tile walk, staging, chaining,
 // stores, row projections and tile sums as in adjoint_kernel.
+// One stage per CTA and four CTAs per SM (128 registers): the other CTAs' tiles hide a tile's copy,
+// and the 512^2 lattice takes 2 rounds instead of 3 (gradient of 200 steps 8.27 ms; three CTAs of
+// two stages 8.41, of one 8.56, five CTAs 9.00).
 template <int VS, bool MASK, bool FORCE, bool LAM, int NST>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 4)
 adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ CUtensorMap tK,
                     float *__restrict__ kout, const Geometry<float> g, const Physics<float> p,
                     const AdjStir<float> st, const float cj, double *__restrict__ acc,
@@ -484,7 +560,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   auto issue_B = [&](int k) {
     if (LAM) return;
     const int t = wid + k * nworkers;
-    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TILE_Y;
+    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TL::TY;
     uint64_t *b = &bar[k % NST];
     mbar_expect_tx(b, stage_bytes);
     tma_load_3d(smem + (k % NST) * STAGE, &tB, b, x0 + TL::XOFF - TL::V, y0, 0);
@@ -492,7 +568,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   auto issue_K = [&](int k) {
     if (!LAM) return;
     const int t = wid + k * nworkers;
-    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TILE_Y;
+    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TL::TY;
     uint64_t *b = &bar[k % NST];
     mbar_expect_tx(b, stage_bytes);
     tma_load_3d(smem + (k % NST) * STAGE, &tK, b, x0 + TL::XOFF - TL::V, y0, 0);
@@ -514,7 +590,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
     if (tid == 0 && k == my_tiles - 1) griddep_launch_dependents();
     const int t = wid + k * nworkers;
     const int tx = t % ntx, ty = t / ntx;
-    const int x = tx * TILE_X + lx, yA = ty * TILE_Y + 2 * ly, yB = yA + 1;
+    const int x = tx * TILE_X + lx, yA = ty * TL::TY + 2 * ly, yB = yA + 1;
     const float *tileB = reinterpret_cast<const float *>(smem + (k % NST) * STAGE);  // without LAM
     const float *tileK = reinterpret_cast<const float *>(smem + (k % NST) * STAGE);  // LAM
     const int b0 = (2 * ly + 1) * TL::TXB + lx + TL::V;
@@ -528,7 +604,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
     // phase rows of the projections below, loaded now (entries tid and tid + 128: k_y row e / 8,
     // tile row e % 8) so that the loads complete while the cells' reverse runs
     R2<float> ey0{0.0f, 0.0f}, ey1{0.0f, 0.0f};
-    const int yj = ty * TILE_Y + (tid & 7);
+    const int yj = ty * TL::TY + (tid & 7);
     if (tid < ney && yj < g.ny)
       ey0 = ey_at<float>(reinterpret_cast<const float *>(st.EY) + (long long)(tid >> 3) * 2 * st.eyp, yj);
     if (tid + NT < ney && yj < g.ny)
@@ -650,7 +726,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
     // projections of the force adjoint on the k_y rows of the stirring tables: the column's
     // 8 values of gF loaded once, (x, y) and (z, w) of each row's sum on packed pairs
     if (proj) {
-      const int jmax = g.ny - ty * TILE_Y;  // rows of this tile inside the lattice (>= 1)
+      const int jmax = g.ny - ty * TL::TY;  // rows of this tile inside the lattice (>= 1)
       F2 Fx8[8], Fy8[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -694,7 +770,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const R2<float> E = j < jmax ? ey_at<float>(reinterpret_cast<const float *>(st.EY) +
-                                                            (long long)r * 2 * st.eyp, ty * TILE_Y + j)
+                                                            (long long)r * 2 * st.eyp, ty * TL::TY + j)
                                          : R2<float>{0.0f, 0.0f};
             const F2 e(E.x, E.y);
             zxy = fma(Fx8[j], e, zxy);
@@ -764,22 +840,43 @@ mode_grad_kernel(const R4<R> *__restrict__ zsum, int nrows, const R2<R> *__restr
     const int c1 = min(m1, c0 + MG_MAX_ROW_MODES);
     for (int mo = c0; mo < c1; ++mo) {
       const int kx = mode_kx[mo];
+      // sum of conj-free products e z over the columns; the residues k_x x mod nx step by a constant
       R a[4] = {R(0), R(0), R(0), R(0)};
+      int t = (int)(((long long)kx * (int)threadIdx.x) % nx), d = (kx * MG_THREADS) % nx;
+      if (t < 0) t += nx;
+      if (d < 0) d += nx;
       for (int x = threadIdx.x; x < nx; x += MG_THREADS) {
-        int t = (kx * x) % nx;
-        if (t < 0) t += nx;
         const R2<R> e = tw[t];
         const R4<R> z = zs[x];
-        a[0] += e.x * z.x - e.y * z.y;
-        a[1] += e.x * z.y + e.y * z.x;
-        a[2] += e.x * z.z - e.y * z.w;
-        a[3] += e.x * z.w + e.y * z.z;
+        a[0] = fma(e.x, z.x, fma(-e.y, z.y, a[0]));
+        a[1] = fma(e.x, z.y, fma(e.y, z.x, a[1]));
+        a[2] = fma(e.x, z.z, fma(-e.y, z.w, a[2]));
+        a[3] = fma(e.x, z.w, fma(e.y, z.z, a[3]));
+        t += d;
+        if (t >= nx) t -= nx;
       }
+      if constexpr (sizeof(R) == 8) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        double v = (double)a[k];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) red[mo - c0][warp][k] = v;
+        for (int k = 0; k < 4; ++k) {
+          double v = a[k];
+          for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+          if (lane == 0) red[mo - c0][warp][k] = v;
+        }
+      } else {
+        // the warp's sums in pairs of FP32 numbers (an FP64 addition occupies the SM's FP64 units for 64
+        // cycles; 20 of them per mode were most of this kernel)
+        DF2 p{F2(a[0], a[1]), F2(0.0f)}, q{F2(a[2], a[3]), F2(0.0f)};
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          p = df_add(p, df_shfl_xor(p, off));
+          q = df_add(q, df_shfl_xor(q, off));
+        }
+        if (lane == 0) {
+          red[mo - c0][warp][0] = (double)p.h.v.x + (double)p.l.v.x;
+          red[mo - c0][warp][1] = (double)p.h.v.y + (double)p.l.v.y;
+          red[mo - c0][warp][2] = (double)q.h.v.x + (double)q.l.v.x;
+          red[mo - c0][warp][3] = (double)q.h.v.y + (double)q.l.v.y;
+        }
       }
     }
     __syncthreads();
@@ -836,10 +933,8 @@ static cudaError_t launch_adjoint_k(const AdjointArgs &a, const Geometry<typenam
   // only a launch with kappa_{n+1} directly follows another reverse step
   using R = typename RealOf<S>::type;
   using TL = Tile<S, VS>;
-  constexpr int NST = 2;
-  // FP32: two cells per thread on packed pairs (128 threads); FP64: one cell per thread
-  constexpr bool PAIR = sizeof(S) == 4;
-  constexpr int NT = PAIR ? 128 : 256;
+  // FP32: two cells per thread on packed pairs; FP64: one cell per thread
+  constexpr int NST = sizeof(S) == 4 ? 1 : 2, NT = TILE_THREADS;
   auto kern = pick_adjoint_kernel<S, VS, MASK, FORCE, LAM, NST>();
   const int smem = NST * TL::IN_STRIDE + 64 + 128;
   static int configured_dev = -1, max_blocks = 0, sms = 0;
@@ -854,7 +949,7 @@ static cudaError_t launch_adjoint_k(const AdjointArgs &a, const Geometry<typenam
     if (e != cudaSuccess) return e;
     configured_dev = dev;
   }
-  const int ntiles = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  const int ntiles = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TL::TY - 1) / TL::TY);
   int workers = max_blocks * sms;
   if (workers > ntiles) workers = ntiles;
   if (workers < 1) workers = 1;

@@ -28,6 +28,9 @@ thread_local std::string g_thread_error;
 constexpr size_t kAlign = 256;
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
+// rows of a tile
+int tile_rows(int prec) { return prec == RLBM_F64 ? TileRows<double>::value : TileRows<float>::value; }
+
 int num_classes(int vset) { return vset == 3 ? VSet<3>::Q : VSet<2>::Q; }
 size_t store_bytes(int prec) { return prec == RLBM_F64 ? 8 : prec == RLBM_F32 ? 4 : 2; }
 size_t real_bytes(int prec) { return prec == RLBM_F64 ? 8 : 4; }
@@ -274,7 +277,7 @@ cudaError_t dispatch_open_ghosts(rlbm_ctx *c, int b) {
 }
 
 // Tensor maps of one population buffer: the whole ghost-padded planes, {pitch, ny + 2,
-// Q}, read in boxes of {32 + 2 V, 10, Q} (a 32 x 8 tile with its halo, V = 16 bytes of
+// Q}, read in boxes of {32 + 2 V, rows + 2, Q} (a tile with its halo, V = 16 bytes of
 // elements).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -305,7 +308,7 @@ std::string encode_state_map(const rlbm_ctx *c, void *base, CUtensorMap *out) {
   const cuuint64_t strides[2] = {(cuuint64_t)c->L.pitch * eb, (cuuint64_t)c->L.plane * eb};
   const cuuint32_t estr[3] = {1, 1, 1};
   const cuuint64_t din[3] = {(cuuint64_t)c->L.pitch, (cuuint64_t)c->cfg.ny + 2, (cuuint64_t)c->L.Q};
-  const cuuint32_t bin[3] = {32 + 2 * V, 10, (cuuint32_t)c->L.Q};
+  const cuuint32_t bin[3] = {32 + 2 * V, (cuuint32_t)tile_rows(prec) + 2, (cuuint32_t)c->L.Q};
   CUresult r = encode(out, dt, 3, base, din, strides, bin, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return "cuTensorMapEncodeTiled (load map) failed with " + std::to_string((int)r);
@@ -338,7 +341,7 @@ std::string make_tensor_maps(rlbm_ctx *c) {
     if (!m.empty()) return m;
   }
   // stirring tables of a tile: G rows {4 nx} (one R4 per column) in boxes {4 * 32, nrows},
-  // EY rows {2 eyp} in boxes {2 * 8, nrows}; staged only for shells of <= 16 k_y rows
+  // EY rows {2 eyp} in boxes {2 * rows, nrows}; staged only for shells of <= 16 k_y rows
   std::memset(c->tmap_G, 0, sizeof(c->tmap_G));
   std::memset(&c->tmap_EY, 0, sizeof(c->tmap_EY));
   if (c->L.nrows > 0 && c->L.nrows <= 16) {
@@ -351,7 +354,7 @@ std::string make_tensor_maps(rlbm_ctx *c) {
     }
     const cuuint64_t de[2] = {(cuuint64_t)2 * c->L.eyp, (cuuint64_t)c->L.nrows};
     const cuuint64_t se[1] = {(cuuint64_t)2 * c->L.eyp * rb};
-    const cuuint32_t be[2] = {2 * 8, (cuuint32_t)c->L.nrows};
+    const cuuint32_t be[2] = {2 * (cuuint32_t)tile_rows(prec), (cuuint32_t)c->L.nrows};
     CUresult r = encode(&c->tmap_EY, rt, 2, c->ws + c->L.EY, de, se, be, e2, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return "cuTensorMapEncodeTiled (phase table map) failed with " + std::to_string((int)r);
@@ -1134,7 +1137,7 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
     d.seed = c->cfg.seed; d.round_key = c->phys.round_key; d.err = c->at<unsigned>(c->L.err);
     d.ntx = (c->cfg.nx + 31) / 32;
     d.rcp_ntx = 1.0f / (float)d.ntx;
-    const int nt = d.ntx * ((c->cfg.ny + 7) / 8);
+    const int ty = tile_rows(c->cfg.precision), nt = d.ntx * ((c->cfg.ny + ty - 1) / ty);
     tile0[i + 1] = tile0[i] + nt;
     const int chunk = c->cfg.precision == RLBM_F64 ? stir_chunk<double>() : stir_chunk<float>();
     prep0[i + 1] = prep0[i] + c->L.nrows * ((c->cfg.nx + chunk - 1) / chunk);
@@ -1299,7 +1302,7 @@ GradLayout grad_layout(const rlbm_ctx *c, int64_t N, int32_t segment) {
   const size_t rb = real_bytes(prec);
   G.state_bytes = align_up(store_bytes(prec) * c->L.Q * c->L.plane);
   G.kap_bytes = align_up(rb * c->L.Q * c->L.plane);
-  G.nby = (c->cfg.ny + 7) / 8;
+  G.nby = (c->cfg.ny + tile_rows(prec) - 1) / tile_rows(prec);
   G.nblocks = (long long)((c->cfg.nx + 31) / 32) * G.nby;
   G.table_bytes = align_up(4 * rb * (size_t)c->L.nrows * c->cfg.nx);
   G.zpart_bytes = 4 * rb * (size_t)G.nby * c->L.nrows * c->cfg.nx;
@@ -1427,15 +1430,15 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
       (e = cudaMemsetAsync(w + G.scratch, 0, G.state_bytes, c->stream)) != cudaSuccess)
     return c->cuda_fail(e, "cudaMemsetAsync");
 
-  // forward: B_{-1} (the context's buffer) to checkpoint 0; B_{k seg - 1} into checkpoint k.
-  // With one segment the recomputation of that segment (below) is the forward itself: it
-  // starts from checkpoint 0 and keeps every state, so no separate forward pass runs.
+  // forward: B_{-1} (the context's buffer) to checkpoint 0; B_{k seg - 1} into checkpoint k.  The last
+  // segment's steps keep their values at once (`recompute` below runs them from its checkpoint),
+  // so those are not run twice, and with one segment no separate forward pass runs.
   const int64_t s0 = c->step;
-  const bool one_pass = G.K == 1;
+  const int64_t plain = (int64_t)(G.K - 1) * G.seg;  // steps before the last segment
   if ((e = cudaMemcpyAsync(ckpt(0), c->ws + c->L.pop[c->cur], G.state_bytes, cudaMemcpyDeviceToDevice, c->stream)) != cudaSuccess)
     return c->cuda_fail(e, "copy of the start state");
   int where = -1;  // B_{n-1}: -1 - k = checkpoint k, 0 / 1 = context buffer
-  for (int64_t n = 0; !one_pass && n < nsteps; ++n) {
+  for (int64_t n = 0; n < plain; ++n) {
     const CUtensorMap *ti = where < 0 ? &mck[-1 - where] : &c->tmap_in[where];
     void *fout;
     int next;
@@ -1451,11 +1454,6 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
       return c->cuda_fail(e, "step kernel launch");
     where = next;
   }
-  if (!one_pass) {
-    c->cur = where;  // the last step writes a context buffer
-    c->step = s0 + nsteps;
-  }
-
   // reverse sweep
   if ((e = launch_adj_twiddles(reinterpret_cast<double2 *>(w + G.tw), reinterpret_cast<float2 *>(w + G.twf), c->cfg.nx,
                                c->stream)) != cudaSuccess)
@@ -1511,11 +1509,11 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
     }
     return cudaSuccess;
   };
-  if (one_pass) {
-    if ((e = recompute(0, 0, nsteps)) != cudaSuccess) {
-      if (!map_error.empty()) return c->fail(RLBM_E_CUDA, map_error);
-      return c->cuda_fail(e, "step kernel launch (forward)");
-    }
+  if ((e = recompute(G.K - 1, plain, nsteps)) != cudaSuccess) {
+    if (!map_error.empty()) return c->fail(RLBM_E_CUDA, map_error);
+    return c->cuda_fail(e, "step kernel launch (last segment)");
+  }
+  {
     // the state after the run, B_{N-1}, into a context buffer, as rlbm_step(N) would leave it
     const int dst = c->cur ^ 1;
     if ((e = cudaMemcpyAsync(c->ws + c->L.pop[dst], w + G.scratch, G.state_bytes, cudaMemcpyDeviceToDevice, c->stream)) != cudaSuccess)
@@ -1536,7 +1534,7 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
   if ((e = dispatch_adjoint(c, a)) != cudaSuccess) return c->cuda_fail(e, "adjoint kernel launch");
   for (int k = G.K - 1; k >= 0; --k) {
     const int64_t lo = (int64_t)k * G.seg, hi = std::min<int64_t>(lo + G.seg, nsteps);
-    if (!one_pass && (e = recompute(k, lo, hi)) != cudaSuccess) {
+    if (k < G.K - 1 && (e = recompute(k, lo, hi)) != cudaSuccess) {
       if (!map_error.empty()) return c->fail(RLBM_E_CUDA, map_error);
       return c->cuda_fail(e, "step kernel launch (recompute)");
     }

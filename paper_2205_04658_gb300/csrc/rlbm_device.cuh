@@ -143,6 +143,17 @@ template <typename S> struct PadLayout {
 };
 
 // ---------------------------------------------------------------------------
+// Tiles: 32 columns by 8 rows, two rows per thread, for the FP32-compute paths; by 4 rows, one per
+// thread, for FP64.  Either way a CTA has four warps, one on each quarter of the SM: a warp's
+// FP64 instruction takes 64 cycles whatever its lanes, and eight warps of an SM share the FP64
+// units (74 ns per instruction instead of 37), so FP64 tiles of 8 rows left half the rate unused
+// on lattices of fewer tiles than SMs.
+// ---------------------------------------------------------------------------
+template <typename S> struct TileRows { static constexpr int value = 8; };
+template <> struct TileRows<double> { static constexpr int value = 4; };
+constexpr int TILE_X = 32, TILE_THREADS = 128;
+
+// ---------------------------------------------------------------------------
 // Parameters
 // ---------------------------------------------------------------------------
 template <typename R> struct alignas(16) R4 { R x, y, z, w; };

@@ -12,8 +12,6 @@
 
 namespace rlbm {
 
-constexpr int TILE_X = 32, TILE_Y = 8, NTHREADS = TILE_X * TILE_Y;
-
 // The ghost column a cell at x also writes (INT_MIN: none): with x periodic, its image
 // beyond the opposite edge; in an open channel, the last column repeats itself beyond the
 // outflow edge and nothing is written into the inflow column.
@@ -27,19 +25,19 @@ __device__ __forceinline__ int ghost_row(int y, int ny, int walls) {
 constexpr long long WAIT_CYCLES = 4000000000ll;  // ~2 s at 2 GHz: bounded TMA waits
 
 template <typename S, int VS> struct Tile {
-  static constexpr int Q = VSet<VS>::Q;
+  static constexpr int Q = VSet<VS>::Q, TY = TileRows<S>::value;
   static constexpr int V = PadLayout<S>::V;
   static constexpr int XOFF = PadLayout<S>::XOFF;
   static constexpr int TXB = TILE_X + 2 * V;         // staged columns (16-byte granules on both sides)
-  static constexpr int TYB = TILE_Y + 2;             // staged rows (one halo row each side)
+  static constexpr int TYB = TY + 2;             // staged rows (one halo row each side)
   static constexpr int IN_BYTES = Q * TYB * TXB * (int)sizeof(S);
   static constexpr int IN_STRIDE = (IN_BYTES + 127) / 128 * 128;
-  // stirring rows of the tile (at most MAX_SROWS k_y rows): G[row][TILE_X] (R4) and EY[row][TILE_Y]
+  // stirring rows of the tile (at most MAX_SROWS k_y rows): G[row][TILE_X] (R4) and EY[row][TY]
   // (R2) after the populations; their size follows the shell at run time
   using R = typename RealOf<S>::type;
   static constexpr int MAX_SROWS = 16;
   static constexpr int G_ROW = TILE_X * 4 * (int)sizeof(R);
-  static constexpr int EY_ROW = TILE_Y * 2 * (int)sizeof(R);
+  static constexpr int EY_ROW = TY * 2 * (int)sizeof(R);
   static_assert(IN_STRIDE % 128 == 0 && G_ROW % 128 == 0, "TMA shared-memory destinations are 128-byte aligned");
   __host__ __device__ static constexpr int g_bytes(int rows) { return (rows * G_ROW + 127) / 128 * 128; }
   __host__ __device__ static constexpr int ey_bytes(int rows) { return (rows * EY_ROW + 127) / 128 * 128; }
@@ -47,7 +45,7 @@ template <typename S, int VS> struct Tile {
   __host__ __device__ static constexpr int smem(int nst, int rows) { return nst * stage(rows) + 64 + 128; }
 };
 
-// One cell per thread (256 threads): the FP64 path.
+// One cell per thread: the FP64 path.
 template <typename S, int VS, bool MASK, bool FORCE, int CPT, class G, class W>
 __device__ __forceinline__ typename std::enable_if<CPT == 1>::type
 tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int tid, const G &g, const W &wts,
@@ -61,6 +59,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     const int x = x0 + lx, y = y0 + ly;
     const S *tile = reinterpret_cast<const S *>(stg);
     const bool inside = x < g.nx && y < g.ny;
+    const bool border = x0 == 0 || y0 == 0 || x0 + TILE_X >= g.nx || y0 + TL::TY >= g.ny;  // the tile's
     unsigned nb = 0;
     if (MASK && g.nbmask && inside) nb = g.nbmask[(long long)y * g.nx + x];
     const bool fluid = inside && !(MASK && (nb & 16u));
@@ -103,7 +102,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
           R2<R> E;
           if (staged) {
             G = reinterpret_cast<const R4<R> *>(stg + TL::IN_STRIDE)[r * TILE_X + lx];
-            E = reinterpret_cast<const R2<R> *>(stg + ey_off)[r * TILE_Y + ly];
+            E = reinterpret_cast<const R2<R> *>(stg + ey_off)[r * TL::TY + ly];
           } else {
             G = st.G_cur[(long long)r * g.nx + x];
             E = st.EY[(long long)r * st.eyp + y];
@@ -138,7 +137,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
       for (int q = 0; q < Q; ++q) o[q * g.plane] = store_h<S, R>(hn[q]);
     }
     // ghost copies of the periodic neighbours (boundary cells only)
-    if (inside) {
+    if (inside && border) {
       const int gxv = ghost_col(x, g.nx, g.walls);
       const int gyv = ghost_row(y, g.ny, g.walls);
       if (gxv != INT_MIN || gyv != INT_MIN) {
@@ -153,7 +152,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     }
 }
 
-// Two cells per thread (128 threads): cells (x, y) and (x, y + 1) of the 32 x 8 tile (y
+// Two cells per thread: cells (x, y) and (x, y + 1) of the 32 x 8 tile (y
 // even), all per-cell arithmetic on packed FP32 pairs.  The FP32, FP16 and BF16 paths.  The
 // two cells are adjacent rows, so the classes that move in y pull one of their rows for
 // both (each such value is read from shared memory and converted once).
@@ -170,6 +169,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
   const int x = x0 + lx, yA = y0 + 2 * ly, yB = yA + 1;
   const S *tile = reinterpret_cast<const S *>(stg);
   const bool inA = x < g.nx && yA < g.ny, inB = x < g.nx && yB < g.ny;
+  const bool border = x0 == 0 || y0 == 0 || x0 + TILE_X >= g.nx || y0 + TL::TY >= g.ny;  // the tile's
   unsigned nbA = 0, nbB = 0;
   if (MASK && g.nbmask) {
     if (inA) nbA = g.nbmask[(long long)yA * g.nx + x];
@@ -197,7 +197,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
         const float4 *Gs = reinterpret_cast<const float4 *>(stg + TL::IN_STRIDE) + lx;
         const float4 *Es = reinterpret_cast<const float4 *>(stg + ey_off) + ly;
 #pragma unroll 4
-        for (int r = 0; r < st.nrows; ++r) add(Gs[r * TILE_X], Es[r * (TILE_Y / 2)]);
+        for (int r = 0; r < st.nrows; ++r) add(Gs[r * TILE_X], Es[r * (TL::TY / 2)]);
       } else if (flA || flB) {
         // (yA is even: yA and yA + 1 share 16 bytes of the phase table)
         const float4 *Gg = reinterpret_cast<const float4 *>(st.G_cur) + x;
@@ -323,6 +323,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     }
   }
   // ghost copies of the periodic neighbours (boundary cells only)
+  if (!border) return;
 #pragma unroll
   for (int lane = 0; lane < 2; ++lane) {
     const int y = lane ? yB : yA;
@@ -342,8 +343,8 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
 
 // ---------------------------------------------------------------------------
 // The fused step (procedure items 2-5 of Sec. "The Standard/Classical LBM", with the
-// driving term of Sec. "The Driving Term").  Persistent CTAs walk the 32 x 8 tiles of
-// the lattice.  Per tile, one 3-D TMA copy stages all Q planes of the tile plus a
+// driving term of Sec. "The Driving Term").  Persistent CTAs walk the tiles of the
+// lattice.  Per tile, one 3-D TMA copy stages all Q planes of the tile plus a
 // one-cell halo (ghost rows/columns carry the periodic wrap) into shared memory, with
 // the tile's stirring rows; NST stages rotate on mbarriers (NST = 2: the next tile is
 // in flight while this one is computed; NST = 1: more CTAs per SM hide the copy
@@ -353,7 +354,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
 // the ghost copies of boundary cells.
 // ---------------------------------------------------------------------------
 template <typename S, int VS, bool MASK, bool FORCE, int CPT, int NST, bool STORE>
-__global__ void __launch_bounds__(NTHREADS / CPT)
+__global__ void __launch_bounds__(TILE_THREADS)
 step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tG,
             const __grid_constant__ CUtensorMap tEY, S *__restrict__ fout,
             const Geometry<typename RealOf<S>::type> g, const Physics<typename RealOf<S>::type> p,
@@ -361,7 +362,7 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
             unsigned *__restrict__ err, typename RealOf<S>::type *__restrict__ macro_out) {
   using R = typename RealOf<S>::type;
   using TL = Tile<S, VS>;
-  constexpr int NT = NTHREADS / CPT;
+  constexpr int NT = TILE_THREADS;
   const int wid = blockIdx.x, nworkers = gridDim.x;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // every TMA box lands on a 128-byte boundary of this aligned base
@@ -376,7 +377,7 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
   int *tile_xy = item_of + NST;
 
   const int tid = threadIdx.x;
-  const int ntx = (g.nx + TILE_X - 1) / TILE_X, nty = (g.ny + TILE_Y - 1) / TILE_Y;
+  const int ntx = (g.nx + TILE_X - 1) / TILE_X, nty = (g.ny + TL::TY - 1) / TL::TY;
   const int ntiles = ntx * nty;
   const float rcp_ntx = 1.0f / (float)ntx;
   const uint32_t stage_bytes = TL::IN_BYTES + srows * (TL::G_ROW + TL::EY_ROW);
@@ -426,7 +427,7 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     while (col < 0) { --row; col += ntx; }
     while (col >= ntx) { ++row; col -= ntx; }
     tile_xy[s] = col | (row << 16);
-    const int x0 = col * TILE_X, y0 = row * TILE_Y;
+    const int x0 = col * TILE_X, y0 = row * TL::TY;
     unsigned char *st0 = smem + s * stage_stride;
     mbar_expect_tx(b, stage_bytes);
     tma_load_3d(st0, &tin, b, x0 + TL::XOFF - TL::V, y0, 0);
@@ -456,7 +457,7 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     if (t >= tile0) {
       const int xy = tile_xy[s];
       tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, fout, (xy & 0xffff) * TILE_X,
-                                          (xy >> 16) * TILE_Y, tid, g, g, p, st, staged, err,
+                                          (xy >> 16) * TL::TY, tid, g, g, p, st, staged, err,
                                           STORE ? macro_out : static_cast<R *>(nullptr));
     } else if (FORCE) {
       const int i = t * (NT / 32) + tid / 32;
@@ -534,13 +535,13 @@ template <typename R> __device__ __forceinline__ Stir<R> member_stir(const Membe
 }
 
 template <typename S, int VS, bool MASK, bool FORCE, int CPT, int NST>
-__global__ void __launch_bounds__(NTHREADS / CPT, CPT == 2 ? 4 : 1)  // two-cell paths: 4 CTAs/SM
+__global__ void __launch_bounds__(TILE_THREADS, CPT == 2 ? 4 : 1)  // two-cell paths: 4 CTAs/SM
 batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type> wts,
                   const Physics<typename RealOf<S>::type> p0, const int srows_in, const double amp,
                   const long long *__restrict__ bstep_ptr) {
   using R = typename RealOf<S>::type;
   using TL = Tile<S, VS>;
-  constexpr int NT = NTHREADS / CPT;
+  constexpr int NT = TILE_THREADS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
   const bool staged = FORCE && srows_in > 0;
@@ -581,7 +582,7 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     int row = (int)((float)lt * d.rcp_ntx), col = lt - row * d.ntx;
     while (col < 0) { --row; col += d.ntx; }
     while (col >= d.ntx) { ++row; col -= d.ntx; }
-    const int x0 = col * TILE_X, y0 = row * TILE_Y;
+    const int x0 = col * TILE_X, y0 = row * TL::TY;
     const long long n = d.step0 + bstep;
     const int cur = (d.cur0 + (int)(bstep & 1)) & 1;
     ti.dims = BatchDims{d.nx, d.ny, d.pitch, d.walls, d.plane, d.nbmask};
@@ -1074,7 +1075,7 @@ static cudaError_t launch_step_k(const CUtensorMap &tin, const CUtensorMap &tG, 
   using TL = Tile<S, VS>;
   using R = typename RealOf<S>::type;
   constexpr int CPT = sizeof(S) == 8 ? 1 : 2;
-  constexpr int NT = NTHREADS / CPT;
+  constexpr int NT = TILE_THREADS;
   auto kern = step_kernel<S, VS, MASK, FORCE, CPT, NST, STORE>;
   const int srows = (FORCE && s.nrows > 0 && s.nrows <= TL::MAX_SROWS && stir_rows != 2) ? s.nrows : 0;
   const int smem = TL::smem(NST, srows);
@@ -1091,7 +1092,7 @@ static cudaError_t launch_step_k(const CUtensorMap &tin, const CUtensorMap &tG, 
     configured_dev = dev;
     configured_smem = smem;
   }
-  int items = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  int items = ((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TL::TY - 1) / TL::TY);
   if (FORCE && s.G_next) items += (s.nrows * ((g.nx + stir_chunk<R>() - 1) / stir_chunk<R>()) + NT / 32 - 1) / (NT / 32);
   int workers = max_blocks * sms;
   if (grid_limit > 0 && grid_limit < workers) workers = grid_limit;
@@ -1179,7 +1180,7 @@ static cudaError_t launch_batch_v(const BatchTables &bt, const Geometry<typename
                                   const long long *bstep, int grid_limit, int ntiles, cudaStream_t stream) {
   using TL = Tile<S, VS>;
   constexpr int CPT = sizeof(S) == 8 ? 1 : 2;
-  constexpr int NT = NTHREADS / CPT;
+  constexpr int NT = TILE_THREADS;
   auto kern = batch_step_kernel<S, VS, MASK, FORCE, CPT, NST>;
   const int smem = TL::smem(NST, FORCE ? srows : 0) + NST * (int)sizeof(TileInfo);
   static int configured_dev = -1, configured_smem = -1, max_blocks = 0, sms = 0;
