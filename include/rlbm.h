@@ -180,9 +180,10 @@ RLBM_API int32_t rlbm_num_planes(const rlbm_ctx *ctx);
 
 /* Launch shape of the fused step kernel: `ctas` persistent CTAs walk the lattice's
  * 32 x 8 tiles (0 = as many as are resident at once, the default; larger values are
- * clamped), `stages` (1 or 2; 0 keeps the current value) tiles of shared memory rotate
- * in its TMA pipeline (default 2), and `stir_rows` says where the stirring rows of a tile
- * come from: 1 = staged with the tile by TMA (default), 2 = read from global memory (less
+ * clamped; 32 x 4 in FP64), `stages` (1 or 2; 0 keeps the current value; the default
+ * depends on the storage, the mask and whether a step follows another in the same call)
+ * tiles of shared memory rotate in its TMA pipeline, and `stir_rows` says where the
+ * stirring rows of a tile come from: 1 = staged with the tile by TMA (default), 2 = read from global memory (less
  * shared memory per CTA, so more CTAs per SM); 0 keeps the current value.  A tuning
  * control: results do not depend on it.  The paper has no counterpart. */
 RLBM_API rlbm_status rlbm_set_launch(rlbm_ctx *ctx, int32_t ctas, int32_t stages, int32_t stir_rows);

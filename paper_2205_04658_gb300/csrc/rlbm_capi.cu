@@ -208,7 +208,7 @@ struct rlbm_ctx {
   HostPhys phys;
   int sms = 0;                 // multiprocessors of the device
   int grid_limit = 0;          // step kernel: 0 = one wave of resident CTAs
-  int stages = 2;              // shared-memory pipeline depth of the step kernel (1 or 2)
+  int stages = 1, chained_stages = 1;  // shared-memory pipeline depth of the step kernel (1 or 2)
   int stir_rows = 1;           // stirring rows: 1 = staged with each tile, 2 = read from global memory
   unsigned launch_seq = 0;     // step-kernel launches so far (selects the tile counter)
   int halo_faces = 0;          // a strip: faces whose ghost rows come from neighbours (bit 0 below, 1 above)
@@ -241,11 +241,12 @@ cudaError_t dispatch_step_raw(rlbm_ctx *c, const CUtensorMap *ti, void *fout, in
   const void *tg = tgmap ? tgmap : &c->tmap_G[n & 1], *te = &c->tmap_EY;
   int *ctr = c->at<int>(c->L.ctr);
   const unsigned seq = c->launch_seq++;
+  const int stages = chained ? c->chained_stages : c->stages;
   switch (c->cfg.precision) {
-    case RLBM_F64: return launch_step_f64(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    case RLBM_F32: return launch_step_f32(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    case RLBM_F16: return launch_step_f16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    default: return launch_step_bf16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F64: return launch_step_f64(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F32: return launch_step_f32(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F16: return launch_step_f16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    default: return launch_step_bf16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
   }
 }
 
@@ -559,6 +560,14 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   c->geom.nx = cfg->nx; c->geom.ny = cfg->ny; c->geom.pitch = L.pitch; c->geom.plane = L.plane;
   c->geom.walls = is_strip(*cfg) ? STRIP_Y : (cfg->walls_y ? WALLS_Y : 0) | (cfg->open_x ? OPEN_X : 0);
   c->geom.nbmask = nullptr;
+  // FP32 and FP64: one stage (512^2 FP32 10.0 us per step against 12.0, 4096^2 equal); the 16-bit forms
+  // keep two (FP16 4096^2 336 us against 357, 1024^2 26.6 against 27.9, though 512^2 11.1 against 10.5).
+  // With a mask it is the other way round: FP16 2048 x 512 28.1 us with two, 26.7 with one, FP32 25.7 and
+  // 27.1, though there a launch by itself, which waits for its first copy, is faster with one (20 steps
+  // observed one by one at 1024 x 256: 905 us against 933 to 992).  (By the registers the compiler takes
+  // for each form, hence the CTAs that fit on an SM.)
+  c->stages = store_bytes(cfg->precision) == 2 && !needs_mask(*cfg) ? 2 : 1;
+  c->chained_stages = cfg->precision == RLBM_F32 && needs_mask(*cfg) ? 2 : c->stages;
   {
     const std::string tm = make_tensor_maps(c);
     if (!tm.empty()) { c->msg = tm; return bail(RLBM_E_CUDA); }
@@ -912,7 +921,7 @@ rlbm_status rlbm_set_launch(rlbm_ctx *c, int32_t ctas, int32_t stages, int32_t s
   if (ctas < 0 || stages < 0 || stages > 2 || stir_rows < 0 || stir_rows > 2)
     return c->fail(RLBM_E_INVAL, "ctas must be >= 0, stages 0, 1 or 2 and stir_rows 0, 1 or 2");
   c->grid_limit = ctas;
-  if (stages) c->stages = stages;
+  if (stages) c->stages = c->chained_stages = stages;
   if (stir_rows) c->stir_rows = stir_rows;
   return RLBM_OK;
 }
@@ -933,7 +942,7 @@ rlbm_status rlbm_autotune(rlbm_ctx *c, int32_t reps, double *ms_out) {
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return c->fail(RLBM_E_CUDA, "cudaEventCreate failed");
-  const int save_grid = c->grid_limit, save_stages = c->stages, save_rows = c->stir_rows;
+  const int save_grid = c->grid_limit, save_stages = c->stages, save_chained = c->chained_stages, save_rows = c->stir_rows;
   float best = 1e30f;
   int best_grid = save_grid, best_stages = save_stages, best_rows = save_rows;
   const HostStir st = stir_for_step(c, c->step);
@@ -942,7 +951,7 @@ rlbm_status rlbm_autotune(rlbm_ctx *c, int32_t reps, double *ms_out) {
     for (int si = 0; si < 2 && e == cudaSuccess; ++si)
       for (int gi = 0; gi < 4 && e == cudaSuccess; ++gi) {
         c->stir_rows = rows_opts[ri];
-        c->stages = stage_opts[si];
+        c->stages = c->chained_stages = stage_opts[si];
         c->grid_limit = grid_opts[gi];
         // the step kernel reads the current buffer and writes the other one; repeating it
         // leaves the state (and the step counter) as it was.  The repetitions are chained as
@@ -960,10 +969,10 @@ rlbm_status rlbm_autotune(rlbm_ctx *c, int32_t reps, double *ms_out) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->grid_limit = best_grid;
-  c->stages = best_stages;
+  c->stages = c->chained_stages = best_stages;
   c->stir_rows = best_rows;
   if (e != cudaSuccess) {
-    c->grid_limit = save_grid; c->stages = save_stages; c->stir_rows = save_rows;
+    c->grid_limit = save_grid; c->stages = save_stages; c->chained_stages = save_chained; c->stir_rows = save_rows;
     return c->cuda_fail(e, "autotune launch");
   }
   if (ms_out) *ms_out = best / reps;
@@ -1116,7 +1125,6 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
   b->d_prep0 = reinterpret_cast<int *>(b->ws + L.prep0);
   b->d_bstep = reinterpret_cast<long long *>(b->ws + L.bstep);
   b->d_tctr = reinterpret_cast<int *>(b->ws + L.tctr);
-  b->stages = members[0]->stages;
   const int nrows = members[0]->L.nrows;
   b->srows = (nrows > 0 && nrows <= 16) ? nrows : 0;
   std::vector<int> tile0(nmembers + 1, 0), prep0(nmembers + 1, 0);
@@ -1143,6 +1151,9 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
     prep0[i + 1] = prep0[i] + c->L.nrows * ((c->cfg.nx + chunk - 1) / chunk);
     if (c->geom.nbmask) b->mask = true;
   }
+  // (16 x 512^2, us per step with one stage and with two: FP32 108 and 119, FP16 96 and 105, with masks
+  // FP16 96 and 105, but FP32 114 and 105)
+  b->stages = b->mask && members[0]->cfg.precision == RLBM_F32 ? 2 : 1;
   b->ntiles = tile0[nmembers];
   Scoped dev(b->device);
   cudaError_t e;

@@ -24,6 +24,11 @@ __device__ __forceinline__ int ghost_row(int y, int ny, int walls) {
 }
 constexpr long long WAIT_CYCLES = 4000000000ll;  // ~2 s at 2 GHz: bounded TMA waits
 
+// Bytes of the two buffers from which odd steps walk the lattice backwards (step_kernel).  The line lies
+// between 724^2 FP32 (71 MB: no effect; 512^2 lost 4 %) and 896^2 (109 MB: 22.7 -> 21.5 us per step);
+// 1024^2 (142 MB) 29.1 -> 28.0, 4096^2 and FP16 within 1 %.
+constexpr long long BACKWARDS_BYTES = 90000000ll;
+
 template <typename S, int VS> struct Tile {
   static constexpr int Q = VSet<VS>::Q, TY = TileRows<S>::value;
   static constexpr int V = PadLayout<S>::V;
@@ -46,11 +51,12 @@ template <typename S, int VS> struct Tile {
 };
 
 // One cell per thread: the FP64 path.
-template <typename S, int VS, bool MASK, bool FORCE, int CPT, class G, class W>
-__device__ __forceinline__ typename std::enable_if<CPT == 1>::type
+// `release` is called once the staged tile has been read (by every thread); false: wind down.
+template <typename S, int VS, bool MASK, bool FORCE, int CPT, class G, class W, class F>
+__device__ __forceinline__ typename std::enable_if<CPT == 1, bool>::type
 tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int tid, const G &g, const W &wts,
            const Physics<typename RealOf<S>::type> &p, const Stir<typename RealOf<S>::type> &st, bool staged,
-           unsigned *err, typename RealOf<S>::type *macro_out) {
+           unsigned *err, typename RealOf<S>::type *macro_out, F release) {
   using R = typename RealOf<S>::type;
   using V = VSet<VS>;
   using TL = Tile<S, VS>;
@@ -63,11 +69,10 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     unsigned nb = 0;
     if (MASK && g.nbmask && inside) nb = g.nbmask[(long long)y * g.nx + x];
     const bool fluid = inside && !(MASK && (nb & 16u));
-    R hn[Q];
+    R hn[Q], h[Q], Fx = p.body_x, Fy = p.body_y;
     if (fluid) {
       // pull-streaming from the staged tile: cell (lx, ly) at row ly + 1, column lx + V
       const int b0 = (ly + 1) * TL::TXB + lx + TL::V;
-      R h[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const S *pl = tile + q * TL::TYB * TL::TXB + b0;
@@ -91,10 +96,6 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
         }
         h[q] = acc;
       }
-      const Mom<R> M = moments_of<R, R, VS, FORCE>(h);
-      const Macro<R> m = cell_macro<R, VS>(h, M, p.vmax2);
-      if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
-      R Fx = p.body_x, Fy = p.body_y;
       if (FORCE) {  // F = sum_r Re[G_r(x) EY_r(y)], the table holding (Re, -Im)
         R Fx2 = R(0), Fy2 = R(0);
         for (int r = 0; r < st.nrows; ++r) {
@@ -115,6 +116,12 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
         Fx += Fx2;
         Fy += Fy2;
       }
+    }
+    if (!release()) return false;
+    if (fluid) {
+      const Mom<R> M = moments_of<R, R, VS, FORCE>(h);
+      const Macro<R> m = cell_macro<R, VS>(h, M, p.vmax2);
+      if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
       if (macro_out) {  // the cell's Landau solution, force and streamed h, kept for the reverse sweep
         const long long nc = (long long)g.nx * g.ny, c = (long long)y * g.nx + x;
         macro_out[c] = m.eps_m1;
@@ -150,16 +157,17 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
         }
       }
     }
+    return true;
 }
 
 // Two cells per thread: cells (x, y) and (x, y + 1) of the 32 x 8 tile (y
 // even), all per-cell arithmetic on packed FP32 pairs.  The FP32, FP16 and BF16 paths.  The
 // two cells are adjacent rows, so the classes that move in y pull one of their rows for
 // both (each such value is read from shared memory and converted once).
-template <typename S, int VS, bool MASK, bool FORCE, int CPT, class G, class W>
-__device__ __forceinline__ typename std::enable_if<CPT == 2>::type
+template <typename S, int VS, bool MASK, bool FORCE, int CPT, class G, class W, class F>
+__device__ __forceinline__ typename std::enable_if<CPT == 2, bool>::type
 tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int tid, const G &g, const W &wts,
-           const Physics<float> &p, const Stir<float> &st, bool staged, unsigned *err, float *macro_out) {
+           const Physics<float> &p, const Stir<float> &st, bool staged, unsigned *err, float *macro_out, F release) {
   using V = VSet<VS>;
   using TL = Tile<S, VS>;
   using T = F2;
@@ -169,7 +177,8 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
   const int x = x0 + lx, yA = y0 + 2 * ly, yB = yA + 1;
   const S *tile = reinterpret_cast<const S *>(stg);
   const bool inA = x < g.nx && yA < g.ny, inB = x < g.nx && yB < g.ny;
-  const bool border = x0 == 0 || y0 == 0 || x0 + TILE_X >= g.nx || y0 + TL::TY >= g.ny;  // the tile's
+  // whether the tile holds boundary cells
+  const bool border = x0 == 0 || y0 == 0 || x0 + TILE_X >= g.nx || y0 + TL::TY >= g.ny;
   unsigned nbA = 0, nbB = 0;
   if (MASK && g.nbmask) {
     if (inA) nbA = g.nbmask[(long long)yA * g.nx + x];
@@ -210,6 +219,8 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     // (lanes without fluid, outside the lattice or solid, pull what the stage holds there and drop it)
     const int b0 = (2 * ly + 1) * TL::TXB + lx + TL::V;
     T h[Q];
+    auto pull = [&](auto masked) {
+      constexpr bool M = decltype(masked)::value;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const S *pl = tile + q * TL::TYB * TL::TXB + b0;
@@ -218,24 +229,30 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
       T acc = T(wts.beta2[q][0]) * T(load_s_raw<S>(pl), load_s_raw<S>(pl + DB));
       if (sx != 0) {
         float vA = load_s_raw<S>(pl - sx), vB = load_s_raw<S>(pl + DB - sx);
-        if (MASK && ((nbA >> (4 - sx)) & 1u)) vA = load_s_raw<S>(own);
-        if (MASK && ((nbB >> (4 - sx)) & 1u)) vB = load_s_raw<S>(own + DB);
+        if (M && ((nbA >> (4 - sx)) & 1u)) vA = load_s_raw<S>(own);
+        if (M && ((nbB >> (4 - sx)) & 1u)) vB = load_s_raw<S>(own + DB);
         acc = fma(T(wts.beta2[q][1]), T(vA, vB), acc);
       }
       if (sy != 0) {
         float vA = load_s_raw<S>(pl - sy * TL::TXB), vB = load_s_raw<S>(pl + DB - sy * TL::TXB);
-        if (MASK && ((nbA >> (4 - 3 * sy)) & 1u)) vA = load_s_raw<S>(own);
-        if (MASK && ((nbB >> (4 - 3 * sy)) & 1u)) vB = load_s_raw<S>(own + DB);
+        if (M && ((nbA >> (4 - 3 * sy)) & 1u)) vA = load_s_raw<S>(own);
+        if (M && ((nbB >> (4 - 3 * sy)) & 1u)) vB = load_s_raw<S>(own + DB);
         acc = fma(T(wts.beta2[q][2]), T(vA, vB), acc);
       }
       if (sx != 0 && sy != 0) {
         float vA = load_s_raw<S>(pl - sy * TL::TXB - sx), vB = load_s_raw<S>(pl + DB - sy * TL::TXB - sx);
-        if (MASK && ((nbA >> (4 - 3 * sy - sx)) & 1u)) vA = load_s_raw<S>(own);
-        if (MASK && ((nbB >> (4 - 3 * sy - sx)) & 1u)) vB = load_s_raw<S>(own + DB);
+        if (M && ((nbA >> (4 - 3 * sy - sx)) & 1u)) vA = load_s_raw<S>(own);
+        if (M && ((nbB >> (4 - 3 * sy - sx)) & 1u)) vB = load_s_raw<S>(own + DB);
         acc = fma(T(wts.beta2[q][3]), T(vA, vB), acc);
       }
       h[q] = acc;
     }
+    };
+    // warps none of whose cells has a solid neighbour skip the substitutions (a third of an open
+    // channel's instructions; at 15 % discs a third of the warps)
+    if (MASK && __any_sync(0xffffffffu, ((nbA | nbB) & 0x1efu) != 0)) pull(std::true_type());
+    else pull(std::false_type());
+    if (!release()) return false;
     if (!both) {  // a lane without fluid (outside the lattice or solid) computes the rest state
 #pragma unroll
       for (int q = 0; q < Q; ++q) h[q] = T(flA ? h[q].v.x : 0.0f, flB ? h[q].v.y : 0.0f);
@@ -310,7 +327,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
       }
     }
   }
-  {  // coalesced stores straight from registers (one 128-byte line per warp and plane)
+  {  // coalesced stores straight from registers (one 128-byte line per warp, row and plane)
     S *oA = fout + (long long)(yA + 1) * g.pitch + x + TL::XOFF;
     S *oB = oA + g.pitch;
     if (inA) {
@@ -323,7 +340,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     }
   }
   // ghost copies of the periodic neighbours (boundary cells only)
-  if (!border) return;
+  if (!border) return true;
 #pragma unroll
   for (int lane = 0; lane < 2; ++lane) {
     const int y = lane ? yB : yA;
@@ -339,6 +356,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
       for (int q = 0; q < Q; ++q) o[q * g.plane] = lane ? sB[q] : sA[q];
     }
   }
+  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -347,8 +365,8 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
 // lattice.  Per tile, one 3-D TMA copy stages all Q planes of the tile plus a
 // one-cell halo (ghost rows/columns carry the periodic wrap) into shared memory, with
 // the tile's stirring rows; NST stages rotate on mbarriers (NST = 2: the next tile is
-// in flight while this one is computed; NST = 1: more CTAs per SM hide the copy
-// instead).  Each thread pull-streams its cell(s) from shared memory (bilinear
+// in flight while this one is computed; NST = 1: its copy starts after the pull of this one
+// and hides behind the arithmetic, and more CTAs fit on an SM: 512^2 FP32 12.0 -> 10.0 us).  Each thread pull-streams its cell(s) from shared memory (bilinear
 // weights, bounce-back substitution from the mask), takes the moments, Landau-matches,
 // relaxes, adds the force and stores the Q results with coalesced stores, refreshing
 // the ghost copies of boundary cells.
@@ -395,6 +413,10 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
   // started that way were 3 % slower at 4096^2.)
   int *ctr = tile_ctr + (seq & 1u);
   const bool one_each = nitems <= nworkers;
+  // When the two buffers are larger than L2, odd steps walk the lattice backwards: what the step before
+  // wrote (and read) last is then still in L2 when it is read (and overwritten); one way every time
+  // misses on nearly all of it.
+  const bool backwards = (p.step & 1u) && 2ll * VSet<VS>::Q * g.plane * (long long)sizeof(S) > BACKWARDS_BYTES;
 
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) mbar_init(&bar[s], 1);
@@ -422,6 +444,7 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
       return;
     }
     t -= tile0;
+    if (backwards) t = ntiles - 1 - t;
     // row = t / ntx, column = t mod ntx: the float quotient corrected exactly (t < 2^24)
     int row = (int)((float)t * rcp_ntx), col = t - row * ntx;
     while (col < 0) { --row; col += ntx; }
@@ -443,46 +466,56 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
   }
   __syncthreads();
 
-  // Every thread waits for the staged tile (bounded); the vote in the barrier makes the
-  // whole CTA wind down together if a copy never lands.
-  bool alive = true;
-  {
-    const bool ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
+  // Every thread waits for the staged tile (bounded); a vote in a barrier makes the whole CTA
+  // wind down together if a copy never lands.
+  bool alive = true, ok = true;
+  if (NST >= 2) {
+    ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
   for (int k = 0; alive; ++k) {
     const int s = k % NST;
+    if (NST == 1) ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
     const int t = item_of[s];
-    if (t < 0) break;
+    if (NST >= 2 && t < 0) break;
+    // NST = 1: the stage is free, and the next tile's copy starts, once every thread has read its tile
+    // (the barrier also carries the vote); all that follows the pull hides that copy
+    auto release = [&]() {
+      if (NST == 1) {
+        if (__syncthreads_or(!ok)) return false;
+        if (tid == 0 && t >= 0) {
+          fill(0, pending);
+          if (!one_each) pending = atomicAdd(ctr, 1);
+        }
+      }
+      return true;
+    };
     if (t >= tile0) {
       const int xy = tile_xy[s];
-      tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, fout, (xy & 0xffff) * TILE_X,
-                                          (xy >> 16) * TL::TY, tid, g, g, p, st, staged, err,
-                                          STORE ? macro_out : static_cast<R *>(nullptr));
-    } else if (FORCE) {
+      alive = tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, fout, (xy & 0xffff) * TILE_X,
+                                                  (xy >> 16) * TL::TY, tid, g, g, p, st, staged, err,
+                                                  STORE ? macro_out : static_cast<R *>(nullptr), release);
+    } else {
+      alive = release();
+      if (NST == 1 && t < 0) break;
       const int i = t * (NT / 32) + tid / 32;
-      if (i < nprep) {
+      if (FORCE && alive && i < nprep) {
         const int r = i / chunks;
         stir_row_chunk<R>(st.modes, st.step_next, r, i - r * chunks, g.nx, tid & 31, st.G_next + (long long)r * g.nx);
       }
     }
-    if (NST == 1) {  // the only stage is free once every thread is done with it
-      __syncthreads();
+    if (NST >= 2) {
+      // the next stage's barrier completes with its tile, or at once when it has none
+      const int sn = (k + 1) % NST;
+      ok = mbar_wait_bounded(&bar[sn], ((k + 1) / NST) & 1, WAIT_CYCLES);
+      if (__syncthreads_or(!ok)) {  // (also the barrier after which stage s is free)
+        alive = false;
+        break;
+      }
       if (tid == 0) {
-        fill(0, pending);
+        fill(s, pending);
         if (!one_each) pending = atomicAdd(ctr, 1);
       }
-    }
-    // the next stage's barrier completes with its tile, or at once when it has none
-    const int sn = (k + 1) % NST;
-    const bool ok = mbar_wait_bounded(&bar[sn], ((k + 1) / NST) & 1, WAIT_CYCLES);
-    if (__syncthreads_or(!ok)) {  // (NST = 2: also the barrier after which stage s is free)
-      alive = false;
-      break;
-    }
-    if (NST >= 2 && tid == 0) {
-      fill(s, pending);
-      if (!one_each) pending = atomicAdd(ctr, 1);
     }
   }
   if (!alive && tid == 0) {
@@ -606,15 +639,29 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     for (int s = 0; s < NST; ++s) fill(s, atomicAdd(bt.tile_ctr, 1));
     pending = atomicAdd(bt.tile_ctr, 1);
   }
-  bool alive = true;
-  {
-    const bool ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
+  bool alive = true, ok = true;
+  if (NST >= 2) {
+    ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
   for (int k = 0; alive; ++k) {
     const int s = k % NST;
+    if (NST == 1) ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
     const TileInfo ti = info[s];
-    if (ti.m < 0) break;
+    auto release = [&]() {  // (as in step_kernel)
+      if (NST == 1) {
+        if (__syncthreads_or(!ok)) return false;
+        if (tid == 0 && ti.m >= 0) {
+          fill(0, pending);
+          pending = atomicAdd(bt.tile_ctr, 1);
+        }
+      }
+      return true;
+    };
+    if (ti.m < 0) {
+      if (NST == 1) alive = release();
+      break;
+    }
     Physics<R> p = p0;
     p.round_key = ti.round_key;
     p.step = (unsigned)(ti.n & 0xffffffffll);
@@ -622,25 +669,20 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     Stir<R> st{};
     if (FORCE && staged) st.nrows = srows;
     else if (FORCE) st = member_stir<R>(bt.mem[ti.m], ti.n, amp);
-    tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, (S *)ti.fout, ti.x0, ti.y0, tid, ti.dims,
-                                        wts, p, st, staged, ti.err, static_cast<R *>(nullptr));
-    if (NST == 1) {  // the only stage is free once every thread is done with it
-      __syncthreads();
+    alive = tile_cells<S, VS, MASK, FORCE, CPT>(smem + s * stage_stride, ey_off, (S *)ti.fout, ti.x0, ti.y0, tid, ti.dims,
+                                                wts, p, st, staged, ti.err, static_cast<R *>(nullptr), release);
+    if (NST >= 2) {
+      // the next stage's barrier completes with its tile, or at once when it has none
+      const int sn = (k + 1) % NST;
+      ok = mbar_wait_bounded(&bar[sn], ((k + 1) / NST) & 1, WAIT_CYCLES);
+      if (__syncthreads_or(!ok)) {  // (also the barrier after which stage s is free)
+        alive = false;
+        break;
+      }
       if (tid == 0) {
-        fill(0, pending);
+        fill(s, pending);
         pending = atomicAdd(bt.tile_ctr, 1);
       }
-    }
-    // the next stage's barrier completes with its tile, or at once when it has none
-    const int sn = (k + 1) % NST;
-    const bool ok = mbar_wait_bounded(&bar[sn], ((k + 1) / NST) & 1, WAIT_CYCLES);
-    if (__syncthreads_or(!ok)) {  // (NST = 2: also the barrier after which stage s is free)
-      alive = false;
-      break;
-    }
-    if (NST >= 2 && tid == 0) {
-      fill(s, pending);
-      pending = atomicAdd(bt.tile_ctr, 1);
     }
   }
   if (!alive && tid == 0) {
