@@ -346,7 +346,7 @@ template <class C, bool BINS>
 __global__ void __launch_bounds__(512)
 fft_cols_kernel(const C *__restrict__ Z, int nx, int ny, const C *__restrict__ tw, FftPlan plan, int padded, int ncol,
                 double scale, double *__restrict__ bins, int nbins, long long k2lo, long long k2hi,
-                double *__restrict__ partials) {
+                double *__restrict__ partials, double *__restrict__ out4, unsigned *__restrict__ sync) {
   using Sum = typename SumOf<C>::type;
   extern __shared__ __align__(16) unsigned char fft_sm[];
   C *src = reinterpret_cast<C *>(fft_sm), *dst = src + ncol * padded;
@@ -396,11 +396,27 @@ fft_cols_kernel(const C *__restrict__ Z, int nx, int ny, const C *__restrict__ t
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     if (lane == 0) red[warp] = acc;
     __syncthreads();
+    // the last block adds the strips' sums in order
+    __shared__ bool last;
     if (threadIdx.x == 0) {
       double sum = 0.0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
-      partials[(long long)blockIdx.x * 4] = scale * sum;
-      partials[(long long)blockIdx.x * 4 + 1] = partials[(long long)blockIdx.x * 4 + 2] = partials[(long long)blockIdx.x * 4 + 3] = 0.0;
+      partials[blockIdx.x] = scale * sum;
+      __threadfence();
+      last = atomicInc(sync, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(&partials[i]);
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double sum = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
+      out4[0] = sum;
     }
   }
 }
@@ -538,40 +554,38 @@ __global__ void band_kernel(const C *__restrict__ Z, int nx, int ny, long long k
 
 template <class C>
 static cudaError_t band_energy_t(int nx, int ny, const C *twx, const C *twy, C *z0, C *z1, long long k2lo, long long k2hi,
-                                 double *partials, double *out4, cudaStream_t st) {
+                                 double *partials, double *out4, unsigned *sync, cudaStream_t st) {
   const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
   cudaError_t e = cudaSuccess;
-  int blocks = nx;
   if (const int nc = strip_columns(nx, ny)) {
     const FftPlan py = make_plan(ny);
     const int smem = 2 * nc * fft_padded(ny) * (int)sizeof(C);
     if ((e = fft_allow_smem(fft_cols_kernel<C, false>, smem)) != cudaSuccess) return e;
     C *Z = row_transforms(make_plan(nx), ny, twx, z0, z1, st, e);
-    blocks = (nx + nc - 1) / nc;
-    fft_cols_kernel<C, false><<<blocks, cols_threads(py, nc), smem, st>>>(
-        Z, nx, ny, twy, py, fft_padded(ny), nc, scale, nullptr, 0, k2lo, k2hi, partials);
+    fft_cols_kernel<C, false><<<(nx + nc - 1) / nc, cols_threads(py, nc), smem, st>>>(
+        Z, nx, ny, twy, py, fft_padded(ny), nc, scale, nullptr, 0, k2lo, k2hi, partials, out4, sync);
+    return e == cudaSuccess ? cudaGetLastError() : e;
   } else {
     C *Z = velocity_transform(nx, ny, twx, twy, z0, z1, st, e);
     band_kernel<C><<<nx, 256, 0, st>>>(Z, nx, ny, k2lo, k2hi, scale, partials);
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_reduce_partials(partials, blocks, out4, st);
+  return launch_reduce_partials(partials, nx, out4, st);
 }
 
 template <class C>
 static cudaError_t spectrum_t(int nx, int ny, const C *twx, const C *twy, C *z0, C *z1, double *bins, int nbins,
                               cudaStream_t st) {
   const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
-  cudaError_t e = cudaMemsetAsync(bins, 0, sizeof(double) * nbins, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   if (const int nc = strip_columns(nx, ny)) {
     const FftPlan py = make_plan(ny);
     const int smem = 2 * nc * fft_padded(ny) * (int)sizeof(C);
     if ((e = fft_allow_smem(fft_cols_kernel<C, true>, smem)) != cudaSuccess) return e;
     C *Z = row_transforms(make_plan(nx), ny, twx, z0, z1, st, e);
     fft_cols_kernel<C, true><<<(nx + nc - 1) / nc, cols_threads(py, nc), smem, st>>>(
-        Z, nx, ny, twy, py, fft_padded(ny), nc, scale, bins, nbins, 0, 0, nullptr);
+        Z, nx, ny, twy, py, fft_padded(ny), nc, scale, bins, nbins, 0, 0, nullptr, nullptr, nullptr);
   } else {
     C *Z = velocity_transform(nx, ny, twx, twy, z0, z1, st, e);
     const size_t smem = nbins <= 6144 ? sizeof(double) * nbins : 0;
@@ -581,9 +595,9 @@ static cudaError_t spectrum_t(int nx, int ny, const C *twx, const C *twy, C *z0,
 }
 
 cudaError_t launch_band_energy(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, long long k2lo,
-                               long long k2hi, double *partials, double *out4, cudaStream_t st) {
-  if (f64) return band_energy_t<Cd>(nx, ny, (const Cd *)twx, (const Cd *)twy, (Cd *)z0, (Cd *)z1, k2lo, k2hi, partials, out4, st);
-  return band_energy_t<Cf>(nx, ny, (const Cf *)twx, (const Cf *)twy, (Cf *)z0, (Cf *)z1, k2lo, k2hi, partials, out4, st);
+                               long long k2hi, double *partials, double *out4, unsigned *sync, cudaStream_t st) {
+  if (f64) return band_energy_t<Cd>(nx, ny, (const Cd *)twx, (const Cd *)twy, (Cd *)z0, (Cd *)z1, k2lo, k2hi, partials, out4, sync, st);
+  return band_energy_t<Cf>(nx, ny, (const Cf *)twx, (const Cf *)twy, (Cf *)z0, (Cf *)z1, k2lo, k2hi, partials, out4, sync, st);
 }
 
 cudaError_t launch_spectrum(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, double *bins,

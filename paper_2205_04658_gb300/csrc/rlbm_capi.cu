@@ -365,7 +365,7 @@ std::string make_tensor_maps(rlbm_ctx *c) {
 
 // Observation of the current state (rlbm_kernels.cuh): mode 0 the wanted fields and the
 // totals, mode 1 the velocities into z0, mode 2 the column means into L.cols.
-cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = false, bool uy = false) {
+cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = false, bool uy = false, int nbins = 0) {
   const void *fin = c->ws + c->L.pop[c->cur];
   HostObs o{};
   o.eps = eps ? c->at<double>(c->L.eps) : nullptr;
@@ -375,6 +375,8 @@ cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = 
   o.partials = c->at<double>(c->L.partials);
   o.totals = mode == 2 ? c->at<double>(c->L.cols) : c->at<double>(c->L.totals);
   o.sync = c->at<unsigned>(c->L.sync);
+  o.bins = c->at<double>(c->L.bins);
+  o.nbins = nbins;
   unsigned *err = c->at<unsigned>(c->L.err);
   const double e0 = c->cfg.eps0, vm = c->phys.vmax2;
   switch (c->cfg.precision) {
@@ -757,9 +759,9 @@ rlbm_status rlbm_spectrum(rlbm_ctx *c, int32_t nbins, double *E) {
   if (is_strip(c->cfg)) return c->fail(RLBM_E_INVAL, "a strip has no spectrum of its own: it needs the whole lattice");
   if (nbins < 1 || !E) return c->fail(RLBM_E_INVAL, "nbins must be >= 1 and E non-NULL");
   Scoped dev(c->device);
-  cudaError_t e = dispatch_observe(c, 1);
-  if (e != cudaSuccess) return c->cuda_fail(e, "velocity kernel launch");
   const int nb = std::min(nbins, c->L.max_bins);
+  cudaError_t e = dispatch_observe(c, 1, false, false, false, nb);
+  if (e != cudaSuccess) return c->cuda_fail(e, "velocity kernel launch");
   e = launch_spectrum(c->cfg.precision == RLBM_F64, c->cfg.nx, c->cfg.ny,
                       c->at<double2>(c->L.twx), c->at<double2>(c->L.twy), c->at<double2>(c->L.z0),
                       c->at<double2>(c->L.z1), c->at<double>(c->L.bins), nb, c->stream);
@@ -826,7 +828,8 @@ rlbm_status rlbm_band_energy(rlbm_ctx *c, int64_t k2lo, int64_t k2hi, double *E)
   double *out = c->at<double>(c->L.totals);
   e = launch_band_energy(c->cfg.precision == RLBM_F64, c->cfg.nx, c->cfg.ny,
                          c->at<double2>(c->L.twx), c->at<double2>(c->L.twy), c->at<double2>(c->L.z0),
-                         c->at<double2>(c->L.z1), k2lo, k2hi, c->at<double>(c->L.partials), out, c->stream);
+                         c->at<double2>(c->L.z1), k2lo, k2hi, c->at<double>(c->L.partials), out,
+                         c->at<unsigned>(c->L.sync), c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "band energy kernels");
   if (rlbm_status s = check_device(c, c->L.totals + 32)) return s;
   std::memcpy(E, small(c, c->L.totals), sizeof(double));

@@ -778,6 +778,8 @@ struct ObsOut {
   double *partials;       // [blocks][4]
   double *totals;         // [4]; OBS_COLS: [2 nx]
   unsigned *sync;         // zeroed counters of finished blocks: 1, or one per tile column (OBS_COLS)
+  double *bins;           // OBS_V: nbins values cleared for the spectrum's sums
+  int nbins;
 };
 
 template <typename S, int VS, bool MASK, int MODE>
@@ -795,6 +797,8 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
   __shared__ double2 cols[8][32];
   __shared__ int cnt[8];
   __shared__ bool last;
+  if (MODE == OBS_V && blockIdx.x == 0)
+    for (int i = tid; i < out.nbins; i += 256) out.bins[i] = 0.0;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   const DF2 zero{F2(0.0f), F2(0.0f)};
   DF2 accf[4] = {zero, zero, zero, zero};
@@ -1304,7 +1308,7 @@ static cudaError_t launch_observe_t(int vset, int mode, const void *fin, const H
                                     const HostObs &ho, unsigned *err, int sms, cudaStream_t stream) {
   using R = typename RealOf<S>::type;
   const Geometry<R> g = to_geom<S>(hg);
-  const ObsOut o{ho.eps, ho.ux, ho.uy, ho.z, ho.partials, ho.totals, ho.sync};
+  const ObsOut o{ho.eps, ho.ux, ho.uy, ho.z, ho.partials, ho.totals, ho.sync, ho.bins, ho.nbins};
   const bool mask = hg.nbmask != nullptr;
   const S *a = (const S *)fin;
   if (vset == 3) {

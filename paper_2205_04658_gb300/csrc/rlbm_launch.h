@@ -53,6 +53,8 @@ struct HostObs {
   double2 *z;
   double *partials, *totals;
   unsigned *sync;
+  double *bins;  // mode 1: nbins values cleared for the spectrum
+  int nbins;
 };
 
 // One lattice of a batch, as the batched step kernel sees it (device memory, written by
@@ -167,7 +169,9 @@ cudaError_t launch_make_z(const double *ux, const double *uy, double2 *z, long l
 // overwritten.  f64: (re, im) in FP64; else high and low FP32 parts (re_h, im_h, re_l, im_l).
 // twx, twy: exp(-2 pi i t / n) in the same form.
 cudaError_t launch_band_energy(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, long long k2lo,
-                               long long k2hi, double *partials, double *out4, cudaStream_t st);
+                               long long k2hi, double *partials, double *out4, unsigned *sync, cudaStream_t st);
+// (launch_spectrum adds to bins, which the caller has cleared; launch_band_energy uses the zeroed
+// counter `sync` and leaves it zero)
 cudaError_t launch_spectrum(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, double *bins,
                             int nbins, cudaStream_t st);
 

@@ -103,8 +103,8 @@ extern "C" RLBM_API rlbm_status rlbm_spectrum_noalloc(const double *d_ux, const 
   twiddle_kernel<<<(nx + 255) / 256, 256, 0, st>>>(twx, nx);
   twiddle_kernel<<<(ny + 255) / 256, 256, 0, st>>>(twy, ny);
   if ((e = cudaGetLastError()) != cudaSuccess) { rlbm::set_thread_error(std::string("twiddle kernel: ") + cudaGetErrorString(e)); return RLBM_E_CUDA; }
-  // launch_spectrum zeroes the bins before it accumulates into them
-  e = rlbm::launch_make_z(d_ux, d_uy, z0, (long long)nx * ny, st);
+  e = cudaMemsetAsync(bins, 0, sizeof(double) * nbins, st);
+  if (e == cudaSuccess) e = rlbm::launch_make_z(d_ux, d_uy, z0, (long long)nx * ny, st);
   if (e == cudaSuccess) e = rlbm::launch_spectrum(true, nx, ny, twx, twy, z0, z1, bins, nbins, st);
   if (e != cudaSuccess) { rlbm::set_thread_error(std::string("spectrum kernels: ") + cudaGetErrorString(e)); return RLBM_E_CUDA; }
   e = cudaMemcpyAsync(d_E, bins, sizeof(double) * nbins, cudaMemcpyDeviceToDevice, st);
