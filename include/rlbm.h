@@ -145,7 +145,8 @@ RLBM_API rlbm_status rlbm_step(rlbm_ctx *ctx, int64_t nsteps);
  * sum T^00, sum T^0x, sum T^0y, sum 1/2 |v|^2 over fluid cells, v = u^i / u^0.
  * Runs the streaming and Landau matching of the next step without storing it, in the
  * context's compute type: FP64 for F64; FP32 for the others, with the FP64 re-solve of
- * the step kernel and the totals' FP32 deviation sums added per block in FP64. Syncs. */
+ * the step kernel, widened exactly, and the totals' sums in two-float (48-bit) arithmetic
+ * over a warp's cells and FP64 beyond. Syncs. */
 RLBM_API rlbm_status rlbm_moments(rlbm_ctx *ctx, double *eps, double *ux, double *uy, double *totals);
 
 /* Energy spectrum of the current state's velocity v = u^i / u^0 (Sec. "Turbulence"):
@@ -330,13 +331,13 @@ RLBM_API rlbm_status rlbm_set_mode_scale(rlbm_ctx *ctx, const double *sigma, int
  * rlbm_gradient runs the nsteps forward steps (the context ends at s0 + nsteps, exactly as
  * after rlbm_step(ctx, nsteps)), keeping the post-collision state every `segment` steps
  * (0: ceil(sqrt(nsteps))), then the hand-written adjoint backwards, recomputing each
- * segment from its checkpoint: about sqrt(nsteps) states of memory and one extra forward
- * pass.  The recomputation keeps, for every step of the segment in hand, the step's Landau
+ * segment but the last from its checkpoint: about sqrt(nsteps) states of memory and nearly
+ * one extra forward pass.  The run of a segment keeps, for every step of the segment in hand, the step's Landau
  * solution, force and streamed deviations h (5 + 17 values per cell for the paper's set,
  * in the storage type), which the reverse steps read.  segment >= nsteps keeps those
  * values for every step instead (one segment, e.g. 54 GB for 512^2 FP32 and 2000 steps):
- * the forward runs once and no step is recomputed.  The results do not depend on segment.  It returns J and dJ/dsigma_m (host, rlbm_num_modes values; may be NULL),
- * dJ/d(eta/s) (host, 1; may be NULL) and dJ/dF_body (host, 2; may be NULL; zero for the
+ * the forward runs once and no step is recomputed.  The results do not depend on segment.
+ * It returns J and dJ/dsigma_m (host, rlbm_num_modes values; may be NULL), dJ/d(eta/s) (host, 1; may be NULL) and dJ/dF_body (host, 2; may be NULL; zero for the
  * eight-direction set, which has no force term), evaluated at
  * the current sigma, eta/s and body force.  FP64 and FP32 storage only (E_INVAL for the
  * 16-bit forms).  Syncs.

@@ -9,13 +9,13 @@
 //   kappa_n = dj_n/dS_n + (dC_n/dS)^T (P^T kappa_{n+1}),
 //
 // and every step adds (dC_n/dtheta)^T (P^T kappa_{n+1}) to the parameter gradients.
-// One launch per step gathers S_n (forward pull of B_{n-1}) and P^T kappa_{n+1} (the
-// transposed pull: reversed offsets, same bilinear weights, and at a solid corner the
-// cell's own reversed plane, so it has the form of the forward pull), runs the cell's
-// reverse and writes kappa_n.  Landau matching R(v) = m - T v - (T^00 - m.v) v = 0 is
+// One launch per step gathers P^T kappa_{n+1} (the transposed pull: reversed offsets, same
+// bilinear weights, and at a solid corner the cell's own reversed plane, so it has the form of
+// the forward pull) and S_n (kept by the forward; pulled from the last state for the first
+// launch), runs the cell's reverse and writes kappa_n.  Landau matching R(v) = m - T v - (T^00 - m.v) v = 0 is
 // differentiated implicitly: the adjoint w solves (dR/dv)^T w = vbar and the moments
-// receive -(dR/dp)^T w.  The recomputed forward of a segment keeps each step's Landau
-// solution (eps - 1, v) and force (F_x, F_y) per cell; the reverse step reads them instead
+// receive -(dR/dp)^T w.  The forward of a segment keeps each step's Landau solution (eps - 1, v),
+// force (F_x, F_y) and streamed populations per cell; the reverse step reads them instead
 // of solving Landau matching and synthesising the stirring force again (the force
 // adjoint's row projections still use the step's tables).
 #include "rlbm_kernels.cuh"
@@ -28,8 +28,8 @@ template <typename R> struct AdjStir {
   int eyp;
 };
 
-// Pulls of one cell from staged tiles (32 x 8 tile with its one-cell halo, the layout of
-// the forward step kernel's stages; b0 = the cell's offset in a staged plane).
+// Pulls of one cell from staged tiles (the tile with its one-cell halo, in the layout of the
+// forward step kernel's stages; b0 = the cell's offset in a staged plane).
 //   forward pull   h_q(x)   = sum_c beta_{q,c} B_q(x - o_c)
 //   transposed     lam_q(x) = sum_c beta_{q,c} kappa_q(x + o_c)
 // with o_c in {(0,0), (sx,0), (0,sy), (sx,sy)}.  A solid source corner of the forward pull
@@ -523,7 +523,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
 
 // The FP32 reverse step with two cells per thread (128 threads): cells (x, y) and (x, y + 1) of
 // the 32 x 8 tile, the pulls, moments, the cell's reverse and the objective on packed FP32
-// pairs, as the forward step kernel computes its FP32 paths.  Tile walk, staging, chaining,
+// pairs, as the forward step kernel computes its FP32 paths.  Tile walk, boxes, chaining,
 // stores, row projections and tile sums as in adjoint_kernel.
 // One stage per CTA and four CTAs per SM (128 registers): the other CTAs' tiles hide a tile's copy,
 // and the 512^2 lattice takes 2 rounds instead of 3 (gradient of 200 steps 8.27 ms; three CTAs of

@@ -1384,7 +1384,7 @@ rlbm_status rlbm_set_mode_scale(rlbm_ctx *c, const double *sigma, int32_t nmodes
   cudaError_t e = cudaMemcpyAsync(c->ws + c->L.mode_scale, sigma, 8 * (size_t)nmodes, cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "copy of the mode multipliers");
   c->unit_scale = unit;
-  // the coefficients and table of the current and next step are redrawn with them
+  // the table of the current step is built again with them
   if ((e = stir_prime(c, c->step)) != cudaSuccess) return c->cuda_fail(e, "stirring set-up kernels");
   return check_device(c);
 }
@@ -1537,7 +1537,6 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
   }
   int kc = 0;  // kap[kc] holds kappa_{n+1}
   // the last state: objective only (its force terms are multiplied by a zero adjoint)
-  a.B = c->ws + c->L.pop[c->cur];
   a.tB = &c->tmap_in[c->cur];
   a.kin = nullptr;
   a.tK = nullptr;
@@ -1553,8 +1552,7 @@ rlbm_status rlbm_gradient(rlbm_ctx *c, int64_t nsteps, int32_t segment, void *de
       return c->cuda_fail(e, "step kernel launch (recompute)");
     }
     for (int64_t n = hi - 1; n >= lo; --n) {
-      a.B = ckpt(k);  // (not read: the step's streamed h is in its stored values)
-      a.tB = &mck[k];
+      a.tB = &mck[k];  // (not read: the step's streamed h is in its stored values)
       a.kin = w + G.kap[kc];
       a.tK = &mkap[kc];
       a.kout = w + G.kap[kc ^ 1];
