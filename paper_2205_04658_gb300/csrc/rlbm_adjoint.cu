@@ -382,7 +382,9 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
     const bool ok = my_tiles == 0 || mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
-  for (int k = 0; alive && k < my_tiles; ++k) {
+  static_assert(NST >= 2, "a stage is refilled behind the vote at the end of its tile");
+  int k = 0;  // tiles finished; min(NST + k, my_tiles) copies have been started when the CTA winds down
+  for (; alive && k < my_tiles; ++k) {
     // the next reverse step's grid may be scheduled once every CTA is on its last tile
     if (tid == 0 && k == my_tiles - 1) griddep_launch_dependents();
     const int t = wid + k * nworkers;
@@ -502,22 +504,18 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
       // plain read-add-write, without waiting for the read
       atomicAdd(&acc[(long long)t * 4 + tid], sum);
     }
-    if (NST == 1) {  // the only stage is free once every thread is done with it
-      __syncthreads();
-      if (tid == 0 && k + 1 < my_tiles) issue(k + 1);
-    }
     const bool ok = k + 1 >= my_tiles || mbar_wait_bounded(&bar[(k + 1) % NST], ((k + 1) / NST) & 1, WAIT_CYCLES);
-    if (__syncthreads_or(!ok)) {  // (NST = 2: also the barrier after which this stage is free)
+    if (__syncthreads_or(!ok)) {  // (also the barrier after which this stage is free)
       alive = false;
       break;
     }
-    if (NST >= 2 && tid == 0 && k + NST < my_tiles) issue(k + NST);
+    if (tid == 0 && k + NST < my_tiles) issue(k + NST);
   }
   if (!alive && tid == 0) {
     // a staged copy did not land in time: latch the error and wait (bounded) once more
     // for this CTA's copies still in flight before returning
     atomicOr(err, ERR_TIMEOUT);
-    for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
+    wind_down(min(NST + k, my_tiles), NST, [&](int s, int parity) { mbar_wait_bounded(&bar[s], parity, WAIT_CYCLES); });
   }
 }
 
@@ -586,7 +584,8 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   bool alive = true;
   const bool ey_shared = st.nrows <= 32;  // wider shells read the phase rows from global memory below
   const int ney = (FORCE && ey_shared) ? st.nrows * 8 : 0;
-  for (int k = 0; k < my_tiles; ++k) {
+  int k = 0;  // tiles finished; NST + k copies have been started when the CTA winds down
+  for (; k < my_tiles; ++k) {
     const bool ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
     if (tid == 0 && k == my_tiles - 1) griddep_launch_dependents();
     const int t = wid + k * nworkers;
@@ -789,7 +788,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   }
   if (!alive && tid == 0) {
     atomicOr(err, ERR_TIMEOUT);
-    for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
+    wind_down(NST + k, NST, [&](int s, int parity) { mbar_wait_bounded(&bar[s], parity, WAIT_CYCLES); });
   }
 }
 

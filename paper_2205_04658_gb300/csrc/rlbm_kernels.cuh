@@ -5,6 +5,7 @@
 
 #include "rlbm_device.cuh"
 #include "rlbm_launch.h"
+#include "rlbm_stages.h"
 #include "rlbm_tma.cuh"
 
 #include <climits>
@@ -473,7 +474,8 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
-  for (int k = 0; alive; ++k) {
+  int k = 0;
+  for (; alive; ++k) {
     const int s = k % NST;
     if (NST == 1) ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
     const int t = item_of[s];
@@ -522,7 +524,9 @@ step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     // a staged copy did not land in time: latch the error and wait (bounded) once more
     // for this CTA's copies still in flight before returning
     atomicOr(err, ERR_TIMEOUT);
-    for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
+    // fills so far: NST = 1 fails behind the wait for item k - 1 (the last item, of none, has no copy)
+    // and refills after it, NST = 2 has refilled at the end of k items
+    wind_down(NST == 1 ? k : NST + k, NST, [&](int s, int parity) { mbar_wait_bounded(&bar[s], parity, WAIT_CYCLES); });
   }
 }
 
@@ -644,7 +648,8 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
     ok = mbar_wait_bounded(&bar[0], 0, WAIT_CYCLES);
     if (__syncthreads_or(!ok)) alive = false;
   }
-  for (int k = 0; alive; ++k) {
+  int k = 0;
+  for (; alive; ++k) {
     const int s = k % NST;
     if (NST == 1) ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
     const TileInfo ti = info[s];
@@ -687,7 +692,8 @@ batch_step_kernel(const BatchTables bt, const Geometry<typename RealOf<S>::type>
   }
   if (!alive && tid == 0) {
     atomicOr(bt.mem[0].err, ERR_TIMEOUT);
-    for (int s2 = 0; s2 < NST; ++s2) mbar_wait_bounded(&bar[s2], 0, WAIT_CYCLES);
+    // (as in step_kernel)
+    wind_down(NST == 1 ? k : NST + k, NST, [&](int s, int parity) { mbar_wait_bounded(&bar[s], parity, WAIT_CYCLES); });
   }
   if (!alive) return;  // copies may still be in flight: stage 0 is not free
   // The stirring tables of the next step, after the tiles: chunks of rows, members in order, one
