@@ -442,7 +442,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
         Fy = mv[4];
       } else {
         m = cell_macro<R, VS>(h, M, p.vmax2);
-        if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+        if (!m.ok) atomicOr(err, cell_error(m));
       }
       // (without kappa_{n+1}, the state's force meets a zero adjoint: the body force stands in)
       cell_adjoint<R, VS, FORCE>(h, lam, M, m, p.omega0, p.fpref, Fx, Fy, cj, kap, gom, gFx, gFy);
@@ -673,7 +673,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
         Fy = T(mA[4], mB[4]);
       } else {
         m = cell_macro_pair<VS>(h, M, p.vmax2);
-        if (!m.ok) atomicOr(err, (isfinite(m.eps_m1.v.x) && isfinite(m.eps_m1.v.y)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+        if (!m.ok) atomicOr(err, cell_error(m));
         // (without kappa_{n+1}, the state's force meets a zero adjoint: the body force stands in)
       }
       cell_adjoint<T, VS, FORCE>(h, lam, M, m, T(p.omega0), T(p.fpref), Fx, Fy, T(cj), kap, gom, gFx, gFy);

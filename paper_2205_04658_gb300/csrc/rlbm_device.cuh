@@ -687,6 +687,16 @@ template <int VS> __device__ __forceinline__ bool landau_refined(const Mom<doubl
 // Macroscopic result of one cell (eps^ = eps / eps0, u^mu = gamma (1, v)).
 template <typename T> struct Macro { T eps_m1, u0, ux, uy, vx, vy; bool ok; };
 
+// What a cell without a solution (ok false) is reported as: an energy density that is not positive
+// and finite is an unstable run, else Landau matching found no timelike eigenvector.
+template <typename T> __device__ __forceinline__ unsigned cell_error(const Macro<T> &m) {
+  return T(1) + m.eps_m1 > T(0) && isfinite(m.eps_m1) ? ERR_UNPHYSICAL : ERR_UNSTABLE;
+}
+__device__ __forceinline__ unsigned cell_error(const Macro<F2> &m) {  // (of either cell)
+  const float a = m.eps_m1.v.x, b = m.eps_m1.v.y;
+  return 1.0f + a > 0.0f && isfinite(a) && 1.0f + b > 0.0f && isfinite(b) ? ERR_UNPHYSICAL : ERR_UNSTABLE;
+}
+
 template <typename T, int VS>
 __device__ __forceinline__ Macro<T> macro_from(const Mom<T> &M, int maxit, T tol) {
   Macro<T> r;

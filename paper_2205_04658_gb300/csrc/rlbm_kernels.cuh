@@ -122,7 +122,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     if (fluid) {
       const Mom<R> M = moments_of<R, R, VS, FORCE>(h);
       const Macro<R> m = cell_macro<R, VS>(h, M, p.vmax2);
-      if (!m.ok) atomicOr(err, (R(1) + m.eps_m1 > R(0) && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+      if (!m.ok) atomicOr(err, cell_error(m));
       if (macro_out) {  // the cell's Landau solution, force and streamed h, kept for the reverse sweep
         const long long nc = (long long)g.nx * g.ny, c = (long long)y * g.nx + x;
         macro_out[c] = m.eps_m1;
@@ -260,7 +260,7 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
     }
     const Mom<T> M = moments_of<T, T, VS, FORCE>(h);
     const Macro<T> m = cell_macro_pair<VS>(h, M, p.vmax2);
-    if (!m.ok) atomicOr(err, (isfinite(m.eps_m1.v.x) && isfinite(m.eps_m1.v.y)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+    if (!m.ok) atomicOr(err, cell_error(m));
     if (macro_out) {  // the cells' Landau solutions, forces and streamed h, kept for the reverse sweep
       const long long nc = (long long)g.nx * g.ny;
       if (flA) {
@@ -832,7 +832,7 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
         pull_global<S, R, VS, MASK>(fin, g, x, y + k, nb[k], h);
         const Mom<double> M = moments_of<double, R, VS, false>(h);
         const Macro<double> m = macro_from<double, VS>(M, 40, 1e-12);
-        if (!m.ok) atomicOr(err, (1.0 + m.eps_m1 > 0.0 && isfinite(m.eps_m1)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+        if (!m.ok) atomicOr(err, cell_error(m));
         e[k] = m.eps_m1; ux[k] = m.ux; uy[k] = m.uy; vx[k] = m.vx; vy[k] = m.vy;
         if (MODE == OBS_FIELDS) {
           acc[0] += eps0 * (1.0 + M.e);
@@ -847,7 +847,7 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
         pull_global_pair<S, VS, MASK>(fin, g, x, y, nb[0], nb[1], fl[0], fl[1], h);
         const Mom<F2> M = moments_of<F2, F2, VS, false>(h);
         const Macro<F2> m = cell_macro_pair<VS>(h, M, vmax2);  // (a lane without fluid matches the rest state)
-        if (!m.ok) atomicOr(err, (isfinite(m.eps_m1.v.x) && isfinite(m.eps_m1.v.y)) ? ERR_UNPHYSICAL : ERR_UNSTABLE);
+        if (!m.ok) atomicOr(err, cell_error(m));
         e[0] = m.eps_m1.v.x; e[1] = m.eps_m1.v.y;
         ux[0] = m.ux.v.x; ux[1] = m.ux.v.y; uy[0] = m.uy.v.x; uy[1] = m.uy.v.y;
         vx[0] = m.vx.v.x; vx[1] = m.vx.v.y; vy[0] = m.vy.v.x; vy[1] = m.vy.v.y;
