@@ -161,11 +161,25 @@ struct SumD {
   __device__ __forceinline__ void add(Cd z) { v += z.x * z.x + z.y * z.y; }
   __device__ __forceinline__ double value() const { return v; }
 };
+// (The square of a pair has its 48 bits in FP32's range from |z| = 2^-50 on.  FP32 deviations, hence
+// velocities, reach down to 1e-38: smaller values are squared in FP64, which a field with rounding
+// noise of FP32 never needs.)
 struct SumF {
+  static constexpr float SMALL = 0x1p-48f;
   DF2 v{F2(0.0f), F2(0.0f)};
-  __device__ __forceinline__ void add(Cf z) { const DF2 d = df_of(z); v = df_add(v, df_mul(d, d)); }
+  double small = 0.0;
+  __device__ __forceinline__ void add(Cf z) {
+    const float m = fmaxf(fabsf(z.v.x), fabsf(z.v.y));
+    if (m < SMALL && m > 0.0f) {
+      const double re = (double)z.v.x + (double)z.v.z, im = (double)z.v.y + (double)z.v.w;
+      small = fma(re, re, fma(im, im, small));
+      return;
+    }
+    const DF2 d = df_of(z);
+    v = df_add(v, df_mul(d, d));
+  }
   __device__ __forceinline__ double value() const {
-    return ((double)v.h.v.x + (double)v.h.v.y) + ((double)v.l.v.x + (double)v.l.v.y);
+    return (((double)v.h.v.x + (double)v.h.v.y) + ((double)v.l.v.x + (double)v.l.v.y)) + small;
   }
 };
 template <class C> struct SumOf;
