@@ -312,9 +312,13 @@ __device__ __forceinline__ R4<R> stir_draw_r(unsigned long long seed, long long 
 // products of parts that lie side by side, as packed multiply-adds take them.  Each lane draws
 // modes of the row (Philox is counter-based: no state is kept between steps) and every lane
 // adds all of them for its columns x0 + lane, + 32, ...; the phase is read from the table of
-// the nx roots of unity at the exact residue k_x x mod nx (a sine and cosine per mode and
-// column, as the table was built before, took three times the instructions).
-template <typename R> constexpr int stir_chunk() { return 32 * (sizeof(R) == 8 ? 4 : 8); }
+// the nx roots of unity at the exact residue k_x x mod nx.
+// A chunk is one warp's serial chain over the row's modes, up to two dozen at a shell of 6 to 12,
+// and a small lattice's step waits for it: two columns per lane in FP32 keep it short (128^2, 166
+// modes: 4.0 us per step against 5.6 with four and 7.2 with eight; 512^2 9.5, 10.4 and 12.4; 1024^2 and
+// 4096^2 within 0.5 %; one column 4.8 and 10.1, as the draws are then made twice as often).  In FP64
+// the draws are most of it, so a chunk is wider.
+template <typename R> constexpr int stir_chunk() { return 32 * (sizeof(R) == 8 ? 4 : 2); }
 
 template <typename R>
 __device__ __forceinline__ void stir_row_chunk(const StirModes &s, long long step, int r, int chunk, int nx, int lane,
