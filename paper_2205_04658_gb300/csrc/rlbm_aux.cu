@@ -491,10 +491,13 @@ cudaError_t launch_make_z(const double *ux, const double *uy, double2 *z, long l
   return cudaGetLastError();
 }
 
+// Whether a prime factor above 8 (the last radix) takes direct sums.
+static bool direct_sums(const FftPlan &p) { return p.nstages && p.radix[p.nstages - 1] > 8; }
+
 // Threads of a block that transforms `count` rows: one per radix-8 butterfly, or one per
-// output where a prime factor above 8 takes direct sums.
+// output of direct sums.
 static int fft_threads(const FftPlan &p, int count) {
-  const int work = p.nstages && p.radix[p.nstages - 1] > 8 ? p.n : p.n / 8;
+  const int work = direct_sums(p) ? p.n : p.n / 8;
   const int t = (work * count + 31) / 32 * 32;
   return t < 32 ? 32 : t > 512 ? 512 : t;
 }
@@ -519,10 +522,14 @@ static C *row_transforms(const FftPlan &p, int rows, const C *tw, C *z0, C *z1, 
 
 // Columns of a strip: as wide as shared memory and the number of SMs allow, down to two
 // columns (32 bytes, a whole sector of each row); 0 = the columns go through a transpose.
-// Strips of 4 columns fill the chip from 608 columns on and read 64-byte pieces.
-static int strip_columns(int nx, int ny) {
-  const int fit = FFT_SMEM / (2 * fft_padded(ny) * (int)sizeof(Cd));
+// Strips of 4 columns fill the chip from 608 columns on and read 64-byte pieces.  Lengths with a
+// prime factor above 8 are bound by the direct sums of that factor, not by the reads: there one
+// column to a strip shares the work over the most SMs (FP64, 64 columns of 2039: 22.7 ms in
+// strips of two, on 32 SMs).
+static int strip_columns(int nx, const FftPlan &py) {
+  const int fit = FFT_SMEM / (2 * fft_padded(py.n) * (int)sizeof(Cd));
   if (fit < 2) return 0;
+  if (direct_sums(py)) return 1;
   return fit >= 4 && nx >= 4 * 152 ? 4 : 2;
 }
 
@@ -571,8 +578,8 @@ static cudaError_t band_energy_t(int nx, int ny, const C *twx, const C *twy, C *
                                  double *partials, double *out4, unsigned *sync, cudaStream_t st) {
   const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
   cudaError_t e = cudaSuccess;
-  if (const int nc = strip_columns(nx, ny)) {
-    const FftPlan py = make_plan(ny);
+  const FftPlan py = make_plan(ny);
+  if (const int nc = strip_columns(nx, py)) {
     const int smem = 2 * nc * fft_padded(ny) * (int)sizeof(C);
     if ((e = fft_allow_smem(fft_cols_kernel<C, false>, smem)) != cudaSuccess) return e;
     C *Z = row_transforms(make_plan(nx), ny, twx, z0, z1, st, e);
@@ -593,8 +600,8 @@ static cudaError_t spectrum_t(int nx, int ny, const C *twx, const C *twy, C *z0,
                               cudaStream_t st) {
   const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
   cudaError_t e = cudaSuccess;
-  if (const int nc = strip_columns(nx, ny)) {
-    const FftPlan py = make_plan(ny);
+  const FftPlan py = make_plan(ny);
+  if (const int nc = strip_columns(nx, py)) {
     const int smem = 2 * nc * fft_padded(ny) * (int)sizeof(C);
     if ((e = fft_allow_smem(fft_cols_kernel<C, true>, smem)) != cudaSuccess) return e;
     C *Z = row_transforms(make_plan(nx), ny, twx, z0, z1, st, e);
