@@ -191,9 +191,10 @@ RLBM_API rlbm_status rlbm_set_launch(rlbm_ctx *ctx, int32_t ctas, int32_t stages
 
 /* Autotuner: times every launch shape it knows (pipeline depth x CTA count x stirring
  * rows staged or read from global memory), `reps` launches each, chained as rlbm_step
- * chains consecutive steps, on the current state, and keeps the fastest.  The state and the step
- * counter are left as they were (the launches rewrite the next buffer only).  *ms_out
- * (may be NULL) receives the chosen shape's time per step in milliseconds.  Syncs.
+ * chains consecutive steps and of alternating parity, on the current state, and keeps the
+ * fastest; with that, the pipeline depth of steps launched by themselves.  The state and the
+ * step counter are left as they were (the launches rewrite the next buffer only).  *ms_out
+ * (may be NULL) receives the chosen shape's time per chained step in milliseconds.  Syncs.
  * The paper has no counterpart. */
 RLBM_API rlbm_status rlbm_autotune(rlbm_ctx *ctx, int32_t reps, double *ms_out);
 

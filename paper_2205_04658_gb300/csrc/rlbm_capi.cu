@@ -18,6 +18,7 @@
 #include "../../include/rlbm.h"
 #include "rlbm_device.cuh"
 #include "rlbm_launch.h"
+#include "rlbm_tune.h"
 
 using namespace rlbm;
 
@@ -217,6 +218,14 @@ struct rlbm_ctx {
   std::vector<uint8_t> host_stage, host_small;
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
+
+  LaunchShape shape() const { return LaunchShape{grid_limit, chained_stages, stages, stir_rows}; }
+  void use(const LaunchShape &s) {
+    grid_limit = s.grid;
+    chained_stages = s.chained_stages;
+    stages = s.stages;
+    stir_rows = s.rows;
+  }
 
   rlbm_status fail(rlbm_status s, const std::string &m) {
     msg = m;
@@ -431,6 +440,30 @@ cudaError_t stir_tables(rlbm_ctx *c, int64_t n, int count, void *G, size_t table
 
 // The table of step n (each step's launch builds the next one's).
 cudaError_t stir_prime(rlbm_ctx *c, int64_t n) { return stir_tables(c, n, 1, c->ws + c->L.G[n & 1], 0); }
+
+// The trial steps of rlbm_autotune (tune_shape): the step kernel reads the current buffer and writes the
+// other one, so repeating it leaves the state (and the step counter) as it was.  The parity goes to
+// the kernel as the step's number; the stirring tables stay those of the current step.
+struct Tuner {
+  rlbm_ctx *c;
+  HostStir stir;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  cudaError_t err = cudaSuccess;
+  bool step(const LaunchShape &s, bool odd, bool chained) {
+    c->use(s);
+    const int64_t at = c->phys.step;
+    c->phys.step = (c->step & ~int64_t(1)) + (odd ? 1 : 0);
+    err = dispatch_step(c, c->cur, stir, chained);
+    c->phys.step = at;
+    return err == cudaSuccess;
+  }
+  bool start() { return (err = cudaEventRecord(e0, c->stream)) == cudaSuccess; }
+  bool stop(float &ms) {
+    if ((err = cudaEventRecord(e1, c->stream)) == cudaSuccess && (err = cudaEventSynchronize(e1)) == cudaSuccess)
+      err = cudaEventElapsedTime(&ms, e0, e1);
+    return err == cudaSuccess;
+  }
+};
 
 // Waits for the stream, reads the device error word and latches it.  The word comes in one
 // copy with the small results behind it (up to byte offset `end` of the workspace), which the
@@ -934,51 +967,21 @@ rlbm_status rlbm_autotune(rlbm_ctx *c, int32_t reps, double *ms_out) {
   if (rlbm_status s = usable(c)) return s;
   if (reps < 1) return c->fail(RLBM_E_INVAL, "reps must be >= 1");
   Scoped dev(c->device);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  // candidate launch shapes: pipeline depth x persistent CTA count (0 = all resident) x
-  // where the stirring rows come from (staged with each tile, or global memory)
-  const int stage_opts[2] = {2, 1};
-  const int grid_opts[4] = {0, 2 * sms, 3 * sms, 4 * sms};
-  const int rows_opts[2] = {1, 2};
+  // persistent CTA counts (0 = all resident) to try with each pipeline depth and source of the stirring
+  // rows (staged with each tile, or global memory)
+  const int grids[4] = {0, 2 * c->sms, 3 * c->sms, 4 * c->sms};
   const int nrows_opts = (c->L.nrows > 0 && c->L.nrows <= 16) ? 2 : 1;
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-    return c->fail(RLBM_E_CUDA, "cudaEventCreate failed");
-  const int save_grid = c->grid_limit, save_stages = c->stages, save_chained = c->chained_stages, save_rows = c->stir_rows;
-  float best = 1e30f;
-  int best_grid = save_grid, best_stages = save_stages, best_rows = save_rows;
-  const HostStir st = stir_for_step(c, c->step);
-  cudaError_t e = cudaSuccess;
-  for (int ri = 0; ri < nrows_opts && e == cudaSuccess; ++ri)
-    for (int si = 0; si < 2 && e == cudaSuccess; ++si)
-      for (int gi = 0; gi < 4 && e == cudaSuccess; ++gi) {
-        c->stir_rows = rows_opts[ri];
-        c->stages = c->chained_stages = stage_opts[si];
-        c->grid_limit = grid_opts[gi];
-        // the step kernel reads the current buffer and writes the other one; repeating it
-        // leaves the state (and the step counter) as it was.  The repetitions are chained as
-        // rlbm_step chains consecutive steps (programmatic dependent launch), so the shape is
-        // chosen for the way the steps run.
-        if ((e = dispatch_step(c, c->cur, st)) != cudaSuccess) break;  // warm-up
-        cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = dispatch_step(c, c->cur, st, r > 0);
-        cudaEventRecord(e1, c->stream);
-        if (e != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess) break;
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best) { best = ms; best_grid = c->grid_limit; best_stages = c->stages; best_rows = c->stir_rows; }
-      }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  c->grid_limit = best_grid;
-  c->stages = c->chained_stages = best_stages;
-  c->stir_rows = best_rows;
-  if (e != cudaSuccess) {
-    c->grid_limit = save_grid; c->stages = save_stages; c->chained_stages = save_chained; c->stir_rows = save_rows;
-    return c->cuda_fail(e, "autotune launch");
-  }
-  if (ms_out) *ms_out = best / reps;
+  const LaunchShape saved = c->shape();
+  Tuner gpu{c, stir_for_step(c, c->step)};
+  if ((gpu.err = cudaEventCreate(&gpu.e0)) == cudaSuccess) gpu.err = cudaEventCreate(&gpu.e1);
+  LaunchShape best = saved;
+  float ms = 0.0f;
+  const bool done = gpu.err == cudaSuccess && tune_shape(gpu, grids, 4, nrows_opts, reps, best, ms);
+  if (gpu.e0) cudaEventDestroy(gpu.e0);
+  if (gpu.e1) cudaEventDestroy(gpu.e1);
+  c->use(done ? best : saved);
+  if (!done) return c->cuda_fail(gpu.err, "autotune");
+  if (ms_out) *ms_out = ms;
   return check_device(c);
 }
 
