@@ -315,8 +315,10 @@ __device__ __forceinline__ R4<R> stir_draw_r(unsigned long long seed, long long 
 // the nx roots of unity at the exact residue k_x x mod nx.
 // A chunk is one warp's serial chain over the row's modes, up to two dozen at a shell of 6 to 12,
 // and a small lattice's step waits for it: two columns per lane in FP32 keep it short (128^2, 166
-// modes: 4.0 us per step against 5.6 with four and 7.2 with eight; 512^2 9.5, 10.4 and 12.4; 1024^2 and
-// 4096^2 within 0.5 %; one column 4.8 and 10.1, as the draws are then made twice as often).  In FP64
+// modes: 5.1 us per step against 7.2 with eight; 512^2 10.0 against 12.2; 1024^2 and 4096^2 alike; one
+// column: the draws are then made twice as often).  The loop over the modes is not unrolled: copies
+// of its body take 1 us more off those two, but cost masked FP32 lattices, whose body force
+// compiles the same kernel without running the loop, 6 % (1024 x 256: 9.1 us against 8.5).  In FP64
 // the draws are most of it, so a chunk is wider.
 template <typename R> constexpr int stir_chunk() { return 32 * (sizeof(R) == 8 ? 4 : 2); }
 
@@ -340,6 +342,7 @@ __device__ __forceinline__ void stir_row_chunk(const StirModes &s, long long ste
     int d = (32 * kx) % nx;
     if (d < 0) d += nx;
     const int cnt = m1 - m0 < 32 ? m1 - m0 : 32;
+#pragma unroll 1
     for (int k = 0; k < cnt; ++k) {
       const R4<R> a{__shfl_sync(0xffffffffu, c.x, k), __shfl_sync(0xffffffffu, c.y, k),
                     __shfl_sync(0xffffffffu, c.z, k), __shfl_sync(0xffffffffu, c.w, k)};

@@ -42,7 +42,7 @@ def test_rows_at_the_edges_of_chunks(R, nx, precision, tol):
 
 def test_a_shell_of_many_modes_does_not_set_the_step_time(R):
     """128^2: building the rows of 166 modes hides behind the step's other work, as that of 20 modes
-    does (3.7 and 4.0 us per step; 3.9 and 7.2 with chunks of 256 columns)."""
+    does (3.7 and 5.1 us per step; 4.0 and 7.1 with chunks of 256 columns)."""
     import torch
     stream = torch.cuda.Stream()
     us = {}
