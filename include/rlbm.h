@@ -293,7 +293,9 @@ RLBM_API rlbm_status rlbm_batch_query_workspace(int32_t nmembers, size_t *bytes)
 RLBM_API rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *dev_workspace,
                                      size_t bytes, void *cuda_stream, rlbm_batch **out);
 
-/* Launch shape of the batched step kernel (as rlbm_set_launch). */
+/* Launch shape of the batched step kernel (as rlbm_set_launch).  A batch starts with the
+ * `stages` that were set (rlbm_set_launch) or tuned (rlbm_autotune) on members[0] before
+ * rlbm_batch_init, else with a default by storage and mask. */
 RLBM_API rlbm_status rlbm_batch_set_launch(rlbm_batch *b, int32_t ctas, int32_t stages);
 
 /* Autotuner of the batched launch: times every launch shape it knows (pipeline depth x

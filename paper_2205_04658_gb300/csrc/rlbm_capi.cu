@@ -210,6 +210,7 @@ struct rlbm_ctx {
   int sms = 0;                 // multiprocessors of the device
   int grid_limit = 0;          // step kernel: 0 = one wave of resident CTAs
   int stages = 1, chained_stages = 1;  // shared-memory pipeline depth of the step kernel (1 or 2)
+  bool own_stages = false;     // the depth was set or tuned (else rlbm_init's choice)
   int stir_rows = 1;           // stirring rows: 1 = staged with each tile, 2 = read from global memory
   unsigned launch_seq = 0;     // step-kernel launches so far (selects the tile counter)
   int halo_faces = 0;          // a strip: faces whose ghost rows come from neighbours (bit 0 below, 1 above)
@@ -957,7 +958,10 @@ rlbm_status rlbm_set_launch(rlbm_ctx *c, int32_t ctas, int32_t stages, int32_t s
   if (ctas < 0 || stages < 0 || stages > 2 || stir_rows < 0 || stir_rows > 2)
     return c->fail(RLBM_E_INVAL, "ctas must be >= 0, stages 0, 1 or 2 and stir_rows 0, 1 or 2");
   c->grid_limit = ctas;
-  if (stages) c->stages = c->chained_stages = stages;
+  if (stages) {
+    c->stages = c->chained_stages = stages;
+    c->own_stages = true;
+  }
   if (stir_rows) c->stir_rows = stir_rows;
   return RLBM_OK;
 }
@@ -981,6 +985,7 @@ rlbm_status rlbm_autotune(rlbm_ctx *c, int32_t reps, double *ms_out) {
   if (gpu.e1) cudaEventDestroy(gpu.e1);
   c->use(done ? best : saved);
   if (!done) return c->cuda_fail(gpu.err, "autotune");
+  c->own_stages = true;
   if (ms_out) *ms_out = ms;
   return check_device(c);
 }
@@ -1160,6 +1165,7 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
   // (16 x 512^2, us per step with one stage and with two: FP32 108 and 119, FP16 96 and 105, with masks
   // FP16 96 and 105, but FP32 114 and 105)
   b->stages = b->mask && members[0]->cfg.precision == RLBM_F32 ? 2 : 1;
+  if (members[0]->own_stages) b->stages = members[0]->chained_stages;  // a depth set or tuned on the members stays
   b->ntiles = tile0[nmembers];
   Scoped dev(b->device);
   cudaError_t e;
