@@ -276,8 +276,9 @@ RLBM_API rlbm_status rlbm_halo_unpack(rlbm_ctx *ctx, int32_t face, const void *d
  * whole chunks of steps replay a captured CUDA graph.
  * Members are ordinary contexts (rlbm_init) that share the velocity set, storage type,
  * a, dt, eta/s, eps0, body force, stirring shell and amplitude, rounding and
- * fp64_landau_vmax; they may differ in size, walls, solids, seeds and initial fields,
- * and in their current step.  After rlbm_batch_step every member has advanced by nsteps
+ * fp64_landau_vmax; they may differ in size, walls, solids, seeds, stirring multipliers
+ * (rlbm_set_mode_scale) and initial fields, and in their current step.  After
+ * rlbm_batch_step every member has advanced by nsteps
  * (rlbm_current_step, rlbm_moments ... work on it as usual); work of the batch is queued
  * on the batch's stream, so give the members the same stream or synchronise.  Graphs are
  * used on a non-default stream only.  The paper has no counterpart (its runs were one
