@@ -471,8 +471,8 @@ struct Tuner {
 // caller then finds through small(c, offset): a synchronisation, a copy of the results and a
 // copy of the word were three round trips of some 10 us each.
 rlbm_status check_device(rlbm_ctx *c, size_t end = 0) {
-  c->host_small.resize(std::max(end, c->L.err + sizeof(unsigned)) - c->L.err);
-  cudaError_t e = cudaMemcpyAsync(c->host_small.data(), c->ws + c->L.err, c->host_small.size(), cudaMemcpyDeviceToHost, c->stream);
+  const size_t bytes = std::max(end, c->L.err + sizeof(unsigned)) - c->L.err;  // (host_small holds all of them)
+  cudaError_t e = cudaMemcpyAsync(c->host_small.data(), c->ws + c->L.err, bytes, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "copy of the error word");
   unsigned w = 0;
@@ -584,6 +584,13 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   if (c->cfg.fp64_landau_vmax == 0.0) c->cfg.fp64_landau_vmax = 0.5;
 
   auto bail = [&](rlbm_status s) { g_thread_error = c->msg; delete c; return s; };
+  // (here, so that no later call allocates for it: an exception must not leave a C entry point)
+  try {
+    c->host_small.resize(L.bins + 8 * (size_t)L.max_bins - L.err);
+  } catch (const std::bad_alloc &) {
+    c->msg = "host allocation failed";
+    return bail(RLBM_E_NOMEM);
+  }
   auto put = [&](size_t off, const void *src, size_t n) -> cudaError_t {
     if (n == 0) return cudaSuccess;
     return cudaMemcpyAsync(c->ws + off, src, n, cudaMemcpyHostToDevice, c->stream);
