@@ -161,25 +161,13 @@ struct SumD {
   __device__ __forceinline__ void add(Cd z) { v += z.x * z.x + z.y * z.y; }
   __device__ __forceinline__ double value() const { return v; }
 };
-// (The square of a pair has its 48 bits in FP32's range from |z| = 2^-50 on.  FP32 deviations, hence
-// velocities, reach down to 1e-38: smaller values are squared in FP64, which a field with rounding
-// noise of FP32 never needs.)
+// (The square of a pair has its 48 bits in FP32's range from |z| = 2^-50 on, while FP32 velocities reach
+// down to 1e-38: pairs are transformed scaled by spectrum_scale.)
 struct SumF {
-  static constexpr float SMALL = 0x1p-48f;
   DF2 v{F2(0.0f), F2(0.0f)};
-  double small = 0.0;
-  __device__ __forceinline__ void add(Cf z) {
-    const float m = fmaxf(fabsf(z.v.x), fabsf(z.v.y));
-    if (m < SMALL && m > 0.0f) {
-      const double re = (double)z.v.x + (double)z.v.z, im = (double)z.v.y + (double)z.v.w;
-      small = fma(re, re, fma(im, im, small));
-      return;
-    }
-    const DF2 d = df_of(z);
-    v = df_add(v, df_mul(d, d));
-  }
+  __device__ __forceinline__ void add(Cf z) { const DF2 d = df_of(z); v = df_add(v, df_mul(d, d)); }
   __device__ __forceinline__ double value() const {
-    return (((double)v.h.v.x + (double)v.h.v.y) + ((double)v.l.v.x + (double)v.l.v.y)) + small;
+    return ((double)v.h.v.x + (double)v.h.v.y) + ((double)v.l.v.x + (double)v.l.v.y);
   }
 };
 template <class C> struct SumOf;
@@ -573,10 +561,16 @@ __global__ void band_kernel(const C *__restrict__ Z, int nx, int ny, long long k
   }
 }
 
+// 1/2 / (nx ny)^2 of the energies, with the scale of the velocities undone.
+template <class C> static double energy_scale(int nx, int ny) {
+  const double s = std::is_same<C, Cd>::value ? 1.0 : (double)spectrum_scale((long long)nx * ny);
+  return 0.5 / ((double)nx * ny * (double)nx * ny) / (s * s);
+}
+
 template <class C>
 static cudaError_t band_energy_t(int nx, int ny, const C *twx, const C *twy, C *z0, C *z1, long long k2lo, long long k2hi,
                                  double *partials, double *out4, unsigned *sync, cudaStream_t st) {
-  const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
+  const double scale = energy_scale<C>(nx, ny);
   cudaError_t e = cudaSuccess;
   const FftPlan py = make_plan(ny);
   if (const int nc = strip_columns(nx, py)) {
@@ -598,7 +592,7 @@ static cudaError_t band_energy_t(int nx, int ny, const C *twx, const C *twy, C *
 template <class C>
 static cudaError_t spectrum_t(int nx, int ny, const C *twx, const C *twy, C *z0, C *z1, double *bins, int nbins,
                               cudaStream_t st) {
-  const double scale = 0.5 / ((double)nx * ny * (double)nx * ny);
+  const double scale = energy_scale<C>(nx, ny);
   cudaError_t e = cudaSuccess;
   const FftPlan py = make_plan(ny);
   if (const int nc = strip_columns(nx, py)) {

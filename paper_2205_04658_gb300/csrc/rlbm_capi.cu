@@ -385,6 +385,7 @@ cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = 
   o.partials = c->at<double>(c->L.partials);
   o.totals = mode == 2 ? c->at<double>(c->L.cols) : c->at<double>(c->L.totals);
   o.sync = c->at<unsigned>(c->L.sync);
+  o.zscale = spectrum_scale((long long)c->cfg.nx * c->cfg.ny);
   o.bins = c->at<double>(c->L.bins);
   o.nbins = nbins;
   unsigned *err = c->at<unsigned>(c->L.err);

@@ -779,14 +779,15 @@ __device__ __forceinline__ void pull_global_pair(const S *__restrict__ fin, cons
 
 struct ObsOut {
   double *eps, *ux, *uy;  // OBS_FIELDS (each may be NULL)
-  double2 *z;             // OBS_V (FP32 states: float4 v_x, v_y, 0, 0: high and low parts); OBS_COLS: the
-                          // blocks' partial column sums (the same two forms)
+  double2 *z;             // OBS_V (FP32 states: float4 v_x, v_y, 0, 0, high and low parts, times zscale);
+                          // OBS_COLS: the blocks' partial column sums (the same two forms)
   double *partials;       // [blocks][4]
   double *totals;         // [4]; OBS_COLS: [2 nx]
   unsigned *sync;         // zeroed counters of finished blocks: 1, or one per tile column (OBS_COLS)
   double *bins;           // OBS_V: nbins values cleared for the spectrum's sums
   int nbins;
 };
+  float zscale;           // OBS_V, FP32 states: the factor of z
 
 template <typename S, int VS, bool MASK, int MODE>
 __global__ void __launch_bounds__(256)
@@ -945,7 +946,7 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
       } else if constexpr (F64) {
         out.z[c] = make_double2(vx[k], vy[k]);
       } else {
-        reinterpret_cast<float4 *>(out.z)[c] = make_float4(vx[k], vy[k], 0.0f, 0.0f);
+        reinterpret_cast<float4 *>(out.z)[c] = make_float4(out.zscale * vx[k], out.zscale * vy[k], 0.0f, 0.0f);
       }
     }
   }
@@ -1314,7 +1315,7 @@ static cudaError_t launch_observe_t(int vset, int mode, const void *fin, const H
                                     const HostObs &ho, unsigned *err, int sms, cudaStream_t stream) {
   using R = typename RealOf<S>::type;
   const Geometry<R> g = to_geom<S>(hg);
-  const ObsOut o{ho.eps, ho.ux, ho.uy, ho.z, ho.partials, ho.totals, ho.sync, ho.bins, ho.nbins};
+  const ObsOut o{ho.eps, ho.ux, ho.uy, ho.z, ho.partials, ho.totals, ho.sync, ho.bins, ho.nbins, ho.zscale};
   const bool mask = hg.nbmask != nullptr;
   const S *a = (const S *)fin;
   if (vset == 3) {

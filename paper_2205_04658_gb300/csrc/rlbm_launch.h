@@ -55,7 +55,17 @@ struct HostObs {
   unsigned *sync;
   double *bins;  // mode 1: nbins values cleared for the spectrum
   int nbins;
+  float zscale;  // mode 1, FP32 states: the factor of z (spectrum_scale)
 };
+
+// The power of two that FP32 velocities are scaled by for their transform (an exact product): the
+// largest for which sum |Z|^2 <= (nx ny)^2 max |v|^2 stays below 2^126, so that the squares of all
+// velocities of FP32's normal range count.
+inline float spectrum_scale(long long ncell) {
+  float s = 0x1p63f;
+  for (long long n = 1; n < ncell; n *= 2) s *= 0.5f;
+  return s;
+}
 
 // One lattice of a batch, as the batched step kernel sees it (device memory, written by
 // the host before the launches; 128-byte aligned so its tensor maps are 64-byte aligned).
@@ -165,7 +175,8 @@ cudaError_t launch_reduce_partials(const double *partials, long long nblocks, do
 // The velocity field z = v_x + i v_y (interleaved, [y][x]) of caller-provided u^x, u^y.
 cudaError_t launch_make_z(const double *ux, const double *uy, double2 *z, long long ncell, cudaStream_t st);
 // Spectrum and band energy of z0; both buffers hold nx * ny complex numbers of 16 bytes and are
-// overwritten.  f64: (re, im) in FP64; else high and low FP32 parts (re_h, im_h, re_l, im_l).
+// overwritten.  f64: (re, im) in FP64; else high and low FP32 parts (re_h, im_h, re_l, im_l) of the
+// velocities times spectrum_scale(nx * ny).
 // twx, twy: exp(-2 pi i t / n) in the same form.
 cudaError_t launch_band_energy(bool f64, int nx, int ny, const void *twx, const void *twy, void *z0, void *z1, long long k2lo,
                                long long k2hi, double *partials, double *out4, unsigned *sync, cudaStream_t st);
