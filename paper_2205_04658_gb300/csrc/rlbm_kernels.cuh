@@ -786,8 +786,8 @@ struct ObsOut {
   unsigned *sync;         // zeroed counters of finished blocks: 1, or one per tile column (OBS_COLS)
   double *bins;           // OBS_V: nbins values cleared for the spectrum's sums
   int nbins;
-};
   float zscale;           // OBS_V, FP32 states: the factor of z
+};
 
 template <typename S, int VS, bool MASK, int MODE>
 __global__ void __launch_bounds__(256)
