@@ -489,7 +489,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
       }
     }
     // tile sums (fixed order) added to this tile's accumulators: warp sums in the compute
-    // type (GB300's FP64 rate is 1/64 of FP32), the eight warp sums in FP64
+    // type (GB300's FP64 rate is 1/64 of FP32), the four warp sums in FP64
     R v[4] = {gom, gFx, gFy, jv};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -526,7 +526,7 @@ adjoint_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ C
 // One stage per CTA and four CTAs per SM (128 registers): the other CTAs' tiles hide a tile's copy,
 // and the 512^2 lattice takes 2 rounds instead of 3 (gradient of 200 steps 8.27 ms; three CTAs of
 // two stages 8.41, of one 8.56, five CTAs 9.00).
-template <int VS, bool MASK, bool FORCE, bool LAM, int NST>
+template <int VS, bool MASK, bool FORCE, bool LAM>
 __global__ void __launch_bounds__(128, 4)
 adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constant__ CUtensorMap tK,
                     float *__restrict__ kout, const Geometry<float> g, const Physics<float> p,
@@ -541,7 +541,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   constexpr int NT = 128;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + NST * STAGE);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + STAGE);
   __shared__ R2<float> sF[8][32];
   __shared__ __align__(16) R2<float> sE[32][8];  // the tile's phase rows EY_r(y0 + j) of the projections
   __shared__ double red[4][4];
@@ -551,48 +551,34 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   const int my_tiles = wid < ntiles ? (ntiles - 1 - wid) / nworkers + 1 : 0;
   const uint32_t stage_bytes = TL::IN_BYTES;
   if (tid == 0) {
-    for (int s2 = 0; s2 < NST; ++s2) mbar_init(&bar[s2], 1);
+    mbar_init(bar, 1);
     fence_mbar_init();
   }
   __syncthreads();
-  auto issue_B = [&](int k) {
-    if (LAM) return;
+  auto issue = [&](int k) {
     const int t = wid + k * nworkers;
     const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TL::TY;
-    uint64_t *b = &bar[k % NST];
-    mbar_expect_tx(b, stage_bytes);
-    tma_load_3d(smem + (k % NST) * STAGE, &tB, b, x0 + TL::XOFF - TL::V, y0, 0);
+    mbar_expect_tx(bar, stage_bytes);
+    tma_load_3d(smem, LAM ? &tK : &tB, bar, x0 + TL::XOFF - TL::V, y0, 0);
   };
-  auto issue_K = [&](int k) {
-    if (!LAM) return;
-    const int t = wid + k * nworkers;
-    const int x0 = (t % ntx) * TILE_X, y0 = (t / ntx) * TL::TY;
-    uint64_t *b = &bar[k % NST];
-    mbar_expect_tx(b, stage_bytes);
-    tma_load_3d(smem + (k % NST) * STAGE, &tK, b, x0 + TL::XOFF - TL::V, y0, 0);
-  };
-  auto issue = [&](int k) { issue_B(k); issue_K(k); };
-  if (tid == 0)
-    for (int k = 0; k < NST && k < my_tiles; ++k) issue_B(k);
+  // (B_{n-1} before the wait, kappa_{n+1} behind it, as in adjoint_kernel)
+  if (!LAM && tid == 0 && my_tiles > 0) issue(0);
   griddep_wait();
-  if (tid == 0)
-    for (int k = 0; k < NST && k < my_tiles; ++k) issue_K(k);
+  if (LAM && tid == 0 && my_tiles > 0) issue(0);
   // Every wait is bounded, and the barrier after the pull carries a vote: the whole CTA winds down
   // together if a copy never lands.  With that barrier every thread has read the tile, and the
   // next one's copy starts behind the rest of this one's work (a gradient at 512^2: 8.03 -> 7.86 ms).
-  static_assert(NST == 1, "the stage is refilled after the pull");
   bool alive = true;
   const bool ey_shared = st.nrows <= 32;  // wider shells read the phase rows from global memory below
   const int ney = (FORCE && ey_shared) ? st.nrows * 8 : 0;
-  int k = 0;  // tiles finished; NST + k copies have been started when the CTA winds down
+  int k = 0;  // tiles finished; k + 1 copies have been started when the CTA winds down
   for (; k < my_tiles; ++k) {
-    const bool ok = mbar_wait_bounded(&bar[0], k & 1, WAIT_CYCLES);
+    const bool ok = mbar_wait_bounded(bar, k & 1, WAIT_CYCLES);
     if (tid == 0 && k == my_tiles - 1) griddep_launch_dependents();
     const int t = wid + k * nworkers;
     const int tx = t % ntx, ty = t / ntx;
     const int x = tx * TILE_X + lx, yA = ty * TL::TY + 2 * ly, yB = yA + 1;
-    const float *tileB = reinterpret_cast<const float *>(smem + (k % NST) * STAGE);  // without LAM
-    const float *tileK = reinterpret_cast<const float *>(smem + (k % NST) * STAGE);  // LAM
+    const float *tile = reinterpret_cast<const float *>(smem);  // of kappa_{n+1} (LAM) or B_{n-1}
     const int b0 = (2 * ly + 1) * TL::TXB + lx + TL::V;
     const bool inA = x < g.nx && yA < g.ny, inB = x < g.nx && yB < g.ny;
     unsigned nbA = 0, nbB = 0;
@@ -634,9 +620,9 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
       }
 #pragma unroll
       for (int q = 0; q < Q; ++q) h[q] = T(hA[q], hB[q]);
-      pull_staged_pair<VS, MASK, 1>(tileK, PL, TL::TXB, b0, DB, g, nbA, nbB, lam);
+      pull_staged_pair<VS, MASK, 1>(tile, PL, TL::TXB, b0, DB, g, nbA, nbB, lam);
     } else {
-      pull_staged_pair<VS, MASK, -1>(tileB, PL, TL::TXB, b0, DB, g, nbA, nbB, h);
+      pull_staged_pair<VS, MASK, -1>(tile, PL, TL::TXB, b0, DB, g, nbA, nbB, h);
 #pragma unroll
       for (int q = 0; q < Q; ++q) lam[q] = T(0.0f);
     }
@@ -788,7 +774,7 @@ adjoint_pair_kernel(const __grid_constant__ CUtensorMap tB, const __grid_constan
   }
   if (!alive && tid == 0) {
     atomicOr(err, ERR_TIMEOUT);
-    wind_down(NST + k, NST, [&](int s, int parity) { mbar_wait_bounded(&bar[s], parity, WAIT_CYCLES); });
+    wind_down(1 + k, 1, [&](int, int parity) { mbar_wait_bounded(bar, parity, WAIT_CYCLES); });
   }
 }
 
@@ -917,7 +903,7 @@ __global__ void adj_twiddle_kernel(double2 *tw, float2 *twf, int n) {
 // The reverse-step kernel of a storage type (same parameters for both forms).
 template <typename S, int VS, bool MASK, bool FORCE, bool LAM, int NST>
 static auto pick_adjoint_kernel() {
-  if constexpr (sizeof(S) == 4) return adjoint_pair_kernel<VS, MASK, FORCE, LAM, NST>;
+  if constexpr (sizeof(S) == 4) return adjoint_pair_kernel<VS, MASK, FORCE, LAM>;
   else return adjoint_kernel<S, VS, MASK, FORCE, LAM, NST>;
 }
 

@@ -411,7 +411,6 @@ HostStir stir_for_step(rlbm_ctx *c, int64_t n) {
   HostStir s{};
   const Layout &L = c->L;
   s.nrows = L.nrows;
-  s.nmodes = L.nmodes;
   if (L.nmodes == 0) return s;
   s.G_cur = c->ws + L.G[n & 1];
   s.G_next = c->ws + L.G[(n + 1) & 1];

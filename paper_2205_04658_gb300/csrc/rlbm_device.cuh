@@ -379,7 +379,8 @@ template <typename R> __device__ __forceinline__ R2<R> ey_at(const R *row, int y
 }
 
 // ---------------------------------------------------------------------------
-// Arithmetic helpers: exact in FP64, hardware approximations (<= 2 ulp) in FP32.
+// Arithmetic helpers: correctly rounded or within an ulp or two in FP64, hardware approximations
+// (<= 2 ulp) in FP32.
 // ---------------------------------------------------------------------------
 template <typename T> struct FM;
 // FP64 roots by Newton's method from the FP32 approximation (1e-7), two steps (1e-14, rounding):
@@ -494,9 +495,6 @@ __device__ __forceinline__ DF2 df_mul(const DF2 &a, const DF2 &b) {
   const F2 p = a.h * b.h;
   return df_norm(p, fma(a.l, b.h, fma(a.h, b.l, fma(a.h, b.h, -p))));
 }
-// the two lanes exchanged
-__device__ __forceinline__ F2 swap(F2 a) { return F2(a.v.y, a.v.x); }
-__device__ __forceinline__ DF2 swap(const DF2 &a) { return DF2{swap(a.h), swap(a.l)}; }
 __device__ __forceinline__ F2 shfl_xor(F2 a, int off) {
   return F2(__shfl_xor_sync(0xffffffffu, a.v.x, off), __shfl_xor_sync(0xffffffffu, a.v.y, off));
 }
@@ -645,9 +643,10 @@ __device__ __forceinline__ bool landau(const Mom<T> &M, int maxit, T tol, T &vx,
     d2 = dx * dx + dy * dy;
     if constexpr (sizeof(T) == 8) {
       // Newton converges quadratically: after a step of |dv| = 1e-12 |v| the error is at rounding.
-      // (A limit at the rounding itself, |dv| = 1e-16 |v|, is missed by the noise of the residual,
-      // and whole warps then ran all 40 steps on the FP64 units, 1/64 of FP32's rate: 200 steps of
-      // a 64^2 lattice took 26.5-31.4 ms and take 5.4 ms.)
+      // (A limit at the rounding itself, |dv| = 1e-16 |v|, is missed by the noise of the residual, and
+      // whole warps run all 40 steps on the FP64 units, 1/64 of FP32's rate: 200 steps of a 64^2
+      // lattice, all by this path, 5.4 ms against 26.5-31.4.  Cells that landau_refined solves
+      // do not come here.)
       if (d2 <= 1e-24 * (vx * vx + vy * vy) + 1e-300) break;
     } else {
       if (d2 <= tol * tol * (T(1e-6) + vx * vx + vy * vy)) break;

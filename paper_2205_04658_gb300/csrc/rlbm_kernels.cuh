@@ -25,9 +25,9 @@ __device__ __forceinline__ int ghost_row(int y, int ny, int walls) {
 }
 constexpr long long WAIT_CYCLES = 4000000000ll;  // ~2 s at 2 GHz: bounded TMA waits
 
-// Bytes of the two buffers from which odd steps walk the lattice backwards (step_kernel).  The line lies
-// between 724^2 FP32 (71 MB: no effect; 512^2 lost 4 %) and 896^2 (109 MB: 22.7 -> 21.5 us per step);
-// 1024^2 (142 MB) 29.1 -> 28.0, 4096^2 and FP16 within 1 %.
+// Bytes of the two buffers, ghosts and padding included, from which odd steps walk the lattice backwards
+// (step_kernel).  The line lies between 724^2 FP32 (76 MB: no effect; 512^2, 40 MB, lost 4 %) and 896^2
+// (117 MB: 22.7 -> 21.5 us per step); 1024^2 (152 MB) 29.1 -> 28.0, 4096^2 and FP16 within 1 %.
 constexpr long long BACKWARDS_BYTES = 90000000ll;
 
 template <typename S, int VS> struct Tile {
@@ -367,10 +367,11 @@ tile_cells(const unsigned char *stg, int ey_off, S *fout, int x0, int y0, int ti
 // one-cell halo (ghost rows/columns carry the periodic wrap) into shared memory, with
 // the tile's stirring rows; NST stages rotate on mbarriers (NST = 2: the next tile is
 // in flight while this one is computed; NST = 1: its copy starts after the pull of this one
-// and hides behind the arithmetic, and more CTAs fit on an SM: 512^2 FP32 12.0 -> 10.0 us).  Each thread pull-streams its cell(s) from shared memory (bilinear
-// weights, bounce-back substitution from the mask), takes the moments, Landau-matches,
-// relaxes, adds the force and stores the Q results with coalesced stores, refreshing
-// the ghost copies of boundary cells.
+// and hides behind the arithmetic, and more CTAs fit on an SM: 512^2 FP32 12.0 -> 10.0 us).
+// Each thread pull-streams its cell(s) from shared memory (bilinear weights, bounce-back
+// substitution from the mask), takes the moments, Landau-matches, relaxes, adds the force
+// and stores the Q results with coalesced stores, refreshing the ghost copies of boundary
+// cells.
 // ---------------------------------------------------------------------------
 template <typename S, int VS, bool MASK, bool FORCE, int CPT, int NST, bool STORE>
 __global__ void __launch_bounds__(TILE_THREADS)

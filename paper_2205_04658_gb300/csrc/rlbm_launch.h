@@ -34,7 +34,7 @@ struct HostPhys {
 
 // A lattice's stirring: modes and phase tables (device pointers) and the tables of a step.
 struct HostStir {
-  int nrows, nmodes;
+  int nrows;
   const void *G_cur, *EY;
   int eyp;
   void *G_next;              // the table of step_next, built by the launch (NULL: none)

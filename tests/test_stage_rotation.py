@@ -80,4 +80,4 @@ def test_every_tiled_kernel_winds_down(name, kernels):
     latched = [m.end() for m in re.finditer(r"atomicOr\([^;]*ERR_TIMEOUT\);", src)]
     assert len(latched) == kernels
     for at in latched:
-        assert re.match(r"\s*(//[^\n]*\n\s*)*wind_down\((NST == 1 \? k : NST \+ k|NST \+ k|min\(NST \+ k, my_tiles\)), NST,", src[at:]), src[at:at + 200]
+        assert re.match(r"\s*(//[^\n]*\n\s*)*wind_down\((NST == 1 \? k : NST \+ k, NST|min\(NST \+ k, my_tiles\), NST|1 \+ k, 1),", src[at:]), src[at:at + 200]
