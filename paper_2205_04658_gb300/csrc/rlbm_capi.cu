@@ -209,7 +209,7 @@ struct rlbm_ctx {
   HostPhys phys;
   int sms = 0;                 // multiprocessors of the device
   int grid_limit = 0;          // step kernel: 0 = one wave of resident CTAs
-  int stages = 1, chained_stages = 1;  // shared-memory pipeline depth of the step kernel (1 or 2)
+  int stages = 1;              // shared-memory pipeline depth of the step kernel (1 or 2)
   bool own_stages = false;     // the depth was set or tuned (else rlbm_init's choice)
   int stir_rows = 1;           // stirring rows: 1 = staged with each tile, 2 = read from global memory
   unsigned launch_seq = 0;     // step-kernel launches so far (selects the tile counter)
@@ -220,10 +220,9 @@ struct rlbm_ctx {
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
 
-  LaunchShape shape() const { return LaunchShape{grid_limit, chained_stages, stages, stir_rows}; }
+  LaunchShape shape() const { return LaunchShape{grid_limit, stages, stir_rows}; }
   void use(const LaunchShape &s) {
     grid_limit = s.grid;
-    chained_stages = s.chained_stages;
     stages = s.stages;
     stir_rows = s.rows;
   }
@@ -251,12 +250,11 @@ cudaError_t dispatch_step_raw(rlbm_ctx *c, const CUtensorMap *ti, void *fout, in
   const void *tg = tgmap ? tgmap : &c->tmap_G[n & 1], *te = &c->tmap_EY;
   int *ctr = c->at<int>(c->L.ctr);
   const unsigned seq = c->launch_seq++;
-  const int stages = chained ? c->chained_stages : c->stages;
   switch (c->cfg.precision) {
-    case RLBM_F64: return launch_step_f64(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    case RLBM_F32: return launch_step_f32(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    case RLBM_F16: return launch_step_f16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
-    default: return launch_step_bf16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F64: return launch_step_f64(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F32: return launch_step_f32(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    case RLBM_F16: return launch_step_f16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
+    default: return launch_step_bf16(c->cfg.vset, ti, tg, te, fout, c->geom, c->phys, s, err, c->grid_limit, c->stages, c->stir_rows, ctr, seq, chained, macro_out, c->stream);
   }
 }
 
@@ -388,6 +386,7 @@ cudaError_t dispatch_observe(rlbm_ctx *c, int mode, bool eps = false, bool ux = 
   o.zscale = spectrum_scale((long long)c->cfg.nx * c->cfg.ny);
   o.bins = c->at<double>(c->L.bins);
   o.nbins = nbins;
+  o.zscale = spectrum_scale((long long)c->cfg.nx * c->cfg.ny);
   unsigned *err = c->at<unsigned>(c->L.err);
   const double e0 = c->cfg.eps0, vm = c->phys.vmax2;
   switch (c->cfg.precision) {
@@ -603,14 +602,15 @@ rlbm_status rlbm_init(const rlbm_config *cfg, void *dev_workspace, size_t bytes,
   c->geom.nx = cfg->nx; c->geom.ny = cfg->ny; c->geom.pitch = L.pitch; c->geom.plane = L.plane;
   c->geom.walls = is_strip(*cfg) ? STRIP_Y : (cfg->walls_y ? WALLS_Y : 0) | (cfg->open_x ? OPEN_X : 0);
   c->geom.nbmask = nullptr;
-  // FP32 and FP64: one stage (512^2 FP32 10.0 us per step against 12.0, 4096^2 equal); the 16-bit forms
-  // keep two (FP16 4096^2 336 us against 357, 1024^2 26.6 against 27.9, though 512^2 11.1 against 10.5).
-  // With a mask it is the other way round: FP16 2048 x 512 28.1 us with two, 26.7 with one, FP32 25.7 and
-  // 27.1, though there a launch by itself, which waits for its first copy, is faster with one (20 steps
-  // observed one by one at 1024 x 256: 905 us against 933 to 992).  (By the registers the compiler takes
-  // for each form, hence the CTAs that fit on an SM.)
-  c->stages = store_bytes(cfg->precision) == 2 && !needs_mask(*cfg) ? 2 : 1;
-  c->chained_stages = cfg->precision == RLBM_F32 && needs_mask(*cfg) ? 2 : c->stages;
+  // Depth by form, us per chained step with one stage and with two: FP32 26.8 and 27.4 (stirred 1024^2),
+  // with a mask 27.4 and 25.9 (body force, 2048 x 512), 24.1 and 24.2 (no force), 29.1 and 30.3 (stirred);
+  // FP16 26.5 and 25.8 (stirred 1024^2), with a mask 27.9 and 26.4 (body force, discs 15 %), 28.2 and
+  // 27.3 (stirred), but 21.6 and 22.7 without a force.  FP64 has one.  Steps by themselves take the same
+  // depth: between launches of different depths the SMs change their shared memory over, 1 to 7 us.
+  const bool masked = needs_mask(*cfg), stirred = L.nmodes > 0;
+  const bool forced = stirred || cfg->body_force[0] != 0.0 || cfg->body_force[1] != 0.0;
+  if (store_bytes(cfg->precision) == 2) c->stages = masked && !forced ? 1 : 2;
+  else c->stages = cfg->precision == RLBM_F32 && masked && forced && !stirred ? 2 : 1;
   {
     const std::string tm = make_tensor_maps(c);
     if (!tm.empty()) { c->msg = tm; return bail(RLBM_E_CUDA); }
@@ -966,7 +966,7 @@ rlbm_status rlbm_set_launch(rlbm_ctx *c, int32_t ctas, int32_t stages, int32_t s
     return c->fail(RLBM_E_INVAL, "ctas must be >= 0, stages 0, 1 or 2 and stir_rows 0, 1 or 2");
   c->grid_limit = ctas;
   if (stages) {
-    c->stages = c->chained_stages = stages;
+    c->stages = stages;
     c->own_stages = true;
   }
   if (stir_rows) c->stir_rows = stir_rows;
@@ -1169,10 +1169,11 @@ rlbm_status rlbm_batch_init(rlbm_ctx *const *members, int32_t nmembers, void *de
     prep0[i + 1] = prep0[i] + c->L.nrows * ((c->cfg.nx + chunk - 1) / chunk);
     if (c->geom.nbmask) b->mask = true;
   }
-  // (16 x 512^2, us per step with one stage and with two: FP32 108 and 119, FP16 96 and 105, with masks
-  // FP16 96 and 105, but FP32 114 and 105)
-  b->stages = b->mask && members[0]->cfg.precision == RLBM_F32 ? 2 : 1;
-  if (members[0]->own_stages) b->stages = members[0]->chained_stages;  // a depth set or tuned on the members stays
+  // 16 x 512^2, us per step with one stage and with two: FP32 107 and 118, FP16 96 and 106, with masks FP16
+  // 95 and 102 (body force), 108 and 118 (stirred), but FP32 115 and 105 (body force), 114 and 102 (no
+  // force); stirred FP32 124 and 129
+  b->stages = b->mask && members[0]->cfg.precision == RLBM_F32 && members[0]->L.nmodes == 0 ? 2 : 1;
+  if (members[0]->own_stages) b->stages = members[0]->stages;  // a depth set or tuned on the members stays
   b->ntiles = tile0[nmembers];
   Scoped dev(b->device);
   cudaError_t e;
