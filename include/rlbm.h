@@ -152,7 +152,9 @@ RLBM_API rlbm_status rlbm_moments(rlbm_ctx *ctx, double *eps, double *ux, double
 /* Energy spectrum of the current state's velocity v = u^i / u^0 (Sec. "Turbulence"):
  * E[n] = 1/2 sum_{k: round(|k|) = n} |v^(k)|^2 / (nx ny)^2, n = 0 .. nbins-1, integer
  * wave numbers, v^(k) = sum_x v(x) exp(-i k.x), v = 0 at solid cells.  E: host array of
- * nbins doubles.  Syncs. */
+ * nbins doubles.  F64 states are transformed and summed in FP64; the others, whose v is
+ * an FP32 number per cell, in two-float (48-bit) arithmetic over FP32's normal range of
+ * velocities, and the bins are added up in FP64.  Syncs. */
 RLBM_API rlbm_status rlbm_spectrum(rlbm_ctx *ctx, int32_t nbins, double *E);
 
 /* Energy of a band of wave vectors of the current state's velocity field (v = u^i / u^0):
@@ -160,15 +162,15 @@ RLBM_API rlbm_status rlbm_spectrum(rlbm_ctx *ctx, int32_t nbins, double *E);
  * indices; k2hi <= 0 means no upper bound.  With k2lo = 0 and k2hi = kmin^2 it is the mean
  * kinetic energy of the velocities filtered to the range below the stirring shell (Part I,
  * "Model and Methods": the recorded velocities are filtered to remove the driven range);
- * sqrt(2 E) is the filtered rms velocity.  Same normalisation as rlbm_spectrum (the band
- * [0, infinity) is half the mean |v|^2).  Syncs. */
+ * sqrt(2 E) is the filtered rms velocity.  Same normalisation and arithmetic as
+ * rlbm_spectrum (the band [0, infinity) is half the mean |v|^2).  Syncs. */
 RLBM_API rlbm_status rlbm_band_energy(rlbm_ctx *ctx, int64_t k2lo, int64_t k2hi, double *E);
 
 /* Column means of the current state's velocity v = u^i / u^0 (solid cells count as 0):
  * jx[x] = (1/ny) sum_y v^x(x, y), jy likewise; host arrays of nx values (either may be NULL).
  * The current density of Part II ("Model and Methods") in units of the particle speed:
  * jx[nx - 1] at the outflow border over time gives j(t), jx over a span of columns j(x).
- * Syncs. */
+ * Summed in FP64 for F64 states, in two-float (48-bit) arithmetic for the others.  Syncs. */
 RLBM_API rlbm_status rlbm_column_means(rlbm_ctx *ctx, double *jx, double *jy);
 
 /* Copy the stored populations out or in (checkpoint / resume).  host: (planes x ny x nx)
@@ -179,12 +181,11 @@ RLBM_API rlbm_status rlbm_get_state(rlbm_ctx *ctx, double *host, int64_t *step);
 RLBM_API rlbm_status rlbm_set_state(rlbm_ctx *ctx, const double *host, int64_t step);
 RLBM_API int32_t rlbm_num_planes(const rlbm_ctx *ctx);
 
-/* Launch shape of the fused step kernel: `ctas` persistent CTAs walk the lattice's
- * 32 x 8 tiles (0 = as many as are resident at once, the default; larger values are
- * clamped; 32 x 4 in FP64), `stages` (1 or 2; 0 keeps the current value; the default
- * depends on the storage, the mask and whether a step follows another in the same call)
- * tiles of shared memory rotate in its TMA pipeline, and `stir_rows` says where the
- * stirring rows of a tile come from: 1 = staged with the tile by TMA (default), 2 = read from global memory (less
+/* Launch shape of the fused step kernel.  `ctas` persistent CTAs walk the lattice's tiles of
+ * 32 x 8 cells (32 x 4 in FP64): 0 = as many as are resident at once, the default; larger
+ * values are clamped.  `stages` (1 or 2) tiles of shared memory rotate in its TMA pipeline;
+ * 0 keeps the current value, and the default depends on the storage, the mask and the force.  `stir_rows` says where the stirring rows of a tile
+ * come from: 1 = staged with the tile by TMA (default), 2 = read from global memory (less
  * shared memory per CTA, so more CTAs per SM); 0 keeps the current value.  A tuning
  * control: results do not depend on it.  The paper has no counterpart. */
 RLBM_API rlbm_status rlbm_set_launch(rlbm_ctx *ctx, int32_t ctas, int32_t stages, int32_t stir_rows);
@@ -192,9 +193,9 @@ RLBM_API rlbm_status rlbm_set_launch(rlbm_ctx *ctx, int32_t ctas, int32_t stages
 /* Autotuner: times every launch shape it knows (pipeline depth x CTA count x stirring
  * rows staged or read from global memory), `reps` launches each, chained as rlbm_step
  * chains consecutive steps and of alternating parity, on the current state, and keeps the
- * fastest; with that, the pipeline depth of steps launched by themselves.  The state and the
- * step counter are left as they were (the launches rewrite the next buffer only).  *ms_out
- * (may be NULL) receives the chosen shape's time per chained step in milliseconds.  Syncs.
+ * fastest.  The state and the step counter are left as they were (the launches rewrite the
+ * next buffer only).  *ms_out (may be NULL) receives the chosen shape's time per step in
+ * milliseconds.  Syncs.
  * The paper has no counterpart. */
 RLBM_API rlbm_status rlbm_autotune(rlbm_ctx *ctx, int32_t reps, double *ms_out);
 
@@ -336,14 +337,14 @@ RLBM_API rlbm_status rlbm_set_mode_scale(rlbm_ctx *ctx, const double *sigma, int
  * after rlbm_step(ctx, nsteps)), keeping the post-collision state every `segment` steps
  * (0: ceil(sqrt(nsteps))), then the hand-written adjoint backwards, recomputing each
  * segment but the last from its checkpoint: about sqrt(nsteps) states of memory and nearly
- * one extra forward pass.  The run of a segment keeps, for every step of the segment in hand, the step's Landau
- * solution, force and streamed deviations h (5 + 17 values per cell for the paper's set,
- * in the storage type), which the reverse steps read.  segment >= nsteps keeps those
+ * one extra forward pass.  The run of a segment keeps, for every step of the segment in
+ * hand, the step's Landau solution, force and streamed deviations h (5 + 17 values per cell
+ * for the paper's set, in the storage type), which the reverse steps read.  segment >= nsteps keeps those
  * values for every step instead (one segment, e.g. 54 GB for 512^2 FP32 and 2000 steps):
  * the forward runs once and no step is recomputed.  The results do not depend on segment.
- * It returns J and dJ/dsigma_m (host, rlbm_num_modes values; may be NULL), dJ/d(eta/s) (host, 1; may be NULL) and dJ/dF_body (host, 2; may be NULL; zero for the
- * eight-direction set, which has no force term), evaluated at
- * the current sigma, eta/s and body force.  FP64 and FP32 storage only (E_INVAL for the
+ * It returns J and dJ/dsigma_m (host, rlbm_num_modes values; may be NULL), dJ/d(eta/s)
+ * (host, 1; may be NULL) and dJ/dF_body (host, 2; may be NULL; zero for the eight-direction
+ * set, which has no force term), evaluated at the current sigma, eta/s and body force.  FP64 and FP32 storage only (E_INVAL for the
  * 16-bit forms).  Syncs.
  * Workspace: rlbm_gradient_query_workspace bytes of caller-owned device memory, 256-byte
  * aligned, used only during the call.  Device errors of the run are latched as usual. */
