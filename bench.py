@@ -103,7 +103,8 @@ def workload_name(args):
             "dt 0.05, a 0.1, eps0 1 at rest" % (args.nx, args.ny, args.precision.upper()))
 
 
-STEP_KERNEL_SOURCES = ("rlbm_device.cuh", "rlbm_kernels.cuh", "rlbm_tma.cuh", "rlbm_launch.h", "rlbm_kernels_f32.cu")
+STEP_KERNEL_SOURCES = ("rlbm_device.cuh", "rlbm_kernels.cuh", "rlbm_tma.cuh", "rlbm_stages.h", "rlbm_launch.h",
+                       "rlbm_kernels_f32.cu")
 
 
 def csrc_digest():
