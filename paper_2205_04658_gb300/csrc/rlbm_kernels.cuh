@@ -780,7 +780,7 @@ __device__ __forceinline__ void pull_global_pair(const S *__restrict__ fin, cons
 
 struct ObsOut {
   double *eps, *ux, *uy;  // OBS_FIELDS (each may be NULL)
-  double2 *z;             // OBS_V (FP32 states: float4 v_x, v_y, 0, 0, high and low parts, times zscale);
+  double2 *z;             // OBS_V (FP32 states: float4 of the high and low parts of v_x, v_y, times zscale);
                           // OBS_COLS: the blocks' partial column sums (the same two forms)
   double *partials;       // [blocks][4]
   double *totals;         // [4]; OBS_COLS: [2 nx]
@@ -789,6 +789,19 @@ struct ObsOut {
   int nbins;
   float zscale;           // OBS_V, FP32 states: the factor of z
 };
+
+// v = u / u^0 = u / sqrt(1 + u^2) of two cells in pairs: the root from the FP32 approximation by one Newton
+// step, its residual 1 - s y^2 in two-float arithmetic.
+__device__ __forceinline__ void over_u0(F2 ux, F2 uy, DF2 &vx, DF2 &vy) {
+  const F2 xx = ux * ux, yy = uy * uy;
+  const DF2 s = df_add(df_add(DF2{xx, fma(ux, ux, -xx)}, DF2{yy, fma(uy, uy, -yy)}), F2(1.0f));
+  const F2 y = FM<F2>::rsqrt(s.h), t = y * y, tl = fma(y, y, -t);
+  const F2 r = fma(s.h, t, F2(-1.0f)) + fma(s.h, tl, s.l * t);  // s y^2 - 1
+  const F2 c = F2(-0.5f) * y * r;
+  const F2 hx = ux * y, hy = uy * y;
+  vx = df_norm(hx, fma(ux, c, fma(ux, y, -hx)));
+  vy = df_norm(hy, fma(uy, c, fma(uy, y, -hy)));
+}
 
 template <typename S, int VS, bool MASK, int MODE>
 __global__ void __launch_bounds__(256)
@@ -824,8 +837,12 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
       fl[k] = in[k] && !(MASK && (nb[k] & 16u));
     }
     R e[NC], ux[NC], uy[NC], vx[NC], vy[NC];
+    float wx[NC], wy[NC];  // FP32 state: the low parts of v
 #pragma unroll
-    for (int k = 0; k < NC; ++k) e[k] = ux[k] = uy[k] = vx[k] = vy[k] = R(0);
+    for (int k = 0; k < NC; ++k) {
+      e[k] = ux[k] = uy[k] = vx[k] = vy[k] = R(0);
+      wx[k] = wy[k] = 0.0f;
+    }
     if constexpr (F64) {
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
@@ -852,7 +869,14 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
         if (!m.ok) atomicOr(err, cell_error(m));
         e[0] = m.eps_m1.v.x; e[1] = m.eps_m1.v.y;
         ux[0] = m.ux.v.x; ux[1] = m.ux.v.y; uy[0] = m.uy.v.x; uy[1] = m.uy.v.y;
-        vx[0] = m.vx.v.x; vx[1] = m.vx.v.y; vy[0] = m.vy.v.x; vy[1] = m.vy.v.y;
+        if (MODE != OBS_FIELDS) {
+          // v of the fields u that OBS_FIELDS hands out, to 45 bits: the v that Landau matching ends with lies
+          // up to 3e-8 |v| to one side (its last step is not iterated), which a mean over cells keeps
+          DF2 px, py;
+          over_u0(m.ux, m.uy, px, py);
+          vx[0] = px.h.v.x; vx[1] = px.h.v.y; vy[0] = py.h.v.x; vy[1] = py.h.v.y;
+          wx[0] = px.l.v.x; wx[1] = px.l.v.y; wy[0] = py.l.v.x; wy[1] = py.l.v.y;
+        }
         if (MODE == OBS_FIELDS) {
           // the deviations e, m_x, m_y (order u) beside the exact count of fluid cells
           // (T^00 = eps0 (1 + e))
@@ -876,7 +900,7 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
         }
       } else {
         float4 *cf = reinterpret_cast<float4 *>(&cols[0][0]), *zf = reinterpret_cast<float4 *>(out.z);
-        DF2 a = df_add(DF2{F2(vx[0], vy[0]), F2(0.0f)}, F2(vx[NC - 1], vy[NC - 1]));
+        DF2 a = df_add(DF2{F2(vx[0], vy[0]), F2(wx[0], wy[0])}, DF2{F2(vx[NC - 1], vy[NC - 1]), F2(wx[NC - 1], wy[NC - 1])});
         cf[ly * 32 + lx] = make_float4(a.h.v.x, a.h.v.y, a.l.v.x, a.l.v.y);
         __syncthreads();
         if (ly == 0 && x < g.nx) {
@@ -947,7 +971,8 @@ observe_kernel(const S *__restrict__ fin, const Geometry<typename RealOf<S>::typ
       } else if constexpr (F64) {
         out.z[c] = make_double2(vx[k], vy[k]);
       } else {
-        reinterpret_cast<float4 *>(out.z)[c] = make_float4(out.zscale * vx[k], out.zscale * vy[k], 0.0f, 0.0f);
+        const float s = out.zscale;
+        reinterpret_cast<float4 *>(out.z)[c] = make_float4(s * vx[k], s * vy[k], s * wx[k], s * wy[k]);
       }
     }
   }
