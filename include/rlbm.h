@@ -152,9 +152,9 @@ RLBM_API rlbm_status rlbm_moments(rlbm_ctx *ctx, double *eps, double *ux, double
 /* Energy spectrum of the current state's velocity v = u^i / u^0 (Sec. "Turbulence"):
  * E[n] = 1/2 sum_{k: round(|k|) = n} |v^(k)|^2 / (nx ny)^2, n = 0 .. nbins-1, integer
  * wave numbers, v^(k) = sum_x v(x) exp(-i k.x), v = 0 at solid cells.  E: host array of
- * nbins doubles.  F64 states are transformed and summed in FP64; the others, whose v is
- * an FP32 number per cell, in two-float (48-bit) arithmetic over FP32's normal range of
- * velocities, and the bins are added up in FP64.  Syncs. */
+ * nbins doubles.  F64 states are transformed and summed in FP64; the others, whose u is
+ * matched in FP32, form v of it, transform and sum in two-float (48-bit) arithmetic over
+ * FP32's normal range of velocities, and the bins are added up in FP64.  Syncs. */
 RLBM_API rlbm_status rlbm_spectrum(rlbm_ctx *ctx, int32_t nbins, double *E);
 
 /* Energy of a band of wave vectors of the current state's velocity field (v = u^i / u^0):
